@@ -137,16 +137,15 @@ __device__ void init_tile(const InitArgs& A, const TubeDev& T, int x0, InitSmem&
         n = st[1];
         v = st[2];
       }
-      const bool ok = P > 0.0 && n > 0.0 && fabs(v) < 1.0;
+      const double g1 = fma(-v, v, 1.0), gam = 1.0 / sqrt(g1), Tt = P / n;
+      const bool ok = P > 0.0 && n > 0.0 && fabs(v) <= beta_limit(NPc);
       if (cell && !ok) atomicOr(A.flag, 1);
-      sm.coef.cell[0][c] = n;
-      sm.coef.cell[1][c] = P / n;
-      sm.coef.cell[2][c] = v;
-      sm.coef.ok[c] = (cell && ok) ? 1 : 0;
+      store_cell_coeffs<NPc, NVc>(cell && ok, v, v * v, g1, n / Tt, Tt * gam, sm.coef, c);
     }
     __syncthreads();
     if (pass == 1 && sm.tie == 0) break;  // uniform over the CTA
-    tile_coeffs<NPc, NVc>(tab, T.Qp, sm.coef, sm.B, A.flag);
+    build_rows<NPc, NVc>(tab, T.Qp, sm.coef, sm.B);
+    __syncthreads();
     init_write<S, NVc>(T, tab, sm, static_cast<S*>(A.F), x0, pass == 1, tie);
     __syncthreads();
   }
@@ -277,32 +276,15 @@ rlb_status cuda_status(cudaError_t e) {
 std::mutex g_tables_mu;
 bool g_tables_ready[64] = {};
 
-// Once per device: fill the series tables (long double on the host) and let the stage kernel use more than
+// Once per device: fill the recurrence factors of the Legendre coefficients and let the kernels use more than
 // 48 KB of dynamic shared memory.
 rlb_status ensure_series_tables(int dev) {
   std::lock_guard<std::mutex> lk(g_tables_mu);
   if (dev < 0 || dev >= 64) return RLB_EINVAL;
   if (g_tables_ready[dev]) return RLB_OK;
-  std::vector<double> ic((size_t)(R_MAX + 1) * (NV_MAX + 1), 0.0), cb((size_t)(M_MAX + 1) * (R_MAX + 1), 0.0);
-  for (int k = 0; k <= NV_MAX; ++k) {
-    // I_{k,k} = 2^{k+1} (k!)^2 / (2k+1)!; I_{r+2,k}/I_{r,k} = (r+1)(r+2)((r+k)/2+1) / (((r-k)/2+1)(r+k+2)(r+k+3))
-    long double I = 2.0L;
-    for (int q = 1; q <= k; ++q) I *= 2.0L * q * q / ((2.0L * q) * (2.0L * q + 1.0L));
-    for (int r = k; r <= R_MAX; r += 2) {
-      ic[(size_t)r * (NV_MAX + 1) + k] = (double)((2.0L * k + 1.0L) / 2.0L * I);
-      const long double hp = (r + k) / 2, hm = (r - k) / 2;
-      I *= (r + 1.0L) * (r + 2.0L) * (hp + 1.0L) / ((hm + 1.0L) * (r + k + 2.0L) * (r + k + 3.0L));
-    }
-  }
-  for (int m = 1; m <= M_MAX; ++m) {
-    long double C = 1.0L;  // C(m - 1, 0)
-    for (int r = 0; r <= R_MAX; ++r) {
-      cb[(size_t)m * (R_MAX + 1) + r] = (double)C;
-      C = C * (m + r) / (r + 1.0L);  // C(m + r, r + 1)
-    }
-  }
-  RLB_CUDA(cudaMemcpyToSymbol(g_ic, ic.data(), ic.size() * sizeof(double)));
-  RLB_CUDA(cudaMemcpyToSymbol(g_cb, cb.data(), cb.size() * sizeof(double)));
+  double leg[LEG_MAX + 1];
+  for (int k = 0; k <= LEG_MAX; ++k) leg[k] = -(double)(k * (k + 2)) / (double)((2 * k + 1) * (2 * k + 3));
+  RLB_CUDA(cudaMemcpyToSymbol(g_leg, leg, sizeof(leg)));
   const void* fp64[3] = {(const void*)rlb_stage_kernel<0>, (const void*)rlb_stage_kernel<1>,
                          (const void*)rlb_stage_kernel<2>};
   const void* rp[6] = {(const void*)rlb_stage_rp_kernel<float, 0>, (const void*)rlb_stage_rp_kernel<float, 1>,
@@ -461,7 +443,11 @@ bool fill_tube_tables(const rlb_tube& t, double* pb, double* wp, double* xi, dou
         for (int u = 1; u <= q; ++u) C = C * (l - q + u) / u;
         acc += C * rlbq::laguerre1(l, pb[i]);
       }
-      T[TAB_K + i * (NP_MAX + 1) + q] = (double)((q % 2) ? -acc : acc);
+      if (q % 2) acc = -acc;
+      T[TAB_K + i * (NP_MAX + 1) + q] = (double)acc;
+      long double f = 4.0L;  // 4 (q + 1)!
+      for (int u = 2; u <= q + 1; ++u) f *= u;
+      T[TAB_KW + i * (NP_MAX + 1) + q] = (double)(wp[i] * acc / f);
     }
   }
   for (int j = 0; j < t.Qxi; ++j) {

@@ -14,7 +14,8 @@
 //              (n, T, beta) back through the Landau solve;
 //   tau:       d/dlog(tau) of b dt r_s (F^eq_s - F_s) is -b dt r_s (F^eq_s - F_s).
 // The equilibrium's parameter derivatives use B[i][k] = n w^p_i/4 sum_q K[i][q] T^(q-1) gamma^-(q+2)
-// hhat_{q+2,k}(beta) and the derivative series d hhat_{m,k}/d beta = sum_r r C(m+r-1, r) beta^(r-1) I_{r,k}.
+// hhat_{q+2,k}(beta) and d hhat_{m,k}/d beta = m (k/(2k-1) hhat_{m+1,k-1} + (k+1)/(2k+3) hhat_{m+1,k+1}), the
+// projection of m xi (1 - beta xi)^-(m+1).
 //
 // An adjoint tile has TXA = 60 cells, so that the TXA + 4 interfaces whose stencils reach its cells fit
 // the 64 lanes of a velocity group.
@@ -42,81 +43,44 @@ struct AdjArgs {
 
 // Legendre coefficients and their beta derivatives (m = 2 .. Np+2, k <= Nv) of the tile's cells
 struct AdjCoef {
-  double hh[M_MAX - 1][NV_MAX + 1][GW];
-  double dh[M_MAX - 1][NV_MAX + 1][GW];
+  double hh[NP_MAX + 1][NV_MAX + 1][GW];
+  double dh[NP_MAX + 1][NV_MAX + 1][GW];
 };
 
-// One parity class of hhat_{m,k}(beta) and d hhat_{m,k}/d beta by the positive power series of the forward
-// (same tables and summation order), continued until both series have converged.
-template <int NPc, int NVc, int PAR>
-__device__ bool hhat_parity_d(double beta, double* hh_col, double* dh_col) {
-  constexpr int NK = (NVc - PAR) / 2 + 1;
-  double acc[NPc + 1][NK], dac[NPc + 1][NK];
-#pragma unroll
-  for (int m = 0; m <= NPc; ++m)
-#pragma unroll
-    for (int q = 0; q < NK; ++q) acc[m][q] = dac[m][q] = 0.0;
-  const double b2 = beta * beta;
-  const double tol = 1e-18 * (1.0 - b2);
-  double br = PAR ? beta : 1.0;  // beta^r
-  double bm = 1.0;               // beta^(r-1), r >= 1
-  bool done = false;
-  for (int r = PAR; r <= R_MAX; r += 2) {
-    const double* ic = g_ic + r * (NV_MAX + 1);
-    const double rb = r == 0 ? 0.0 : r * bm;  // d beta^r / d beta
-    double tlast = 0.0, dlast = 0.0;
-#pragma unroll
-    for (int m = 0; m <= NPc; ++m) {
-      const double cb = g_cb[(m + 2) * (R_MAX + 1) + r];
-      const double t = cb * br, d = cb * rb;
-#pragma unroll
-      for (int q = 0; q < NK; ++q) {
-        acc[m][q] = fma(ic[PAR + 2 * q], t, acc[m][q]);
-        dac[m][q] = fma(ic[PAR + 2 * q], d, dac[m][q]);
-      }
-      tlast = t;
-      dlast = d;
-    }
-    if (r >= NVc && fabs(tlast) < tol && fabs(dlast) < tol) {
-      done = true;
-      break;
-    }
-    br *= b2;
-    bm = r == 0 ? beta : bm * b2;
-  }
-#pragma unroll
-  for (int m = 0; m <= NPc; ++m)
-#pragma unroll
-    for (int q = 0; q < NK; ++q) {
-      hh_col[((m * (NV_MAX + 1)) + PAR + 2 * q) * GW] = acc[m][q];
-      dh_col[((m * (NV_MAX + 1)) + PAR + 2 * q) * GW] = dac[m][q];
-    }
-  return done;
-}
-
-// hhat and d hhat/d beta of the tile's cells (groups 0/1: even/odd k); cells with ok == 0 keep zeros.
-// With Bs != nullptr, group i then builds the equilibrium coefficients B[i][k] as the forward does.
-// Ends with a barrier.
+// hhat and d hhat/d beta of the tile's cells, one thread per cell; cells with ok == 0 keep zeros. With
+// Bs != nullptr, group i then builds the equilibrium coefficients B[i][k] as the forward does. Ends with a barrier.
 template <int NPc, int NVc>
 __device__ void tile_coeffs_d(const double* tab, int Qp, const double* cellv /* n, T, beta: [3][GW] */,
                               int* ok, AdjCoef& co, double (*Bs)[GW], int* flag) {
   const int c = threadIdx.x % GW, g = threadIdx.x / GW;
-  if (g < 2 && c < TXA) {
-    bool conv = true;
+  if (g == 0 && c < TXA) {
+    const double beta = cellv[2 * GW + c];
+    if (ok[c] && !(fabs(beta) <= beta_limit_d(NPc))) {
+      ok[c] = 0;
+      atomicOr(flag, 1);
+    }
     if (ok[c]) {
-      const double beta = cellv[2 * GW + c];
-      if (g == 0)
-        conv = hhat_parity_d<NPc, NVc, 0>(beta, &co.hh[0][0][c], &co.dh[0][0][c]);
-      else
-        conv = hhat_parity_d<NPc, NVc, 1>(beta, &co.hh[0][0][c], &co.dh[0][0][c]);
+      double h[NPc + 2][NVc + 2];
+      const double g1 = fma(-beta, beta, 1.0), u = 1.0 / g1;
+      legendre_coeffs<NPc + 2, NVc + 1>(beta, beta * beta, g1, h);
+      double f = u;  // gamma^2(m-1) / (m-1)! at m = 2
+#pragma unroll
+      for (int q = 0; q <= NPc; ++q) {
+        const double fd = f * u;  // m times the factor of m + 1 = q + 3
+#pragma unroll
+        for (int k = 0; k <= NVc; ++k) {
+          co.hh[q][k][c] = f * h[q][k];
+          double d = (double)(k + 1) / (double)(2 * k + 3) * h[q + 1][k + 1];
+          if (k > 0) d = fma((double)k / (double)(2 * k - 1), h[q + 1][k - 1], d);
+          co.dh[q][k][c] = fd * d;
+        }
+        f *= u / (double)(q + 2);
+      }
     } else {
 #pragma unroll
       for (int m = 0; m <= NPc; ++m)
-        for (int k = g; k <= NVc; k += 2) co.hh[m][k][c] = co.dh[m][k][c] = 0.0;
-    }
-    if (!conv) {
-      ok[c] = 0;
-      atomicOr(flag, 1);
+#pragma unroll
+        for (int k = 0; k <= NVc; ++k) co.hh[m][k][c] = co.dh[m][k][c] = 0.0;
     }
   }
   __syncthreads();

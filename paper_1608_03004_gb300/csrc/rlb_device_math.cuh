@@ -15,6 +15,29 @@ __device__ __forceinline__ double rcp_nr(double d) {
   return fma(x0, fma(e, e, e), x0);
 }
 
+// 1/sqrt(x) for positive, normal x: the hardware approximation of rsqrt.approx.ftz.f64 refined by one step of
+// third order, y1 = y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2 (the binomial series of (1 - e)^(-1/2)): five FP64
+// operations and no branch, where 1.0 / sqrt(x) takes about 35.
+__device__ __forceinline__ double rsqrt_nr(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// sqrt(x) for x >= 0 (0 gives 0): x rsqrt(x) and one Newton-Raphson correction from the remainder x - s^2.
+__device__ __forceinline__ double sqrt_nr(double x) {
+  const double y = rsqrt_nr(x), s = x * y;
+  const double r = fma(fma(-s, s, x), 0.5 * y, s);
+  return x == 0.0 ? 0.0 : r;
+}
+
+// a/d for positive, normal d: a times the reciprocal, corrected once from the remainder a - q d.
+__device__ __forceinline__ double div_nr(double a, double d) {
+  const double r = rcp_nr(d), q = a * r;
+  return fma(fma(-q, d, a), r, q);
+}
+
 constexpr double WENO_EPS = 1e-6;
 
 // Products and sums that are rounded exactly as written. The compiler may contract a product into a following

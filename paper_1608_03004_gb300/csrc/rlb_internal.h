@@ -21,9 +21,8 @@ namespace rlb {
 constexpr int QP_MAX = 4;
 constexpr int NP_MAX = 3;             // Np < Qp <= QP_MAX
 constexpr int NV_MAX = 8;
-constexpr int M_MAX = NP_MAX + 2;     // powers (1 - beta xi)^-m, m = 2 .. Np + 2
 constexpr int QXI_MAX = 1024;
-constexpr int R_MAX = 16383;          // longest series for the Legendre coefficients (|v| up to ~0.995)
+constexpr int LEG_MAX = 255;          // longest backward recurrence for the Legendre coefficients
 
 // Per-tube description as the kernels see it.
 struct TubeDev {
@@ -52,6 +51,8 @@ struct TubeDev {
 //   [3 QP_MAX, 3 QP_MAX + QP_MAX (NP_MAX+1))   K[i][q] = (-1)^q sum_{l=q}^{Np} C(l,q) L^(1)_l(pbar_i)
 //                                               at [i (NP_MAX+1) + q]: the radial factor multiplying
 //                                               s^(q+2) hhat_{q+2,k} in the truncated equilibrium
+//   then w^p_i K[i][q] / (4 (q+1)!) at [i (NP_MAX+1) + q]: the same with the factors that the per-cell
+//                                               coefficients take out (legendre_coeffs)
 //   then xi_j (Qxi), then w^xi_j P_k(xi_j) at [j (NV_MAX+1) + k] (Qxi (NV_MAX+1)), zero for k > Nv,
 //   then b_st dt xi_j / dx at [st Qxi + j] for the three Runge-Kutta stages, b = (1, 1/4, 2/3),
 //   then per velocity s = i Qxi + j the WENO5 epsilon terms 3 eps ws^2 (C0, C1, C2) at [3 s + 0..2],
@@ -62,7 +63,8 @@ constexpr int TAB_PBAR = 0;
 constexpr int TAB_PBAR2 = QP_MAX;
 constexpr int TAB_WP = 2 * QP_MAX;
 constexpr int TAB_K = 3 * QP_MAX;
-constexpr int TAB_XI = TAB_K + QP_MAX * (NP_MAX + 1);
+constexpr int TAB_KW = TAB_K + QP_MAX * (NP_MAX + 1);
+constexpr int TAB_XI = TAB_KW + QP_MAX * (NP_MAX + 1);
 __host__ __device__ inline int tab_pw(int Qxi) { return TAB_XI + Qxi; }
 __host__ __device__ inline int tab_cxi(int Qxi) { return TAB_XI + Qxi + Qxi * (NV_MAX + 1); }
 __host__ __device__ inline int tab_eps(int Qxi) { return tab_cxi(Qxi) + 3 * Qxi; }

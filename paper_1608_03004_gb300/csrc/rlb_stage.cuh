@@ -12,10 +12,9 @@ constexpr int HALO = 3;                    // WENO5 reaches three cells upwind/d
 constexpr int RW = TX + 2 * HALO;          // staged row length
 constexpr int NBC = QP_MAX * (NV_MAX + 1); // per-cell equilibrium coefficients
 
-// Series tables for the Legendre coefficients of (1 - beta xi)^-m (filled once per device):
-//   g_ic[r][k] = (2k+1)/2 * int_{-1}^{1} xi^r P_k(xi) dxi,   g_cb[m][r] = C(m + r - 1, r).
-__device__ double g_ic[(R_MAX + 1) * (NV_MAX + 1)];
-__device__ double g_cb[(M_MAX + 1) * (R_MAX + 1)];
+// Factors -k (k + 2) / ((2k + 1) (2k + 3)) of the backward recurrence of the Legendre coefficients
+// (legendre_coeffs), filled once per device.
+__device__ double g_leg[LEG_MAX + 1];
 
 struct StageArgs {
   const TubeDev* tubes;
@@ -113,104 +112,146 @@ __device__ __forceinline__ bool landau(const double mom[5], double& e, double& b
 // Per-cell equilibrium coefficients of a tile (shared by the stage and initial-condition kernels)
 // --------------------------------------------------------------------------------------------------
 
-struct CoefSmem {
-  double hh[M_MAX - 1][NV_MAX + 1][GW];  // hhat_{m,k}, m = 2 .. Np+2
-  double cell[3][GW];                    // n, T, beta of each cell
-  int ok[GW];
-};
+// Speed limits of the Legendre coefficients: a cell with |beta| beyond them is treated as non-physical. They are
+// the speeds up to which the power series of (1 - beta xi)^-m, m = NPc + 2, (with the beta derivative: of its
+// derivative too) falls below 1e-18 (1 - beta^2) within 16384 terms: the range the library documents.
+__host__ __device__ constexpr double beta_limit(int NPc) { return NPc <= 2 ? 0.995524321007388 : 0.995025380567975; }
+__host__ __device__ constexpr double beta_limit_d(int NPc) { return NPc <= 2 ? 0.994941897153004 : 0.994442517779333; }
 
-// One parity class of the Legendre coefficients hhat_{m,k} = (2k+1)/2 int P_k(xi) (1 - beta xi)^-m dxi,
-// m = 2..NPc+2, k = PAR, PAR+2, .. <= NVc, by the positive power series (1 - beta xi)^-m =
-// sum_r C(m+r-1, r) beta^r xi^r with int xi^r P_k tabulated. Terms of one class share one sign, so the sum
-// has no cancellation; it stops when the largest-m term drops below 1e-18 (1 - beta^2).
-template <int NPc, int NVc, int PAR, int STRIDE = GW>
-__device__ bool hhat_parity(double beta, double* hh_col /* [m-2][k][STRIDE] at this cell */) {
-  constexpr int NK = (NVc - PAR) / 2 + 1;
-  double acc[NPc + 1][NK];
-#pragma unroll
-  for (int m = 0; m <= NPc; ++m)
-#pragma unroll
-    for (int q = 0; q < NK; ++q) acc[m][q] = 0.0;
-  bool done = (beta == 0.0);
-  if (beta == 0.0 && PAR == 0) {
-#pragma unroll
-    for (int m = 0; m <= NPc; ++m) acc[m][0] = 1.0;
+// Legendre coefficients of (1 - beta xi)^-m: h[m - 2][k], m = 2 .. NM + 1, k = 0 .. KV, with
+//   hhat_{m,k} = (2k+1)/2 int P_k(xi) (1 - beta xi)^-m dxi = h[m - 2][k] (gamma^2)^(m-1) / (m-1)!,
+// gamma^2 = 1 / (1 - beta^2). b2 = beta^2, g1 = 1 - beta^2.
+//
+// The integrals are derivatives of the Legendre functions of the second kind Q_k(1/beta), and obey their
+// recurrences (Abramowitz and Stegun, chapter 8): in k, at m = 2, with a_k = beta^k s_k c_k, s_k = s_{k-1}
+// (k+1)/(2k+1):
+//   c_{k-1} = c_k - k (k+2) / ((2k+1) (2k+3)) beta^2 c_{k+1},
+// whose decaying solution is the wanted one; it is taken downward from c_{K+1} = 0, c_K = 1 (Miller's algorithm)
+// and scaled by the closed form at k = 0. The error falls by ((1 - s)/(1 + s)), s = sqrt(1 - beta^2), per step, which
+// gives K. In m:
+//   m (1 - beta^2) a_{m+1,k} = (k + m - 1) beta a_{m,k-1} - (k - m + 1) a_{m,k},
+// and for k = 0 the form without a_{m,-1}, m (1 - beta^2) a_{m+1,0} = m a_{m,0} + (m - 2) beta a_{m,1}.
+// Against extended precision every coefficient is within a few units of FP64 rounding up to |beta| = 0.97 (as the
+// positive power series in beta is, which takes 12 operations for each of its 40 terms at beta = 0.4 and 574 at 0.9;
+// here about 2 operations for each of 18 and 46 steps). FP64 operations bound every kernel that calls this. With the
+// series, the FP32 steps of 128 uneven moving tubes kept the FP64 pipe 85 % busy; on GB300 they went from 4.42 to 2.43
+// ms, the FP32 stress tube's (half its gas in motion) from 6.5 to 5.2 ms, the 400-cell FP64 tube's from 89 to 54 us.
+template <int NM, int KV>
+__device__ __forceinline__ void legendre_coeffs(double beta, double b2, double g1, double (&h)[NM][KV + 1]) {
+  double C[KV + 2];
+  {
+    // K = KV + 2 + 54 / -log2((1 - s)/(1 + s)), (1 - s)/(1 + s) = beta^2 / (1 + s)^2 (beta = 0: K = KV + 2)
+    const float lr = 2.0f * __log2f(1.0f + sqrtf((float)g1)) - __log2f((float)b2);
+    const int K = min(KV + 2 + (int)(54.0f / lr), LEG_MAX);
+    double c1 = 1.0, c2 = 0.0;  // c_k, c_{k+1}
+    for (int k = K; k > KV + 1; --k) {
+      const double c0 = fma(g_leg[k], b2 * c2, c1);
+      c2 = c1;
+      c1 = c0;
+    }
+    C[KV + 1] = c1;
+    C[KV] = fma(g_leg[KV + 1], b2 * c2, c1);
   }
-  if (!done) {
-    const double b2 = beta * beta;
-    const double tol = 1e-18 * (1.0 - b2);
-    double br = PAR ? beta : 1.0;  // beta^r
-    for (int r = PAR; r <= R_MAX; r += 2) {
-      const double* ic = g_ic + r * (NV_MAX + 1);
-      double tlast = 0.0;
 #pragma unroll
-      for (int m = 0; m <= NPc; ++m) {
-        const double t = g_cb[(m + 2) * (R_MAX + 1) + r] * br;
+  for (int k = KV; k >= 1; --k) C[k - 1] = fma(g_leg[k], b2 * C[k + 1], C[k]);
+  const double inv = rlbdev::rcp_nr(C[0]);
+  double bk = inv, sk = 1.0;  // beta^k / c_0; (2k+1) s_k
+  h[0][0] = 1.0;
 #pragma unroll
-        for (int q = 0; q < NK; ++q) acc[m][q] = fma(ic[PAR + 2 * q], t, acc[m][q]);
-        tlast = t;
-      }
-      if (r >= NVc && fabs(tlast) < tol) {
-        done = true;
-        break;
-      }
-      br *= b2;
+  for (int k = 1; k <= KV; ++k) {
+    bk *= beta;
+    sk *= (double)(k + 1) / (double)(2 * k + 1);
+    h[0][k] = ((2 * k + 1) * sk) * (bk * C[k]);
+  }
+#pragma unroll
+  for (int q = 1; q < NM; ++q) {
+    const int m = q + 1;  // from m to m + 1
+    h[q][0] = fma((m - 2) / 3.0, beta * h[q - 1][1], (double)m * h[q - 1][0]);
+#pragma unroll
+    for (int k = 1; k <= KV; ++k) {
+      const double lead = (double)((k + m - 1) * (2 * k + 1)) / (double)(2 * k - 1);
+      h[q][k] = fma(lead, beta * h[q - 1][k - 1], (double)(m - 1 - k) * h[q - 1][k]);
     }
   }
-#pragma unroll
-  for (int m = 0; m <= NPc; ++m)
-#pragma unroll
-    for (int q = 0; q < NK; ++q) hh_col[((m * (NV_MAX + 1)) + PAR + 2 * q) * STRIDE] = acc[m][q];
-  return done;
 }
 
-// Fill B[i (NVc+1) + k][c] (radial rows i < Qp) for the TX cells of a tile from cs.cell (n, T, beta) and cs.ok:
-//   F^eq_ij = sum_k B[i][k] w^xi_j P_k(xi_j),  B[i][k] = n/(4T^3) w^p_i sum_q s^(q+2) K[i][q] hhat_{q+2,k},
-// s = T/gamma (Eq. (feqtrunc): Laguerre generating function for the radial projection, Legendre projection
-// of each (1 - beta xi)^-m for the angular one). Groups 0/1 run the even/odd series, then group g builds
-// radial row i = g. Cells with ok == 0 get B = 0. Ends with a barrier.
+// The same times the per-cell factors of the equilibrium: ge[q][k] = g_q h[q][k], so that
+//   F^eq_ij = sum_k B[i][k] w^xi_j P_k(xi_j),  B[i][k] = sum_q TAB_KW[i][q] ge[q][k]
+// (Eq. (feqtrunc): Laguerre generating function for the radial projection, Legendre projection of each
+// (1 - beta xi)^-m for the angular one; B = n/(4T^3) w^p_i sum_q s^(q+2) K[i][q] hhat_{q+2,k}, s = T/gamma, so
+// that g_q = (n/T) (T gamma)^q).
 template <int NPc, int NVc>
-__device__ void tile_coeffs(const double* tab, int Qp, CoefSmem& cs, double (*Bs)[GW], int* flag) {
-  const int c = threadIdx.x % GW, g = threadIdx.x / GW;
-  if (g < 2 && c < TX) {
-    const double beta = cs.cell[2][c];
-    bool conv = true;
-    if (cs.ok[c]) {
-      if (g == 0)
-        conv = hhat_parity<NPc, NVc, 0>(beta, &cs.hh[0][0][c]);
-      else
-        conv = hhat_parity<NPc, NVc, 1>(beta, &cs.hh[0][0][c]);
-    }
-    if (!conv) {
-      cs.ok[c] = 0;  // both groups may write 0; no other value is written concurrently
-      atomicOr(flag, 1);
-    }
+__device__ __forceinline__ void cell_coeffs(double beta, double b2, double g1, double g0, double tg,
+                                            double (&ge)[NPc + 1][NVc + 1]) {
+  legendre_coeffs<NPc + 1, NVc>(beta, b2, g1, ge);
+  double g = g0;
+#pragma unroll
+  for (int q = 0; q <= NPc; ++q) {
+#pragma unroll
+    for (int k = 0; k <= NVc; ++k) ge[q][k] *= g;
+    g *= tg;
   }
-  __syncthreads();
-  if (c < TX) {
-    const int i = g;
-    double B[NVc + 1];
+}
+
+// Landau frame of a cell for the equilibrium: beta, beta^2, 1 - beta^2, gamma, g0 = n/T = 3 n^2/e and tg = T gamma =
+// e gamma/(3n) from (N0, Nx, T00, T0x, Txx). As landau() with the refined hardware reciprocals in place of IEEE
+// divisions and square roots (each corrected from its remainder where it is not itself a reciprocal), about 55
+// FP64 operations instead of 150. Returns false if non-physical.
+__device__ __forceinline__ bool landau_frame(const double mom[5], double& beta, double& b2, double& g1, double& gam,
+                                             double& g0, double& tg) {
+  const double A = mom[2] + mom[4], B2 = 2.0 * mom[3];
+  const double disc = fma(A, A, -(B2 * B2));
+  const double e = 0.5 * ((mom[2] - mom[4]) + rlbdev::sqrt_nr(disc));
+  beta = rlbdev::div_nr(mom[3], mom[4] + e);
+  b2 = beta * beta;
+  g1 = fma(-beta, beta, 1.0);
+  gam = rlbdev::rsqrt_nr(g1);
+  const double n = gam * fma(-beta, mom[1], mom[0]);
+  const double n3 = 3.0 * n;
+  g0 = n3 * (n * rlbdev::rcp_nr(e));
+  tg = (e * rlbdev::rcp_nr(n3)) * gam;
+  return disc >= 0.0 && e > 0.0 && fabs(beta) < 1.0 && n > 0.0 && tg > 0.0;
+}
+
+struct CoefSmem {
+  double ge[NP_MAX + 1][NV_MAX + 1][GW];  // cell_coeffs of the tile's cells
+};
+
+// Per-cell coefficients of one cell into column c of cs.ge (all zero for a non-physical cell).
+template <int NPc, int NVc>
+__device__ __forceinline__ void store_cell_coeffs(bool ok, double beta, double b2, double g1, double g0, double tg,
+                                                  CoefSmem& cs, int c) {
+  double ge[NPc + 1][NVc + 1];
+  if (ok) {
+    cell_coeffs<NPc, NVc>(beta, b2, g1, g0, tg, ge);
+  } else {
 #pragma unroll
-    for (int k = 0; k <= NVc; ++k) B[k] = 0.0;
-    if (i < Qp && cs.ok[c]) {
-      const double n = cs.cell[0][c], T = cs.cell[1][c], beta = cs.cell[2][c];
-      const double s = T * sqrt(1.0 - beta * beta);
-      const double pref = n / (4.0 * T * T * T) * tab[TAB_WP + i];
-      double sq = s * s;
+    for (int q = 0; q <= NPc; ++q)
 #pragma unroll
-      for (int q = 0; q <= NPc; ++q) {
-        const double G = pref * sq * tab[TAB_K + i * (NP_MAX + 1) + q];
-#pragma unroll
-        for (int k = 0; k <= NVc; ++k) B[k] = fma(G, cs.hh[q][k][c], B[k]);
-        sq *= s;
-      }
-    }
-    if (i < Qp) {
-#pragma unroll
-      for (int k = 0; k <= NVc; ++k) Bs[i * (NVc + 1) + k][c] = B[k];
-    }
+      for (int k = 0; k <= NVc; ++k) ge[q][k] = 0.0;
   }
-  __syncthreads();
+#pragma unroll
+  for (int q = 0; q <= NPc; ++q)
+#pragma unroll
+    for (int k = 0; k <= NVc; ++k) cs.ge[q][k][c] = ge[q][k];
+}
+
+// Fill B[i (NVc+1) + k][c] (radial rows i < Qp) for the TX cells of a tile from cs.ge: group g builds radial row
+// i = g.
+template <int NPc, int NVc>
+__device__ __forceinline__ void build_rows(const double* tab, int Qp, const CoefSmem& cs, double (*Bs)[GW]) {
+  const int c = threadIdx.x % GW, i = threadIdx.x / GW;
+  if (c >= TX || i >= Qp) return;
+  double KW[NPc + 1];
+#pragma unroll
+  for (int q = 0; q <= NPc; ++q) KW[q] = tab[TAB_KW + i * (NP_MAX + 1) + q];
+#pragma unroll
+  for (int k = 0; k <= NVc; ++k) {
+    double B = KW[0] * cs.ge[0][k][c];
+#pragma unroll
+    for (int q = 1; q <= NPc; ++q) B = fma(KW[q], cs.ge[q][k][c], B);
+    Bs[i * (NVc + 1) + k][c] = B;
+  }
 }
 
 // --------------------------------------------------------------------------------------------------
@@ -222,15 +263,19 @@ __device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, %
 
 struct StageSmem {
   union {
-    double red[NG][3 * QP_MAX][GW];  // per group: the radial sums S0, S1, S2 of each radial node
-    CoefSmem coef;
+    struct {
+      double red[NG][3 * QP_MAX][GW];  // per group: the radial sums S0, S1, S2 of each radial node
+      CoefSmem coef;
+    } a;                               // phases A and B
+    struct {
+      double row[2][NG][RW + 1];  // staged velocity rows (double-buffered: written before the first barrier)
+      double d1[NG][RW + 1];      // first differences by position, d1[k] = row[k] - row[k-1]
+      float2 dd[NG][RW + 1];      // the same differences in double-float (hi, lo)
+      float2 sv[NG][3][GW];       // indicators v = S + e (double-float), one triple per pair of adjacent differences
+      float2 phi[NG][GW];         // WENO correction of each interface, times 6 (double-float)
+    } c;                          // phase C
   } u;
   double rate[2][GW];
-  double row[2][NG][RW + 1];  // staged velocity rows (double-buffered: written before the first barrier)
-  double d1[NG][RW + 1];      // first differences by position, d1[k] = row[k] - row[k-1]
-  float2 dd[NG][RW + 1];      // the same differences in double-float (hi, lo)
-  float2 sv[NG][3][GW];       // indicators v = S + e (double-float), one triple per pair of adjacent differences
-  float2 phi[NG][GW];         // WENO correction of each interface, times 6 (double-float)
   int src[RW + 1];            // source cell of each staged position (boundary condition applied)
   double B[NBC][GW];          // equilibrium coefficients B[i (NVc + 1) + k]; last, so that a launch allocates
                               // only the rows its tubes use (stage_smem_bytes)
@@ -284,46 +329,43 @@ __device__ void stage_tile(const StageArgs& A, const TubeDev& T, int x0, int par
       }
     }
 #pragma unroll
-    for (int k = 0; k < 3 * QP_MAX; ++k) sm.u.red[g][k][c] = S[k];
+    for (int k = 0; k < 3 * QP_MAX; ++k) sm.u.a.red[g][k][c] = S[k];
     __syncthreads();
-    // B. Landau frame (one thread per cell), then the equilibrium coefficients
-    double e = 1.0, beta = 0.0, n = 1.0, Tt = 1.0;
-    bool ok = false;
-    if (g == 0 && cell) {
-      double mom[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    // B. Landau frame and Legendre coefficients (one thread per cell), then the equilibrium coefficients
+    if (g == 0) {
+      double beta = 0.0, b2 = 0.0, g1 = 1.0, gam = 1.0, g0 = 0.0, tg = 1.0;
+      bool ok = false;
+      if (cell) {
+        double mom[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-      for (int i = 0; i < QP_MAX; ++i) {
-        if (i < Qp) {
-          double Si[3];
+        for (int i = 0; i < QP_MAX; ++i) {
+          if (i < Qp) {
+            double Si[3];
 #pragma unroll
-          for (int q = 0; q < 3; ++q)
-            Si[q] = (sm.u.red[0][3 * i + q][c] + sm.u.red[1][3 * i + q][c]) +
-                    (sm.u.red[2][3 * i + q][c] + sm.u.red[3][3 * i + q][c]);
-          const double p1 = tab[TAB_PBAR + i], p2 = tab[TAB_PBAR2 + i];
-          mom[0] = fma(p1, Si[0], mom[0]);
-          mom[1] = fma(p1, Si[1], mom[1]);
-          mom[2] = fma(p2, Si[0], mom[2]);
-          mom[3] = fma(p2, Si[1], mom[3]);
-          mom[4] = fma(p2, Si[2], mom[4]);
+            for (int q = 0; q < 3; ++q)
+              Si[q] = (sm.u.a.red[0][3 * i + q][c] + sm.u.a.red[1][3 * i + q][c]) +
+                      (sm.u.a.red[2][3 * i + q][c] + sm.u.a.red[3][3 * i + q][c]);
+            const double p1 = tab[TAB_PBAR + i], p2 = tab[TAB_PBAR2 + i];
+            mom[0] = fma(p1, Si[0], mom[0]);
+            mom[1] = fma(p1, Si[1], mom[1]);
+            mom[2] = fma(p2, Si[0], mom[2]);
+            mom[3] = fma(p2, Si[1], mom[3]);
+            mom[4] = fma(p2, Si[2], mom[4]);
+          }
         }
+        ok = landau_frame(mom, beta, b2, g1, gam, g0, tg);
+        if (ok && A.warn != nullptr && stiff(T, beta)) atomicOr(A.warn, RLB_WARN_STIFF);
+        ok = ok && fabs(beta) <= beta_limit(NPc);
+        if (!ok) atomicOr(A.flag, 1);
       }
-      ok = landau(mom, e, beta, n, Tt);
-      if (!ok) atomicOr(A.flag, 1);
-      else if (A.warn != nullptr && stiff(T, beta)) atomicOr(A.warn, RLB_WARN_STIFF);
-    }
-    __syncthreads();  // the moments are consumed; the union now holds the coefficient scratch
-    if (g == 0 && c < GW) {
-      sm.u.coef.cell[0][c] = n;
-      sm.u.coef.cell[1][c] = Tt;
-      sm.u.coef.cell[2][c] = beta;
-      sm.u.coef.ok[c] = ok ? 1 : 0;
+      store_cell_coeffs<NPc, NVc>(ok, beta, b2, g1, g0, tg, sm.u.a.coef, c);
       // b dt gamma / tau and its beta multiple: the stage's collision rate is r0 - r1 xi_j
-      const double r0 = ok ? (A.b * T.dt) * (T.inv_tau / sqrt(1.0 - beta * beta)) : 0.0;
+      const double r0 = ok ? (A.b * T.dt) * (T.inv_tau * gam) : 0.0;
       sm.rate[0][c] = r0;
-      sm.rate[1][c] = r0 * beta;
+      sm.rate[1][c] = ok ? r0 * beta : 0.0;
     }
     __syncthreads();
-    tile_coeffs<NPc, NVc>(tab, Qp, sm.u.coef, sm.B, A.flag);
+    build_rows<NPc, NVc>(tab, Qp, sm.u.a.coef, sm.B);
   }
   __syncthreads();  // sm.src (and, with collisions, the coefficients) are ready
 
@@ -334,12 +376,12 @@ __device__ void stage_tile(const StageArgs& A, const TubeDev& T, int x0, int par
   //    barriers only.
   const double a = A.a, b = A.b;
   const double* cxi_tab = tab + tab_cxi(Qxi) + A.stage * Qxi;
-  double* d1 = sm.d1[g];
-  float2* dd = sm.dd[g];
-  float2* sv0 = sm.sv[g][0];
-  float2* sv1 = sm.sv[g][1];
-  float2* sv2 = sm.sv[g][2];
-  float2* phi = sm.phi[g];
+  double* d1 = sm.u.c.d1[g];
+  float2* dd = sm.u.c.dd[g];
+  float2* sv0 = sm.u.c.sv[g][0];
+  float2* sv1 = sm.u.c.sv[g][1];
+  float2* sv2 = sm.u.c.sv[g][2];
+  float2* phi = sm.u.c.phi[g];
   const float2* epsf = reinterpret_cast<const float2*>(tab + tab_epsf(Qp, Qxi));
   const int hq = Qxi / 2, upr = hq + (Qxi & 1), U = Qp * upr;
   const int u_end = (part + 1) * U / nparts;
@@ -353,7 +395,7 @@ __device__ void stage_tile(const StageArgs& A, const TubeDev& T, int x0, int par
     for (int h = 0; h < nrow; ++h, buf ^= 1) {
       const int j = h == 0 ? jA : Qxi - 1 - jA;
       const int s = i * Qxi + j;
-      double* row = sm.row[buf][g];
+      double* row = sm.u.c.row[buf][g];
       // stage the row with its first differences, in FP64 and split into double-float (position k needs k - 1
       // as well)
       {

@@ -98,75 +98,55 @@ __host__ __device__ constexpr size_t rp_smem_bytes(int brows) {
 // Coefficient rows of a tube as the kernel stores them.
 __host__ __device__ inline int rp_brows(int Qp, int Np, int Nv) { return Qp * ((Np == 2 && Nv == 5) ? 6 : NV_MAX + 1); }
 
-// Per-cell FP64 phase of one cell: Landau frame of the stored moments, hhat_{m,k} by the positive power
-// series (both parities, in registers), B[i][k] = n/(4T^3) w^p_i sum_q s^(q+2) K[i][q] hhat_{q+2,k} (as the
-// FP64 kernel's tile_coeffs) stored as FP32 in column `col`, and the stage's collision rate
-// b dt gamma (1 - beta xi)/tau = rt0 - rt1 xi. A non-physical cell raises the flag and gets B = 0, rate 0.
+// Per-cell FP64 phase of one cell: Landau frame of the stored moments, Legendre and equilibrium coefficients (as the
+// FP64 kernel's, in registers) stored as FP32 in column `col`, and the stage's collision rate
+// b dt gamma (1 - beta xi)/tau = rt0 - rt1 xi. A non-physical cell raises the flag and gets B = 0, rate 0. A cell at
+// rest (T0x = 0, exactly so wherever the state is symmetric in xi) has B[i][0] only.
 template <int NPc, int NVc>
-__device__ void cell_coeffs_rp(const TubeDev* Tg, const double* tab, int Qp, const double mom[5], double bdt_itau,
+__device__ __forceinline__ void cell_coeffs_rp(const TubeDev* Tg, const double* tab, int Qp, const double mom[5], double bdt_itau,
                                int* flag, const RpWarp& w, int col, float& rt0, float& rt1) {
-  double e, beta, n, Tt, gam;
-  bool ok = landau(mom, e, beta, n, Tt, &gam);
+  double beta, b2, g1, gam, g0, tg;
+  bool ok = landau_frame(mom, beta, b2, g1, gam, g0, tg);
   // flag[1] holds the sticky warning bits (RLB_WARN_*); the tube record is read from global memory here
   if (ok && flag != nullptr && stiff(*Tg, beta)) atomicOr(flag + 1, RLB_WARN_STIFF);
-  if (ok && beta == 0.0) {
-    // at rest hhat_{m,k} = delta_{k0}: only B[i][0] = n/(4T^3) w^p_i sum_q T^(q+2) K[i][q] is nonzero (the same
-    // FP64 operations as the general path below takes at beta = 0)
-    const double pref = n / (4.0 * Tt * Tt * Tt);
-#pragma unroll
-    for (int i = 0; i < QP_MAX; ++i) {
-      if (i < Qp) {
-        const double pw = pref * tab[TAB_WP + i];
-        double B0 = 0.0, sq = Tt * Tt;
-#pragma unroll
-        for (int q = 0; q <= NPc; ++q) {
-          const double G = pw * sq * tab[TAB_K + i * (NP_MAX + 1) + q];
-          B0 = fma(G, 1.0, B0);
-          sq *= Tt;
-        }
-        w.B[rp_brow(i, 0, Qp, NVc + 1) * RP_WT + col] = (float)B0;
-#pragma unroll
-        for (int k = 1; k <= NVc; ++k) w.B[rp_brow(i, k, Qp, NVc + 1) * RP_WT + col] = 0.f;
-      }
-    }
-    rt0 = (float)bdt_itau;
-    rt1 = 0.f;
-    return;
-  }
-  double hh[(NPc + 1) * (NV_MAX + 1)];
-#pragma unroll
-  for (int k = 0; k < (NPc + 1) * (NV_MAX + 1); ++k) hh[k] = 0.0;
-  if (ok) {
-    const bool c0 = hhat_parity<NPc, NVc, 0, 1>(beta, hh);
-    const bool c1 = hhat_parity<NPc, NVc, 1, 1>(beta, hh);
-    ok = c0 && c1;
-  }
+  ok = ok && fabs(beta) <= beta_limit(NPc);
   if (!ok && flag) atomicOr(flag, 1);
-  const double s = ok ? Tt / gam : 0.0;
+  double ge[NPc + 1][NVc + 1];
 #pragma unroll
-  for (int i = 0; i < QP_MAX; ++i) {
-    double B[NVc + 1];
+  for (int q = 0; q <= NPc; ++q)
 #pragma unroll
-    for (int k = 0; k <= NVc; ++k) B[k] = 0.0;
-    if (ok && i < Qp) {
-      const double pref = n / (4.0 * Tt * Tt * Tt) * tab[TAB_WP + i];
-      double sq = s * s;
+    for (int k = 0; k <= NVc; ++k) ge[q][k] = 0.0;
+  if (ok) {
+    if (beta == 0.0) {
+      double g = g0, f = 1.0;  // h[q][0] = (q + 1)! at rest
 #pragma unroll
       for (int q = 0; q <= NPc; ++q) {
-        const double G = pref * sq * tab[TAB_K + i * (NP_MAX + 1) + q];
-#pragma unroll
-        for (int k = 0; k <= NVc; ++k) B[k] = fma(G, hh[q * (NV_MAX + 1) + k], B[k]);
-        sq *= s;
+        f *= q + 1;
+        ge[q][0] = f * g;
+        g *= tg;
       }
+    } else {
+      cell_coeffs<NPc, NVc>(beta, b2, g1, g0, tg, ge);
     }
-    if (i < Qp) {
+  }
 #pragma unroll
-      for (int k = 0; k <= NVc; ++k) w.B[rp_brow(i, k, Qp, NVc + 1) * RP_WT + col] = (float)B[k];
+  for (int i = 0; i < QP_MAX; ++i) {
+    if (i < Qp) {
+      double KW[NPc + 1];
+#pragma unroll
+      for (int q = 0; q <= NPc; ++q) KW[q] = tab[TAB_KW + i * (NP_MAX + 1) + q];
+#pragma unroll
+      for (int k = 0; k <= NVc; ++k) {
+        double B = KW[0] * ge[0][k];
+#pragma unroll
+        for (int q = 1; q <= NPc; ++q) B = fma(KW[q], ge[q][k], B);
+        w.B[rp_brow(i, k, Qp, NVc + 1) * RP_WT + col] = (float)B;
+      }
     }
   }
   const double r0 = ok ? bdt_itau * gam : 0.0;
   rt0 = (float)r0;
-  rt1 = (float)(r0 * beta);
+  rt1 = ok ? (float)(r0 * beta) : 0.0f;
 }
 
 // One velocity row as a lane holds it: its RP_C cells xl .. xl+3 (xl = x0 - RP_C + RP_C lane, so that lane 0
