@@ -3,7 +3,7 @@
 // its C ABI (include/rlb.h).
 //
 // One SSP-RK3 stage is one launch of rlb_stage_kernel over every tile of every tube. A CTA owns a tile of
-// TX = 61 cells of one tube and, for those cells:
+// TX = 60 cells of one tube and, for those cells:
 //   A. reduces F over all Q velocities to N^0, N^x, T^00, T^0x, T^xx (section "Relativistic lattice
 //      Boltzmann equation");
 //   B. solves the Landau-frame eigenproblem T^mu_nu u^nu = -e u^mu for e, v, n and builds the per-cell
@@ -452,6 +452,7 @@ bool fill_tube_tables(const rlb_tube& t, double* pb, double* wp, double* xi, dou
   }
   for (int j = 0; j < t.Qxi; ++j) {
     T[TAB_XI + j] = xi[j];
+    T[tab_xi2(t.Qp, t.Qxi) + j] = xi[j] * xi[j];
     for (int k = 0; k <= NV_MAX; ++k)
       T[tab_pw(t.Qxi) + j * (NV_MAX + 1) + k] = k <= t.Nv ? wxi[j] * rlbq::legendre(k, xi[j]) : 0.0;
     for (int st = 0; st < 3; ++st) T[tab_cxi(t.Qxi) + st * t.Qxi + j] = RK_B[st] * t.dt * xi[j] / t.dx;

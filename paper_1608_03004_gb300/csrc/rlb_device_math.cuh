@@ -193,17 +193,60 @@ __device__ __forceinline__ void df_add(DF& acc, DF a) {
 
 
 // ---------------------------------------------------------------------------------------------------------
-// WENO5 limiter of the FP64 stage kernel in double-float arithmetic.
+// Packed FP32 arithmetic: two floats in a 64-bit register pair, one instruction per operation on both
+// (fma/add/sub/mul.rn.f32x2: each half rounded as the scalar operation rounds it, never contracted). On GB300 a
+// packed operation occupies the FP32 pipe like two scalar ones (1.94 of them per SM and clock, measured, against 3.9
+// scalar) but takes one issue slot instead of two.
+struct F2 {
+  unsigned long long v;
+};
+__device__ __forceinline__ F2 f2(float x, float y) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ F2 f2(float x) { return f2(x, x); }
+__device__ __forceinline__ float lo_of(F2 a) { return __uint_as_float((unsigned)a.v); }
+__device__ __forceinline__ float hi_of(F2 a) { return __uint_as_float((unsigned)(a.v >> 32)); }
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 sub2(F2 a, F2 b) {
+  F2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ F2 neg2(F2 a) { return {a.v ^ 0x8000000080000000ull}; }
+
+// Two double-floats, one in each half.
+struct DF2 {
+  F2 hi, lo;
+};
+
+// ---------------------------------------------------------------------------------------------------------
+// WENO5 limiter of the FP64 stage kernel in double-float arithmetic, two interfaces at a time.
 //
-// GB300 executes FP32 at 64 times its FP64 rate, and the FP64 stage kernel is bound by the FP64 pipe while
-// its issue slots are mostly idle. The limiter (indicators, nonlinear weights, the weighted candidate sum) is
-// about two thirds of the kernel's FP64 operations, so the kernel evaluates it in double-float: a value is
-// an unevaluated sum hi + lo of two floats (about 47 significant bits), combined with the error-free
-// transformations TwoSum (Knuth), FastTwoSum (Dekker) and the FMA-based TwoProduct. Every product and sum is
-// written with explicit rounding (fmaf, __fmul_rn, __fadd_rn, __fsub_rn), so that the compiler cannot fuse
-// or reorder what the transformations rely on. The differences entering the limiter come from the FP64
-// state; the 6 G returned per interface carries an absolute error of a few 1e-14 of the differences around
-// it (the error of the limiter's FP64 form is ~1e-16 of them), well inside the FP64 path's 1e-12 parity.
+// GB300 executes FP32 at 64 times its FP64 rate, and the FP64 stage kernel is bound by the FP64 pipe. The limiter
+// (indicators, nonlinear weights, the weighted candidate sum) is about two thirds of the method's FP64 operations,
+// so the kernel evaluates it in double-float: a value is an unevaluated sum hi + lo of two floats (about 47
+// significant bits), combined with the error-free transformations TwoSum (Knuth), FastTwoSum (Dekker) and the
+// FMA-based TwoProduct. The two halves of every packed operand belong to the two rows of a mirror pair of
+// directions: the row with the wind toward -x is held in reversed order, so that both rows take the same operations.
+// The differences entering the limiter come from the FP64 state; the 6 G returned per interface carries an
+// absolute error of a few 1e-14 of the differences around it (the error of the limiter's FP64 form is ~1e-16 of
+// them), well inside the FP64 path's 1e-12 parity.
 //
 // Indicators: with the linear weights d = (1, 6, 3)/10 taken out of the squares, the three indicators of a
 // pair of adjacent differences (x, y) are v = S + e with S the integer quadratic forms
@@ -213,52 +256,57 @@ __device__ __forceinline__ void df_add(DF& acc, DF a) {
 // the weights d_k / t_k multiplied through by t0 t1 t2 / 10 (r_k as in weno5_combine6). The v_k of one
 // interface are first scaled by a common power of two so that the largest lies in [1, 2): the weights are
 // homogeneous in t, and the scaling keeps the products of the t's inside the FP32 exponent range.
+//
+// A packed operation has no free sign change, so a product is formed negated where its rounding error needs it
+// (-p from (-a) b, then a b + (-p)) and the sums of such products run on the negated values: negation is exact, so
+// nothing else changes.
 
-// a + b = s + e exactly, |a| >= |b| (or a == 0)
-__device__ __forceinline__ DF fast_two_sum(float a, float b) {
-  const float s = __fadd_rn(a, b);
-  return {s, __fsub_rn(b, __fsub_rn(s, a))};
+// s + e = a + b exactly, for the high parts of sums
+__device__ __forceinline__ void two_sum2(F2 a, F2 b, F2& s, F2& e) {
+  s = add2(a, b);
+  const F2 bb = sub2(s, a);
+  e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
 }
 
-// a + b, robust to cancellation of the high parts
-__device__ __forceinline__ DF df_plus(DF a, DF b) {
-  float s, t;
-  two_sum(a.hi, b.hi, s, t);
-  t = __fadd_rn(t, __fadd_rn(a.lo, b.lo));
-  float u, w;
-  two_sum(s, t, u, w);
-  return {u, w};
+// a + b = s + e exactly, |a| >= |b|, with a given negated (na = -a)
+__device__ __forceinline__ DF2 fast_two_sum_n(F2 na, F2 b) {
+  const F2 s = sub2(b, na);
+  return {s, sub2(b, add2(s, na))};
+}
+
+// a + b of two double-floats whose high parts are summed as s + t, t completed with the low parts: the last TwoSum
+// (robust to cancellation of the high parts)
+__device__ __forceinline__ DF2 renorm2(F2 s, F2 t) {
+  DF2 r;
+  two_sum2(s, t, r.hi, r.lo);
+  return r;
+}
+__device__ __forceinline__ DF2 df2_plus(DF2 a, DF2 b) {
+  F2 s, t;
+  two_sum2(a.hi, b.hi, s, t);
+  return renorm2(s, add2(t, add2(a.lo, b.lo)));
+}
+__device__ __forceinline__ DF2 df2_minus(DF2 a, DF2 b) {
+  const F2 s = sub2(a.hi, b.hi), bb = sub2(s, a.hi);
+  const F2 t = sub2(sub2(a.hi, sub2(s, bb)), add2(b.hi, bb));
+  return renorm2(s, add2(t, sub2(a.lo, b.lo)));
 }
 
 // a + b for a, b >= 0 (no cancellation)
-__device__ __forceinline__ DF df_plus_pos(DF a, DF b) {
-  float s, t;
-  two_sum(a.hi, b.hi, s, t);
-  return fast_two_sum(s, __fadd_rn(t, __fadd_rn(a.lo, b.lo)));
+__device__ __forceinline__ DF2 df2_plus_pos(DF2 a, DF2 b) {
+  F2 s, t;
+  two_sum2(a.hi, b.hi, s, t);
+  t = add2(t, add2(a.lo, b.lo));
+  const F2 u = add2(s, t);
+  return {u, sub2(t, sub2(u, s))};
 }
 
-__device__ __forceinline__ DF df_neg(DF a) { return {-a.hi, -a.lo}; }
+__device__ __forceinline__ DF2 df2_pow2(DF2 a, F2 p) { return {mul2(a.hi, p), mul2(a.lo, p)}; }
 
-// a * 2^k for a float power of two p (exact)
-__device__ __forceinline__ DF df_pow2(DF a, float p) { return {__fmul_rn(a.hi, p), __fmul_rn(a.lo, p)}; }
-
-__device__ __forceinline__ DF df_times(DF a, DF b) {
-  const float p = __fmul_rn(a.hi, b.hi);
-  const float e = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, fmaf(a.hi, b.hi, -p)));
-  return fast_two_sum(p, e);
-}
-
-__device__ __forceinline__ DF df_square(DF a) {
-  const float p = __fmul_rn(a.hi, a.hi);
-  const float e = fmaf(__fadd_rn(a.hi, a.hi), a.lo, fmaf(a.hi, a.hi, -p));
-  return fast_two_sum(p, e);
-}
-
-// a * c for a small integer c (exactly representable), unnormalised: the product of the high parts rounded,
-// its rounding error and c a.lo in the second float
-__device__ __forceinline__ DF df_times_int(DF a, float c) {
-  const float p = __fmul_rn(a.hi, c);
-  return {p, fmaf(a.lo, c, fmaf(a.hi, c, -p))};
+// a * b, with -a.hi given
+__device__ __forceinline__ DF2 df2_times(DF2 a, F2 na, DF2 b) {
+  const F2 np = mul2(na, b.hi);
+  return fast_two_sum_n(np, fma2(a.hi, b.lo, fma2(a.lo, b.hi, fma2(a.hi, b.hi, np))));
 }
 
 // d = hi + lo with hi the top 24 significant bits of d (truncated) and lo the next 23 (|lo| < ulp(hi)); by
@@ -268,8 +316,9 @@ __device__ __forceinline__ DF df_split(double d) {
   const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
   const int e = (int)((hi >> 20) & 0x7FFu);
   if (e <= 896) return {0.0f, 0.0f};
-  if (e >= 1151) return {__double2float_rn(d), 0.0f};
   const unsigned sgn = hi & 0x80000000u;
+  // (integer operations here too: a conversion would be taken out of the branch and occupy the FP64 pipe)
+  if (e >= 1151) return {__uint_as_float(sgn | 0x7F800000u | (e == 2047 && ((hi & 0xFFFFFu) | lo) ? 1u : 0u)), 0.0f};
   const float h = __uint_as_float(sgn | ((unsigned)(e - 896) << 23) | (__funnelshift_l(lo, hi, 3) & 0x7FFFFFu));
   float l = 0.0f;
   if (e >= 920) {  // x 2^(E - 46) with x the next 23 bits, E = e - 1023: (2^23 + x) 2^(E - 23) - 2^(E - 23)
@@ -287,82 +336,141 @@ __device__ __forceinline__ double df_widen(float f) {
   return ef == 0u ? 0.0 : w;
 }
 
-// Indicators v_A, v_B, v_C of the pair (x, y) = (d_j, d_{j+1}) in memory order, e the epsilon term. fwd (wind
-// toward increasing index): (v_A, v_B, v_C) = (SL, SC, SR)(x, y) + e; otherwise SL and SR trade places.
-__device__ __forceinline__ void weno5_pair_df(DF x, DF y, bool fwd, DF e, DF& vA, DF& vB, DF& vC) {
-  // x^2, x y, y^2 as (rounded product of the high parts, its error plus the cross terms)
-  const float px = __fmul_rn(x.hi, x.hi), py = __fmul_rn(y.hi, y.hi), pz = __fmul_rn(x.hi, y.hi);
-  const DF X = {px, fmaf(__fadd_rn(x.hi, x.hi), x.lo, fmaf(x.hi, x.hi, -px))};
-  const DF Y = {py, fmaf(__fadd_rn(y.hi, y.hi), y.lo, fmaf(y.hi, y.hi, -py))};
-  const DF Z = {pz, fmaf(x.hi, y.lo, fmaf(x.lo, y.hi, fmaf(x.hi, y.hi, -pz)))};
-  const DF X4 = df_pow2(X, 4.0f), Y4 = df_pow2(Y, 4.0f);
-  const DF X10 = df_times_int(X, 10.0f), Y10 = df_times_int(Y, 10.0f);
-  const DF Z11 = df_times_int(Z, -11.0f), Z5 = df_times_int(Z, -5.0f);
-  // (a, b, c) + e: exact sums of the high parts, then the low parts and the errors; v > 0 is a positive
-  // definite form plus e, so the final FastTwoSum's ordering holds
-  auto sum3 = [&](DF a, DF b, DF c) {
-    float s, t1, t2, t3;
-    two_sum(a.hi, b.hi, s, t1);
-    two_sum(s, c.hi, s, t2);
-    two_sum(s, e.hi, s, t3);
-    const float lo = __fadd_rn(__fadd_rn(__fadd_rn(a.lo, b.lo), __fadd_rn(c.lo, e.lo)),
-                               __fadd_rn(__fadd_rn(t1, t2), t3));
-    return fast_two_sum(s, lo);
-  };
-  const DF L = sum3(X4, Z11, Y10), R = sum3(X10, Z11, Y4);
-  vA = fwd ? L : R;
-  vB = sum3(X4, Z5, Y4);
-  vC = fwd ? R : L;
+// hi + lo of a normalised double-float (|lo| <= ulp(hi)/2) as one double, rounded at its 53rd bit: an addition on the
+// bits of hi widened, in place of an FP64 operation that widens lo on its own. Where lo points toward zero, the float
+// next to hi is widened and lo is added to 2^29 units of that double's last place, so that the sum never leaves the
+// binade whose units it counts. Zero and subnormal hi give 0; infinities and NaN pass through.
+__device__ __forceinline__ double df_join(float hi, float lo) {
+  const unsigned b = __float_as_uint(hi), ef = (b >> 23) & 0xFFu;
+  if (ef == 0u) return 0.0;
+  // (no conversion instruction here: it would be taken out of the branch and occupy the FP64 pipe for every value)
+  if (ef == 255u) return __hiloint2double((int)((b & 0x80000000u) | 0x7FF00000u | ((b >> 3) & 0xFFFFFu)), (int)(b << 29));
+  const unsigned bl = __float_as_uint(lo), down = (b ^ bl) >> 31, p = b - down, ep = (p >> 23) & 0xFFu;
+  // lo, with hi's sign taken out, in units of 2^(ep - 127 - 52): scale 2^(179 - ep), in two factors where it exceeds
+  // FP32's range
+  float l = __uint_as_float(bl ^ (b & 0x80000000u));
+  unsigned top = 306u;
+  if (ef < 64u) {
+    l = __fmul_rn(l, 0x1p64f);
+    top = 242u;
+  }
+  const unsigned add = (unsigned)__float2int_rn(__fmul_rn(l, __uint_as_float((top - ep) << 23))) + (down << 29);
+  const unsigned wh = (p & 0x80000000u) | (((p & 0x7FFFFFFFu) >> 3) + (896u << 20)), wl = (p << 29) + add;
+  return __hiloint2double((int)(wh + (wl < add ? 1u : 0u)), (int)wl);
 }
 
-// 6 G of the interface from the indicators (v0, v1, v2) of its stencils and the differences d1..d4 in wind
-// order, in double-float.
-__device__ __forceinline__ DF weno5_combine6_df(DF v0, DF v1, DF v2, DF d1, DF d2, DF d3, DF d4) {
-  // common power-of-two scale: the largest v lands in [1, 2)
-  const unsigned em = __float_as_uint(fmaxf(fmaxf(v0.hi, v1.hi), v2.hi)) >> 23;
-  const float sc = __uint_as_float((254u - em) << 23);
-  const DF t0 = df_square(df_pow2(v0, sc)), t1 = df_square(df_pow2(v1, sc)), t2 = df_square(df_pow2(v2, sc));
+// Indicators v_A, v_B, v_C of the pairs (x, y) = (d_j, d_{j+1}) in wind order, e the epsilon term:
+// (v_A, v_B, v_C) = (SL, SC, SR)(x, y) + e.
+__device__ __forceinline__ void weno5_pair_df2(DF2 x, DF2 y, F2 ne_hi, F2 e_lo, DF2& vA, DF2& vB, DF2& vC) {
+  // -x^2, -x y, -y^2 rounded (the high parts), their errors plus the cross terms (the low parts)
+  const F2 nx = neg2(x.hi), ny = neg2(y.hi);
+  const F2 X = mul2(nx, x.hi), Y = mul2(ny, y.hi), Z = mul2(nx, y.hi);
+  const F2 Xl = fma2(add2(x.hi, x.hi), x.lo, fma2(x.hi, x.hi, X));
+  const F2 Yl = fma2(add2(y.hi, y.hi), y.lo, fma2(y.hi, y.hi, Y));
+  const F2 Zl = fma2(x.hi, y.lo, fma2(x.lo, y.hi, fma2(x.hi, y.hi, Z)));
+  const F2 c4 = f2(4.0f), c5 = f2(5.0f), c10 = f2(10.0f), c11 = f2(11.0f);
+  const F2 m5 = f2(-5.0f), m10 = f2(-10.0f), m11 = f2(-11.0f);
+  // the integer multiples, high parts negated
+  const F2 X4 = mul2(X, c4), Y4 = mul2(Y, c4), X4l = mul2(Xl, c4), Y4l = mul2(Yl, c4);
+  const F2 X10 = mul2(X, c10), X10l = fma2(Xl, c10, fma2(X, m10, X10));
+  const F2 Y10 = mul2(Y, c10), Y10l = fma2(Yl, c10, fma2(Y, m10, Y10));
+  const F2 Z11 = mul2(Z, m11), Z11l = fma2(Zl, m11, fma2(Z, c11, Z11));
+  const F2 Z5 = mul2(Z, m5), Z5l = fma2(Zl, m5, fma2(Z, c5, Z5));
+  // (a, b, c) + e: exact sums of the (negated) high parts, then the low parts and the errors; v > 0 is a positive
+  // definite form plus e, so the final FastTwoSum's ordering holds
+  auto sum3 = [&](F2 a, F2 al, F2 b, F2 bl, F2 c, F2 cl) {
+    F2 s, t1, t2, t3;
+    two_sum2(a, b, s, t1);
+    two_sum2(s, c, s, t2);
+    two_sum2(s, ne_hi, s, t3);
+    const F2 lo = sub2(add2(add2(al, bl), add2(cl, e_lo)), add2(add2(t1, t2), t3));
+    return fast_two_sum_n(s, lo);
+  };
+  vA = sum3(X4, X4l, Z11, Z11l, Y10, Y10l);
+  vB = sum3(X4, X4l, Z5, Z5l, Y4, Y4l);
+  vC = sum3(X10, X10l, Z11, Z11l, Y4, Y4l);
+}
+
+// 1 / 2^(exponent of the largest v): the scale that brings it into [1, 2)
+__device__ __forceinline__ float weno5_scale(float v0, float v1, float v2) {
+  return __uint_as_float((254u - (__float_as_uint(fmaxf(fmaxf(v0, v1), v2)) >> 23)) << 23);
+}
+
+// 6 G of two interfaces from the indicators (v0, v1, v2) of their stencils and the differences d1..d4 in wind order.
+__device__ __forceinline__ DF2 weno5_combine6_df2(DF2 v0, DF2 v1, DF2 v2, DF2 d1, DF2 d2, DF2 d3, DF2 d4) {
+  const F2 sc = f2(weno5_scale(lo_of(v0.hi), lo_of(v1.hi), lo_of(v2.hi)),
+                   weno5_scale(hi_of(v0.hi), hi_of(v1.hi), hi_of(v2.hi)));
+  const F2 nsc = neg2(sc);
+  auto square = [&](DF2 v) {
+    const F2 h = mul2(v.hi, sc), nh = mul2(v.hi, nsc), l = mul2(v.lo, sc), np = mul2(nh, h);
+    return fast_two_sum_n(np, fma2(add2(h, h), l, fma2(h, h, np)));
+  };
+  const DF2 t0 = square(v0), t1 = square(v1), t2 = square(v2);
   // r0 = 5 d2 - 2 d1, r1 = d2 + 2 d3, r2 = 4 d3 - d4 (6 times the candidates' corrections)
-  const DF r0 = df_plus(df_times_int(d2, 5.0f), df_pow2(d1, -2.0f));
-  const DF r1 = df_plus(d2, df_pow2(d3, 2.0f));
-  const DF r2 = df_plus(df_pow2(d3, 4.0f), df_neg(d4));
-  const DF a0 = df_times(t1, t2);
-  const DF t0x3 = df_times_int(t0, 3.0f);
-  const DF t03 = fast_two_sum(t0x3.hi, t0x3.lo);
-  const DF num = df_plus(df_times(a0, r0),
-                         df_times(t03, df_plus(df_pow2(df_times(t2, r1), 2.0f), df_times(t1, r2))));
-  const DF den = df_plus_pos(a0, df_times(t03, df_plus_pos(df_pow2(t2, 2.0f), t1)));
-  if (den.hi == 0.0f) {  // all but one t below FP32's range (indicator ratios beyond ~1e19): that stencil's value
-    const bool k0 = v0.hi <= v1.hi && v0.hi <= v2.hi, k1 = !k0 && v1.hi <= v2.hi;
-    return k0 ? r0 : (k1 ? r1 : r2);
-  }
+  const F2 c2 = f2(2.0f), c3 = f2(3.0f), c4 = f2(4.0f), c5 = f2(5.0f), m5 = f2(-5.0f);
+  const F2 n5 = mul2(d2.hi, m5);
+  const DF2 r0 = df2_minus({neg2(n5), fma2(d2.lo, c5, fma2(d2.hi, c5, n5))}, df2_pow2(d1, c2));
+  const DF2 r1 = df2_plus(d2, df2_pow2(d3, c2));
+  const DF2 r2 = df2_minus(df2_pow2(d3, c4), d4);
+  const F2 nt1 = neg2(t1.hi), nt2 = neg2(t2.hi);
+  const DF2 a0 = df2_times(t1, nt1, t2);
+  const F2 n3 = mul2(t0.hi, f2(-3.0f));
+  const DF2 t03 = fast_two_sum_n(n3, fma2(t0.lo, c3, fma2(t0.hi, c3, n3)));
+  const F2 nt03 = neg2(t03.hi);
+  const DF2 num = df2_plus(df2_times(a0, neg2(a0.hi), r0),
+                           df2_times(t03, nt03, df2_plus(df2_pow2(df2_times(t2, nt2, r1), c2), df2_times(t1, nt1, r2))));
+  const DF2 den = df2_plus_pos(a0, df2_times(t03, nt03, df2_plus_pos(df2_pow2(t2, c2), t1)));
   // num / den: a quotient from FP32's reciprocal (approximation refined by one Newton-Raphson step to about
   // half an ulp), then one correction from the remainder
-  float rc;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc) : "f"(den.hi));
-  rc = fmaf(rc, fmaf(-den.hi, rc, 1.0f), rc);
-  const float q1 = __fmul_rn(num.hi, rc);
-  const float p = __fmul_rn(q1, den.hi);
-  const float pe = fmaf(q1, den.lo, fmaf(q1, den.hi, -p));
-  const float rem = __fadd_rn(__fsub_rn(num.hi, p), __fsub_rn(num.lo, pe));
-  float s, t;
-  two_sum(q1, __fmul_rn(rem, rc), s, t);
-  return {s, t};
+  float ra, rb;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ra) : "f"(lo_of(den.hi)));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rb) : "f"(hi_of(den.hi)));
+  F2 rc = f2(ra, rb);
+  const F2 nden = neg2(den.hi);
+  rc = fma2(rc, fma2(nden, rc, f2(1.0f)), rc);
+  const F2 q1 = mul2(num.hi, rc), np = mul2(q1, nden);
+  const F2 pe = fma2(q1, den.lo, fma2(q1, den.hi, np));
+  const F2 rem = add2(add2(num.hi, np), sub2(num.lo, pe));
+  DF2 G;
+  two_sum2(q1, mul2(rem, rc), G.hi, G.lo);
+  // all but one t below FP32's range (indicator ratios beyond ~1e19): that stencil's value
+  const float da = lo_of(den.hi), db = hi_of(den.hi);
+  if (da == 0.0f || db == 0.0f) {
+    auto pick = [&](float a0_, float a1_, float a2_, float x0, float x1, float x2) {
+      const bool k0 = a0_ <= a1_ && a0_ <= a2_, k1 = !k0 && a1_ <= a2_;
+      return k0 ? x0 : (k1 ? x1 : x2);
+    };
+    float gh[2] = {lo_of(G.hi), hi_of(G.hi)}, gl[2] = {lo_of(G.lo), hi_of(G.lo)};
+    if (da == 0.0f) {
+      gh[0] = pick(lo_of(v0.hi), lo_of(v1.hi), lo_of(v2.hi), lo_of(r0.hi), lo_of(r1.hi), lo_of(r2.hi));
+      gl[0] = pick(lo_of(v0.hi), lo_of(v1.hi), lo_of(v2.hi), lo_of(r0.lo), lo_of(r1.lo), lo_of(r2.lo));
+    }
+    if (db == 0.0f) {
+      gh[1] = pick(hi_of(v0.hi), hi_of(v1.hi), hi_of(v2.hi), hi_of(r0.hi), hi_of(r1.hi), hi_of(r2.hi));
+      gl[1] = pick(hi_of(v0.hi), hi_of(v1.hi), hi_of(v2.hi), hi_of(r0.lo), hi_of(r1.lo), hi_of(r2.lo));
+    }
+    G = {f2(gh[0], gh[1]), f2(gl[0], gl[1])};
+  }
+  return G;
 }
 
 // Interface value v2 + G computed as the FP64 stage kernel does with the double-float limiter (differences in
-// FP64, split, pairs, combination, 6 G widened and divided by 6 in FP64); eps: the limiter's epsilon.
+// FP64, split, pairs, combination, 6 G widened and divided by 6 in FP64); eps: the limiter's epsilon. A wind
+// toward decreasing index takes the samples in reversed order. Both halves of the packed operands hold the interface.
 __device__ __forceinline__ double weno5_interface_df(double m0, double m1, double m2, double m3, double m4, bool fwd,
                                                      double eps = WENO_EPS) {
-  const DF D1 = df_split(m1 - m0), D2 = df_split(m2 - m1), D3 = df_split(m3 - m2), D4 = df_split(m4 - m3);
-  const DF e = df_split(3.0 * eps);
-  DF a[3], b[3], c[3];
-  weno5_pair_df(D1, D2, fwd, e, a[0], b[0], c[0]);
-  weno5_pair_df(D2, D3, fwd, e, a[1], b[1], c[1]);
-  weno5_pair_df(D3, D4, fwd, e, a[2], b[2], c[2]);
-  const DF G = fwd ? weno5_combine6_df(a[0], b[1], c[2], D1, D2, D3, D4)
-                   : weno5_combine6_df(a[2], b[1], c[0], df_neg(D4), df_neg(D3), df_neg(D2), df_neg(D1));
-  return fma(df_widen(G.hi), 1.0 / 6.0, fma(df_widen(G.lo), 1.0 / 6.0, m2));
+  const double v0 = fwd ? m0 : m4, v1 = fwd ? m1 : m3, v3 = fwd ? m3 : m1, v4 = fwd ? m4 : m0;
+  auto both = [](DF q) { return DF2{f2(q.hi), f2(q.lo)}; };
+  const DF2 D1 = both(df_split(v1 - v0)), D2 = both(df_split(m2 - v1)), D3 = both(df_split(v3 - m2)),
+            D4 = both(df_split(v4 - v3));
+  const DF2 e = both(df_split(3.0 * eps));
+  const F2 ne = neg2(e.hi);
+  DF2 a[3], b[3], c[3];
+  weno5_pair_df2(D1, D2, ne, e.lo, a[0], b[0], c[0]);
+  weno5_pair_df2(D2, D3, ne, e.lo, a[1], b[1], c[1]);
+  weno5_pair_df2(D3, D4, ne, e.lo, a[2], b[2], c[2]);
+  const DF2 G = weno5_combine6_df2(a[0], b[1], c[2], D1, D2, D3, D4);
+  return fma(df_join(lo_of(G.hi), lo_of(G.lo)), 1.0 / 6.0, m2);
 }
 
 }  // namespace rlbdev

@@ -58,7 +58,8 @@ struct TubeDev {
 //   then per velocity s = i Qxi + j the WENO5 epsilon terms 3 eps ws^2 (C0, C1, C2) at [3 s + 0..2],
 //   ws = w^p_i w^xi_j / 2 (the limiter acts on the weight-normalised population),
 //   then per velocity s the term e = 3 eps ws^2 as a float pair (hi, lo) in the 8 bytes of slot s (the FP64
-//   stage kernel's double-float limiter)
+//   stage kernel's double-float limiter),
+//   then xi_j^2 (Qxi)
 constexpr int TAB_PBAR = 0;
 constexpr int TAB_PBAR2 = QP_MAX;
 constexpr int TAB_WP = 2 * QP_MAX;
@@ -69,7 +70,8 @@ __host__ __device__ inline int tab_pw(int Qxi) { return TAB_XI + Qxi; }
 __host__ __device__ inline int tab_cxi(int Qxi) { return TAB_XI + Qxi + Qxi * (NV_MAX + 1); }
 __host__ __device__ inline int tab_eps(int Qxi) { return tab_cxi(Qxi) + 3 * Qxi; }
 __host__ __device__ inline int tab_epsf(int Qp, int Qxi) { return tab_eps(Qxi) + 3 * Qp * Qxi; }
-inline int tab_size(int Qp, int Qxi) { return tab_epsf(Qp, Qxi) + Qp * Qxi; }
+__host__ __device__ inline int tab_xi2(int Qp, int Qxi) { return tab_epsf(Qp, Qxi) + Qp * Qxi; }
+inline int tab_size(int Qp, int Qxi) { return tab_xi2(Qp, Qxi) + Qxi; }
 // Per-tube FP32 table of the reduced-precision path (floats, starting at TubeDev::tabf): one record of
 // RP_REC floats per velocity s = i Qxi + j, 16-byte aligned, read with vector loads:
 //   R_XI          xi_j

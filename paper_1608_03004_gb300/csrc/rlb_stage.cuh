@@ -7,9 +7,9 @@
 constexpr int NT = 256;                    // threads per CTA
 constexpr int GW = 64;                     // threads per velocity group (one row at a time)
 constexpr int NG = NT / GW;                // velocity rows processed together
-constexpr int TX = GW - 3;                 // cells per tile: their TX + 1 interfaces need GW indicator pairs
+constexpr int TX = GW - 4;                 // cells per tile: the stencils of their TX + 1 interfaces hold GW differences
 constexpr int HALO = 3;                    // WENO5 reaches three cells upwind/downwind
-constexpr int RW = TX + 2 * HALO;          // staged row length
+constexpr int RW = TX + 2 * HALO;          // staged cells x0 - 3 .. x0 + TX + 2
 constexpr int NBC = QP_MAX * (NV_MAX + 1); // per-cell equilibrium coefficients
 
 // Factors -k (k + 2) / ((2k + 1) (2k + 3)) of the backward recurrence of the Legendre coefficients
@@ -65,7 +65,7 @@ __device__ __forceinline__ void for_each_tile(int ntiles, int schedule, int* cou
 // Device helpers
 // --------------------------------------------------------------------------------------------------
 
-// Source of a staged position x in [-HALO, Nx - 1 + GW + HALO] within its row: periodic wrap (Nx >= 3),
+// Source of a staged position x in [-HALO, Nx - 1 + TX + HALO] within its row: periodic wrap (Nx >= 3),
 // zero-gradient ghosts (open boundary), or, on a halo side of a slab, the ghost cells the caller unpacked beside
 // the row (left ghosts -3..-1 at ld-3..ld-1, right ghosts at Nx..Nx+2; ld >= Nx + 6 for slabs; positions past
 // Nx + 2 are never read by a cell and map to Nx + 2). Always in [0, ld).
@@ -237,7 +237,7 @@ __device__ __forceinline__ void store_cell_coeffs(bool ok, double beta, double b
 }
 
 // Fill B[i (NVc+1) + k][c] (radial rows i < Qp) for the TX cells of a tile from cs.ge: group g builds radial row
-// i = g.
+// i = g. Coefficients of w^xi_j P_k(xi_j).
 template <int NPc, int NVc>
 __device__ __forceinline__ void build_rows(const double* tab, int Qp, const CoefSmem& cs, double (*Bs)[GW]) {
   const int c = threadIdx.x % GW, i = threadIdx.x / GW;
@@ -254,6 +254,24 @@ __device__ __forceinline__ void build_rows(const double* tab, int Qp, const Coef
   }
 }
 
+// Orders up to which the stage kernel evaluates the equilibrium as a polynomial in xi (two Horner chains in xi^2) from
+// monomial coefficients; above, from the Legendre ones (the change of basis loses digits as the order grows: its
+// entries reach 63/8 at order 5, 429/16 at 7).
+constexpr int NV_MONO = 5;
+
+// Legendre to monomial coefficients of one column, in place: B[k] of P_k becomes B[k] of xi^k.
+template <int NVc>
+__device__ __forceinline__ void legendre_to_monomial(double* B, int stride) {
+  static_assert(NVc == NV_MONO, "the table is for this order");
+  const double b0 = B[0], b1 = B[stride], b2 = B[2 * stride], b3 = B[3 * stride], b4 = B[4 * stride], b5 = B[5 * stride];
+  B[0] = fma(0.375, b4, fma(-0.5, b2, b0));
+  B[stride] = fma(1.875, b5, fma(-1.5, b3, b1));
+  B[2 * stride] = fma(-3.75, b4, 1.5 * b2);
+  B[3 * stride] = fma(-8.75, b5, 2.5 * b3);
+  B[4 * stride] = 4.375 * b4;
+  B[5 * stride] = 7.875 * b5;
+}
+
 // --------------------------------------------------------------------------------------------------
 // Stage kernel
 // --------------------------------------------------------------------------------------------------
@@ -268,23 +286,30 @@ struct StageSmem {
       CoefSmem coef;
     } a;                               // phases A and B
     struct {
-      double row[2][NG][RW + 1];  // staged velocity rows (double-buffered: written before the first barrier)
-      double d1[NG][RW + 1];      // first differences by position, d1[k] = row[k] - row[k-1]
-      float2 dd[NG][RW + 1];      // the same differences in double-float (hi, lo)
-      float2 sv[NG][3][GW];       // indicators v = S + e (double-float), one triple per pair of adjacent differences
-      float2 phi[NG][GW];         // WENO correction of each interface, times 6 (double-float)
-    } c;                          // phase C
+      double d1[NG][2][GW];         // first differences of a mirror pair's two rows, in wind order
+      float4 dd[NG][GW];            // the same in double-float: (hi, hi', lo, lo')
+      float4 sv[NG][2][GW];         // indicators v_B, v_C of each pair of adjacent differences (both rows)
+      float2 phi[NG][2][GW];        // WENO correction of each interface, times 6 (double-float), by row
+    } c;                            // phase C
   } u;
   double rate[2][GW];
-  int src[RW + 1];            // source cell of each staged position (boundary condition applied)
-  double B[NBC][GW];          // equilibrium coefficients B[i (NVc + 1) + k]; last, so that a launch allocates
-                              // only the rows its tubes use (stage_smem_bytes)
+  double cst[5];                    // 1, 1/6, the Runge-Kutta a, b, and -0, for register operands
+  int src[RW + 1];                  // source cell of each staged position (boundary condition applied)
+  double B[NBC][GW];                // equilibrium coefficients B[i (NVc + 1) + k]; last, so that a launch allocates
+                                    // only the rows its tubes use (stage_smem_bytes)
 };
 // Dynamic shared memory of the FP64 stage kernel for `brows` coefficient rows.
 constexpr size_t stage_smem_bytes(int brows) { return offsetof(StageSmem, B) + (size_t)brows * GW * sizeof(double); }
 
+// Operand forms. On GB300 an FP64 FMA whose three operands are all registers issues every 16 cycles per SM; an
+// addition, a multiplication, or an FMA with a constant-bank or immediate operand every 19 (measured). The hot loops
+// therefore add and multiply by FMAs with a register 1 or -0 (same rounding), and keep their constants in registers
+// that the compiler cannot fold (read from shared memory).
+__device__ __forceinline__ double add_r(double a, double b, double one) { return fma(a, one, b); }
+
 template <int NPc, int NVc>
 __device__ void stage_tile(const StageArgs& A, const TubeDev& T, int x0, int part, int nparts, StageSmem& sm) {
+  constexpr bool MONO = NVc <= NV_MONO;
   const int tid = threadIdx.x, c = tid % GW, g = tid / GW;
   const double* tab = A.tab + T.tab;
   const int Qp = T.Qp, Qxi = T.Qxi, Nx = T.Nx, ld = T.ld;
@@ -294,6 +319,14 @@ __device__ void stage_tile(const StageArgs& A, const TubeDev& T, int x0, int par
   const int x = x0 + c;
   const bool cell = (c < TX) && (x < Nx);
   for (int k = tid; k < RW; k += NT) sm.src[k] = map_cell(x0 - HALO + k, Nx, T.bc, ld);
+  if (tid == 0) {
+    sm.cst[0] = 1.0;
+    sm.cst[1] = 1.0 / 6.0;
+    sm.cst[2] = A.a;
+    sm.cst[3] = A.b;
+    sm.cst[4] = -0.0;
+  }
+  __syncthreads();
 
   if (T.collide) {
     // A. moments of the stage input. The groups split the mirror pairs of directions (xi_jf = -xi_jb > 0) and
@@ -306,17 +339,18 @@ __device__ void stage_tile(const StageArgs& A, const TubeDev& T, int x0, int par
 #pragma unroll
     for (int k = 0; k < 3 * QP_MAX; ++k) S[k] = 0.0;
     const int hq = Qxi / 2;
+    const double one = *const_cast<const volatile double*>(&sm.cst[0]);
     if (cell) {
       for (int jb = g; jb < hq; jb += NG) {
         const int jf = Qxi - 1 - jb;
-        const double xi = tab[TAB_XI + jf], xi2 = xi * xi;
+        const double xi = tab[TAB_XI + jf], xi2 = tab[tab_xi2(Qp, Qxi) + jf];
 #pragma unroll
         for (int i = 0; i < QP_MAX; ++i) {
           if (i < Qp) {
             const double ff = __ldg(Fin + (size_t)(i * Qxi + jf) * ld + x);
             const double fb = __ldg(Fin + (size_t)(i * Qxi + jb) * ld + x);
-            const double sum = ff + fb, dif = ff - fb;
-            S[3 * i] += sum;
+            const double sum = add_r(fb, ff, one), dif = fma(-fb, one, ff);
+            S[3 * i] = add_r(sum, S[3 * i], one);
             S[3 * i + 1] = fma(dif, xi, S[3 * i + 1]);
             S[3 * i + 2] = fma(sum, xi2, S[3 * i + 2]);
           }
@@ -366,130 +400,171 @@ __device__ void stage_tile(const StageArgs& A, const TubeDev& T, int x0, int par
     }
     __syncthreads();
     build_rows<NPc, NVc>(tab, Qp, sm.u.a.coef, sm.B);
+    if constexpr (MONO) {
+      if (c < TX && g < Qp) legendre_to_monomial<NVc>(&sm.B[g * (NVc + 1)][c], GW);
+    }
+    __syncthreads();  // the coefficients are ready, the union is free
   }
-  __syncthreads();  // sm.src (and, with collisions, the coefficients) are ready
 
-  // C. advection + collision + Runge-Kutta combination. The work unit of a 64-thread group is a mirror pair
-  //    of directions (j, Qxi - 1 - j) of one radial node, processed back to back: the nodes are symmetric, so
-  //    w^xi P_k(-xi) = (-1)^k w^xi P_k(xi) and the even and odd Legendre parts of F^eq, summed once, give both
-  //    rows' equilibria (the xi = 0 node of an odd Qxi is a unit of its own). Groups synchronise with named
-  //    barriers only.
-  const double a = A.a, b = A.b;
+  // C. advection + collision + Runge-Kutta combination. The work unit of a 64-thread group is a mirror pair of
+  //    directions (j, Qxi - 1 - j) of one radial node, both rows at once: the row with the wind toward -x is held in
+  //    reversed order, so that every step of the limiter is the same packed operation on both rows. The even and odd
+  //    parts of the equilibrium in xi, summed once, give both rows' equilibria. The xi = 0 node of an odd Qxi is a
+  //    unit of its own. Groups synchronise with named barriers only, three per unit.
   const double* cxi_tab = tab + tab_cxi(Qxi) + A.stage * Qxi;
-  double* d1 = sm.u.c.d1[g];
-  float2* dd = sm.u.c.dd[g];
-  float2* sv0 = sm.u.c.sv[g][0];
-  float2* sv1 = sm.u.c.sv[g][1];
-  float2* sv2 = sm.u.c.sv[g][2];
-  float2* phi = sm.u.c.phi[g];
+  double* d1f = sm.u.c.d1[g][0];
+  double* d1r = sm.u.c.d1[g][1];
+  float4* dd = sm.u.c.dd[g];
+  float4* svb = sm.u.c.sv[g][0];
+  float4* svc = sm.u.c.sv[g][1];
+  float2* phf = sm.u.c.phi[g][0];
+  float2* phr = sm.u.c.phi[g][1];
+  const volatile double* cst = sm.cst;
   const float2* epsf = reinterpret_cast<const float2*>(tab + tab_epsf(Qp, Qxi));
   const int hq = Qxi / 2, upr = hq + (Qxi & 1), U = Qp * upr;
   const int u_end = (part + 1) * U / nparts;
-  int buf = 0;
-  for (int u0 = part * U / nparts; u0 < u_end; u0 += NG) {
-    const int u = u0 + g;
-    if (u >= u_end) continue;  // uniform over the group
-    const int i = u / upr, jA = u - i * upr;  // jA = hq: the xi = 0 node
-    const int nrow = jA < hq ? 2 : 1;
-    double E = 0.0, O = 0.0;  // even and odd parts of sum_k B[i][k] w^xi P_k(xi_jA) at this cell
-    for (int h = 0; h < nrow; ++h, buf ^= 1) {
-      const int j = h == 0 ? jA : Qxi - 1 - jA;
-      const int s = i * Qxi + j;
-      double* row = sm.u.c.row[buf][g];
-      // stage the row with its first differences, in FP64 and split into double-float (position k needs k - 1
-      // as well)
-      {
-        const double* src = Fin + (size_t)s * ld;
-        // positions 0 .. GW-1, one per thread: the previous position's value comes from the lane below by a
-        // shuffle (the first lane of each warp loads it)
-        {
-          const double v = __ldg(src + sm.src[c]);
-          row[c] = v;
-          const double below = __shfl_up_sync(0xffffffffu, v, 1);
-          if (c > 0) {
-            const double dk = v - ((c & 31) == 0 ? __ldg(src + sm.src[c - 1]) : below);
-            d1[c] = dk;
-            const rlbdev::DF q = rlbdev::df_split(dk);
-            dd[c] = make_float2(q.hi, q.lo);
-          }
-        }
-        for (int k = c + GW; k < RW; k += GW) {
-          const double v = __ldg(src + sm.src[k]);
-          row[k] = v;
-          const double dk = v - __ldg(src + sm.src[k - 1]);
-          d1[k] = dk;
-          const rlbdev::DF q = rlbdev::df_split(dk);
-          dd[k] = make_float2(q.hi, q.lo);
-        }
-      }
-      // the Runge-Kutta input of this row's cell, loaded now so that its latency hides behind the limiter
-      const double fnv = (A.stage != 0 && cell) ? __ldg(Fn + (size_t)s * ld + x) : 0.0;
-      group_sync(g);
-      const double xi = tab[TAB_XI + j];
-      const bool fwd = h == 1;  // the mirror row xi_{Qxi-1-jA} > 0; the first row has xi <= 0
-      // pairs: thread c owns the pair of differences at positions (p, p + 1), p = c + 1 (wind toward +x) or
-      // c + 2 (toward -x); these are the pairs the TX + 1 interfaces of the tile use
-      {
-        const int p = c + (fwd ? 1 : 2);
-        const float2 e = epsf[s], x = dd[p], y = dd[p + 1];
-        rlbdev::DF va, vb, vc;
-        rlbdev::weno5_pair_df({x.x, x.y}, {y.x, y.y}, fwd, {e.x, e.y}, va, vb, vc);
-        sv0[c] = make_float2(va.hi, va.lo);
-        sv1[c] = make_float2(vb.hi, vb.lo);
-        sv2[c] = make_float2(vc.hi, vc.lo);
-      }
-      group_sync(g);
-      // interfaces: interface c lies between cells x0 + c - 1 and x0 + c (row index c + 2 | c + 3); its value
-      // is v2 + G with v2 the upwind cell; D = v2(c + 1) - v2(c) is the memory-order difference d1[c + 3]
-      // (wind toward +x) or d1[c + 4] (toward -x)
-      double D = 0.0;
-      if (c <= TX) {
-        auto get = [](const float2* a, int k) { const float2 q = a[k]; return rlbdev::DF{q.x, q.y}; };
-        auto neg = [&](int k) { const float2 q = dd[k]; return rlbdev::DF{-q.x, -q.y}; };
-        rlbdev::DF G;
-        if (fwd) {
-          D = d1[c + 3];
-          G = rlbdev::weno5_combine6_df(get(sv0, c), get(sv1, c + 1), get(sv2, c + 2), get(dd, c + 1),
-                                        get(dd, c + 2), get(dd, c + 3), get(dd, c + 4));
+  auto up = [](float4 q) { return rlbdev::DF2{rlbdev::f2(q.x, q.y), rlbdev::f2(q.z, q.w)}; };
+  auto down = [](rlbdev::DF2 q) {
+    return make_float4(rlbdev::lo_of(q.hi), rlbdev::hi_of(q.hi), rlbdev::lo_of(q.lo), rlbdev::hi_of(q.lo));
+  };
+  for (int u = part * U / nparts + g; u < u_end; u += NG) {
+    const int i = u / upr, jb = u - i * upr;
+    if (jb == hq) {  // the xi = 0 node: no advection
+      if (!cell) continue;
+      const size_t o = (size_t)(i * Qxi + hq) * ld + x;
+      const double F = __ldg(Fin + o);
+      double out = A.stage != 0 ? fma(A.a, __ldg(Fn + o), A.b * F) : F;
+      if (T.collide) {
+        const double* pw = tab + TAB_XI + Qxi + hq * (NV_MAX + 1);
+        double E;
+        if constexpr (MONO) {
+          E = sm.B[i * (NVc + 1)][c] * pw[0];
         } else {
-          D = d1[c + 4];
-          G = rlbdev::weno5_combine6_df(get(sv0, c + 2), get(sv1, c + 1), get(sv2, c), neg(c + 5), neg(c + 4),
-                                        neg(c + 3), neg(c + 2));
-        }
-        phi[c] = make_float2(G.hi, G.lo);
-      }
-      group_sync(g);
-      if (cell) {
-        const double F = row[c + 3];
-        // phi holds 6 G: D + (6 G_{x+1/2} - 6 G_{x-1/2}) / 6, the difference taken in double-float
-        const float2 pr = phi[c + 1], pl = phi[c];
-        const rlbdev::DF dG = rlbdev::df_plus({pr.x, pr.y}, {-pl.x, -pl.y});
-        const double dphi = fma(rlbdev::df_widen(dG.hi), 1.0 / 6.0, fma(rlbdev::df_widen(dG.lo), 1.0 / 6.0, D));
-        double out = F;
-        if (A.stage != 0) out = fma(a, fnv, b * F);  // a = 0 in the first stage
-        out = fma(-cxi_tab[j], dphi, out);  // - b dt xi/dx (Phi_{x+1/2} - Phi_{x-1/2})
-        if (T.collide) {
-          if (h == 0) {
-            const double* pw = tab + TAB_XI + Qxi + jA * (NV_MAX + 1);
+          E = 0.0;
 #pragma unroll
-            for (int k = 0; k <= NVc; ++k) {
-              const double t = sm.B[i * (NVc + 1) + k][c];
-              if (k % 2 == 0)
-                E = fma(t, pw[k], E);
-              else
-                O = fma(t, pw[k], O);
-            }
-          }
-          const double feq = h == 0 ? E + O : E - O;
-          const double rate = fma(-sm.rate[1][c], xi, sm.rate[0][c]);
-          out = fma(rate, feq - F, out);  // + b dt gamma (1 - beta xi)/tau (F^eq - F)
+          for (int k = 0; k <= NVc; k += 2) E = fma(sm.B[i * (NVc + 1) + k][c], pw[k], E);
         }
-        Fout[(size_t)s * ld + x] = out;
+        out = fma(sm.rate[0][c], E - F, out);
       }
+      Fout[o] = out;
+      continue;
+    }
+    const int jf = Qxi - 1 - jb, sf = i * Qxi + jf, sb = i * Qxi + jb;
+    // stage both rows as first differences in wind order, in FP64 and split into double-float: difference k lies
+    // between positions k and k + 1, position p = cell x0 - 3 + p, or x0 + TX + 2 - p in the reversed row. Each lane
+    // loads position c + 1; position c comes from the lane below (the first lane of each warp loads it)
+    rlbdev::DF2 e1;
+    {
+      const double* rf = Fin + (size_t)sf * ld;
+      const double* rb = Fin + (size_t)sb * ld;
+      const double vf = __ldg(rf + sm.src[c + 1]), vr = __ldg(rb + sm.src[RW - 2 - c]);
+      double pf = __shfl_up_sync(0xffffffffu, vf, 1), pr = __shfl_up_sync(0xffffffffu, vr, 1);
+      if ((c & 31) == 0) {
+        pf = __ldg(rf + sm.src[c]);
+        pr = __ldg(rb + sm.src[RW - 1 - c]);
+      }
+      const double one = cst[0];
+      const double df = fma(-pf, one, vf), dr = fma(-pr, one, vr);
+      d1f[c] = df;
+      d1r[c] = dr;
+      const rlbdev::DF qf = rlbdev::df_split(df), qr = rlbdev::df_split(dr);
+      dd[c] = make_float4(qf.hi, qr.hi, qf.lo, qr.lo);
+      e1 = {rlbdev::f2(qf.hi, qr.hi), rlbdev::f2(qf.lo, qr.lo)};
+    }
+    // the cell's own values and Runge-Kutta inputs, loaded now so that their latency hides behind the limiter
+    double Ff = 0.0, Fb = 0.0, nf = 0.0, nb = 0.0;
+    if (cell) {
+      Ff = __ldg(Fin + (size_t)sf * ld + x);
+      Fb = __ldg(Fin + (size_t)sb * ld + x);
+      if (A.stage != 0) {
+        nf = __ldg(Fn + (size_t)sf * ld + x);
+        nb = __ldg(Fn + (size_t)sb * ld + x);
+      }
+    }
+    const float2 ee = epsf[sf];
+    group_sync(g);
+    // pairs: lane c owns the pair of differences (c, c + 1)
+    const int c1 = min(c + 1, GW - 1);
+    const rlbdev::DF2 e2 = up(dd[c1]);
+    rlbdev::DF2 vA, vB, vC;
+    rlbdev::weno5_pair_df2(e1, e2, rlbdev::f2(-ee.x), rlbdev::f2(ee.y), vA, vB, vC);
+    svb[c] = down(vB);
+    svc[c] = down(vC);
+    group_sync(g);
+    // interfaces: lane c owns interface c (between cells x0 + c - 1 and x0 + c, or x0 + TX - c and x0 + TX - 1 - c in
+    // the reversed row); its stencils' differences are c .. c + 3
+    double Df = 0.0, Dr = 0.0;
+    rlbdev::DF2 G = {rlbdev::f2(0.0f), rlbdev::f2(0.0f)};
+    if (c <= TX) {
+      G = rlbdev::weno5_combine6_df2(vA, up(svb[c + 1]), up(svc[c + 2]), e1, e2, up(dd[c + 2]), up(dd[c + 3]));
+      phf[c] = make_float2(rlbdev::lo_of(G.hi), rlbdev::lo_of(G.lo));
+      phr[c] = make_float2(rlbdev::hi_of(G.hi), rlbdev::hi_of(G.lo));
+      if (c < TX) {
+        Df = d1f[c + 2];
+        Dr = d1r[TX + 1 - c];
+      }
+    }
+    group_sync(g);
+    if (cell) {
+      // flux differences: D + (6 G - 6 G') / 6, the difference of the corrections taken in double-float. The cell is
+      // number c of its row and number TX - 1 - c of the reversed one
+      const float2 g1f = phf[c + 1], g1r = phr[TX - c], g0r = phr[TX - 1 - c];
+      const rlbdev::DF2 dG =
+          rlbdev::df2_minus({rlbdev::f2(g1f.x, g1r.x), rlbdev::f2(g1f.y, g1r.y)},
+                            {rlbdev::f2(rlbdev::lo_of(G.hi), g0r.x), rlbdev::f2(rlbdev::lo_of(G.lo), g0r.y)});
+      const double sixth = cst[1], cxi = cxi_tab[jf];
+      const double phi_f = fma(rlbdev::df_join(rlbdev::lo_of(dG.hi), rlbdev::lo_of(dG.lo)), sixth, Df);
+      const double phi_b = fma(rlbdev::df_join(rlbdev::hi_of(dG.hi), rlbdev::hi_of(dG.lo)), sixth, Dr);
+      double of = Ff, ob = Fb;
+      if (A.stage != 0) {  // a = 0 and b = 1 in the first stage
+        const double a = cst[2], b = cst[3], zero = cst[4];
+        of = fma(a, nf, fma(b, Ff, zero));
+        ob = fma(a, nb, fma(b, Fb, zero));
+      }
+      of = fma(-cxi, phi_f, of);  // - b dt |xi|/dx (Phi - Phi'), along each row's wind
+      ob = fma(-cxi, phi_b, ob);
+      if (T.collide) {
+        const double xi = tab[TAB_XI + jf];
+        const double* pw = tab + TAB_XI + Qxi + jf * (NV_MAX + 1);
+        const double(*Bi)[GW] = &sm.B[i * (NVc + 1)];
+        double cf, cb;  // F^eq - F
+        if constexpr (MONO) {
+          const double z = tab[tab_xi2(Qp, Qxi) + jf], w = pw[0];
+          double E = Bi[NVc - NVc % 2][c], O = Bi[NVc - 1 + NVc % 2][c];
+#pragma unroll
+          for (int k = NVc - NVc % 2 - 2; k >= 0; k -= 2) E = fma(E, z, Bi[k][c]);
+#pragma unroll
+          for (int k = NVc - 3 + NVc % 2; k >= 1; k -= 2) O = fma(O, z, Bi[k][c]);
+          cf = fma(w, fma(xi, O, E), -Ff);
+          cb = fma(w, fma(-xi, O, E), -Fb);
+        } else {
+          double E = 0.0, O = 0.0;
+#pragma unroll
+          for (int k = 0; k <= NVc; ++k) {
+            if (k % 2 == 0)
+              E = fma(Bi[k][c], pw[k], E);
+            else
+              O = fma(Bi[k][c], pw[k], O);
+          }
+          cf = (E + O) - Ff;
+          cb = (E - O) - Fb;
+        }
+        const double r0 = sm.rate[0][c], r1 = sm.rate[1][c];
+        of = fma(fma(-r1, xi, r0), cf, of);  // + b dt gamma (1 - beta xi)/tau (F^eq - F)
+        ob = fma(fma(r1, xi, r0), cb, ob);
+      }
+      Fout[(size_t)sf * ld + x] = of;
+      Fout[(size_t)sb * ld + x] = ob;
     }
   }
 }
 
+// What bounds it: the FP64 pipe (88 % busy on the stress tube, 14.3 FP64 operations per node, 35 % of the issue
+// slots). Measured on GB300, FP64 stress tube (2^20 cells x 384 velocities, half of it moving), ms per step: 46.0 with
+// one row at a time in scalar double-float and Legendre-basis equilibria, 37.1 with both rows of a mirror pair packed,
+// register operands and Horner equilibria, 34.8 once no conversion instruction was left in the rows (df_split,
+// df_join). The relaxation-time sweep: 3.62, 2.89, 2.67. 80 registers for 3 CTAs per SM: two CTAs with 128 registers ran
+// 8 % slower on the stress tube, four with 64 registers 1 % faster there and 3 % slower on the sweep.
 // SCHED is the launch's schedule (compile time, so that the one-CTA-per-tile kernel carries no tile loop).
 template <int SCHED>
 __global__ void __launch_bounds__(NT, 3) rlb_stage_kernel(StageArgs A) {
