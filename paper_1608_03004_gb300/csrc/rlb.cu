@@ -41,8 +41,6 @@
 #include "rlb_internal.h"
 
 using namespace rlb;
-using rlbdev::weno5_combine;
-using rlbdev::weno5_pair;
 
 namespace {
 

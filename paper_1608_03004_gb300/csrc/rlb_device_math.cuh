@@ -99,20 +99,6 @@ __device__ __forceinline__ void weno5_pair(T x, T y, bool fwd, T eA, T eB, T eC,
   sC = mul_x(uC, uC);
 }
 
-// weno5_pair from the products x^2, x y, y^2 (the FP64 kernel forms each difference's square once and shares
-// it between the two pairs the difference belongs to).
-template <typename T>
-__device__ __forceinline__ void weno5_pair_q(T qx, T pxy, T qy, bool fwd, T eA, T eB, T eC, T& sA, T& sB, T& sC) {
-  const T ax = fwd ? T(4.0 * C0) : T(10.0 * C0), ay = fwd ? T(10.0 * C0) : T(4.0 * C0);
-  const T cx = fwd ? T(10.0 * C2) : T(4.0 * C2), cy = fwd ? T(4.0 * C2) : T(10.0 * C2);
-  const T uA = fma(ax, qx, fma(T(-11.0 * C0), pxy, fma(ay, qy, eA)));
-  const T uB = fma(T(4.0 * C1), qx, fma(T(-5.0 * C1), pxy, fma(T(4.0 * C1), qy, eB)));
-  const T uC = fma(cx, qx, fma(T(-11.0 * C2), pxy, fma(cy, qy, eC)));
-  sA = uA * uA;
-  sB = uB * uB;
-  sC = uC * uC;
-}
-
 // 6 G of the interface from the three scaled squares (s0, s1, s2) of its stencils and the differences
 // d1..d4 in wind order (the FP64 stage kernel applies the 1/6 in the flux difference, where it costs nothing).
 template <typename T>
@@ -194,7 +180,7 @@ __device__ __forceinline__ void df_add(DF& acc, DF a) {
 
 // ---------------------------------------------------------------------------------------------------------
 // Packed FP32 arithmetic: two floats in a 64-bit register pair, one instruction per operation on both
-// (fma/add/sub/mul.rn.f32x2: each half rounded as the scalar operation rounds it, never contracted). On GB300 a
+// (fma/add/sub/mul.rn.f32x2: each half rounded as the scalar operation rounds it). On GB300 a
 // packed operation occupies the FP32 pipe like two scalar ones (1.94 of them per SM and clock, measured, against 3.9
 // scalar) but takes one issue slot instead of two.
 struct F2 {
@@ -229,6 +215,14 @@ __device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
   return r;
 }
 __device__ __forceinline__ F2 neg2(F2 a) { return {a.v ^ 0x8000000080000000ull}; }
+
+// ptxas fuses a packed product into a following packed sum (measured, with .rn written and with contraction switched
+// off), which would round an interface value differently in different inlined copies and break the error-free
+// transformations. A product that feeds a sum is therefore taken as a b + (-0) with a -0 that the compiler does not
+// know: minus_zero2() reads it from memory once per kernel.
+static __device__ unsigned long long g_minus_zero2 = 0x8000000080000000ull;
+__device__ __forceinline__ F2 minus_zero2() { return {*const_cast<const volatile unsigned long long*>(&g_minus_zero2)}; }
+__device__ __forceinline__ F2 mulx2(F2 a, F2 b, F2 nz) { return fma2(a, b, nz); }
 
 // Two double-floats, one in each half.
 struct DF2 {
@@ -304,8 +298,8 @@ __device__ __forceinline__ DF2 df2_plus_pos(DF2 a, DF2 b) {
 __device__ __forceinline__ DF2 df2_pow2(DF2 a, F2 p) { return {mul2(a.hi, p), mul2(a.lo, p)}; }
 
 // a * b, with -a.hi given
-__device__ __forceinline__ DF2 df2_times(DF2 a, F2 na, DF2 b) {
-  const F2 np = mul2(na, b.hi);
+__device__ __forceinline__ DF2 df2_times(DF2 a, F2 na, DF2 b, F2 nz) {
+  const F2 np = mulx2(na, b.hi, nz);
   return fast_two_sum_n(np, fma2(a.hi, b.lo, fma2(a.lo, b.hi, fma2(a.hi, b.hi, np))));
 }
 
@@ -361,7 +355,8 @@ __device__ __forceinline__ double df_join(float hi, float lo) {
 
 // Indicators v_A, v_B, v_C of the pairs (x, y) = (d_j, d_{j+1}) in wind order, e the epsilon term:
 // (v_A, v_B, v_C) = (SL, SC, SR)(x, y) + e.
-__device__ __forceinline__ void weno5_pair_df2(DF2 x, DF2 y, F2 ne_hi, F2 e_lo, DF2& vA, DF2& vB, DF2& vC) {
+__device__ __forceinline__ void weno5_pair_df2(DF2 x, DF2 y, F2 ne_hi, F2 e_lo, F2 nz, DF2& vA,
+                                               DF2& vB, DF2& vC) {
   // -x^2, -x y, -y^2 rounded (the high parts), their errors plus the cross terms (the low parts)
   const F2 nx = neg2(x.hi), ny = neg2(y.hi);
   const F2 X = mul2(nx, x.hi), Y = mul2(ny, y.hi), Z = mul2(nx, y.hi);
@@ -370,12 +365,12 @@ __device__ __forceinline__ void weno5_pair_df2(DF2 x, DF2 y, F2 ne_hi, F2 e_lo, 
   const F2 Zl = fma2(x.hi, y.lo, fma2(x.lo, y.hi, fma2(x.hi, y.hi, Z)));
   const F2 c4 = f2(4.0f), c5 = f2(5.0f), c10 = f2(10.0f), c11 = f2(11.0f);
   const F2 m5 = f2(-5.0f), m10 = f2(-10.0f), m11 = f2(-11.0f);
-  // the integer multiples, high parts negated
+  // the integer multiples, high parts negated (those by 4 are exact, fused or not)
   const F2 X4 = mul2(X, c4), Y4 = mul2(Y, c4), X4l = mul2(Xl, c4), Y4l = mul2(Yl, c4);
-  const F2 X10 = mul2(X, c10), X10l = fma2(Xl, c10, fma2(X, m10, X10));
-  const F2 Y10 = mul2(Y, c10), Y10l = fma2(Yl, c10, fma2(Y, m10, Y10));
-  const F2 Z11 = mul2(Z, m11), Z11l = fma2(Zl, m11, fma2(Z, c11, Z11));
-  const F2 Z5 = mul2(Z, m5), Z5l = fma2(Zl, m5, fma2(Z, c5, Z5));
+  const F2 X10 = mulx2(X, c10, nz), X10l = fma2(Xl, c10, fma2(X, m10, X10));
+  const F2 Y10 = mulx2(Y, c10, nz), Y10l = fma2(Yl, c10, fma2(Y, m10, Y10));
+  const F2 Z11 = mulx2(Z, m11, nz), Z11l = fma2(Zl, m11, fma2(Z, c11, Z11));
+  const F2 Z5 = mulx2(Z, m5, nz), Z5l = fma2(Zl, m5, fma2(Z, c5, Z5));
   // (a, b, c) + e: exact sums of the (negated) high parts, then the low parts and the errors; v > 0 is a positive
   // definite form plus e, so the final FastTwoSum's ordering holds
   auto sum3 = [&](F2 a, F2 al, F2 b, F2 bl, F2 c, F2 cl) {
@@ -397,29 +392,30 @@ __device__ __forceinline__ float weno5_scale(float v0, float v1, float v2) {
 }
 
 // 6 G of two interfaces from the indicators (v0, v1, v2) of their stencils and the differences d1..d4 in wind order.
-__device__ __forceinline__ DF2 weno5_combine6_df2(DF2 v0, DF2 v1, DF2 v2, DF2 d1, DF2 d2, DF2 d3, DF2 d4) {
+__device__ __forceinline__ DF2 weno5_combine6_df2(DF2 v0, DF2 v1, DF2 v2, DF2 d1, DF2 d2, DF2 d3, DF2 d4,
+                                                   F2 nz) {
   const F2 sc = f2(weno5_scale(lo_of(v0.hi), lo_of(v1.hi), lo_of(v2.hi)),
                    weno5_scale(hi_of(v0.hi), hi_of(v1.hi), hi_of(v2.hi)));
   const F2 nsc = neg2(sc);
   auto square = [&](DF2 v) {
-    const F2 h = mul2(v.hi, sc), nh = mul2(v.hi, nsc), l = mul2(v.lo, sc), np = mul2(nh, h);
+    const F2 h = mul2(v.hi, sc), nh = mul2(v.hi, nsc), l = mul2(v.lo, sc), np = mulx2(nh, h, nz);
     return fast_two_sum_n(np, fma2(add2(h, h), l, fma2(h, h, np)));
   };
   const DF2 t0 = square(v0), t1 = square(v1), t2 = square(v2);
   // r0 = 5 d2 - 2 d1, r1 = d2 + 2 d3, r2 = 4 d3 - d4 (6 times the candidates' corrections)
   const F2 c2 = f2(2.0f), c3 = f2(3.0f), c4 = f2(4.0f), c5 = f2(5.0f), m5 = f2(-5.0f);
-  const F2 n5 = mul2(d2.hi, m5);
+  const F2 n5 = mulx2(d2.hi, m5, nz);
   const DF2 r0 = df2_minus({neg2(n5), fma2(d2.lo, c5, fma2(d2.hi, c5, n5))}, df2_pow2(d1, c2));
   const DF2 r1 = df2_plus(d2, df2_pow2(d3, c2));
   const DF2 r2 = df2_minus(df2_pow2(d3, c4), d4);
   const F2 nt1 = neg2(t1.hi), nt2 = neg2(t2.hi);
-  const DF2 a0 = df2_times(t1, nt1, t2);
-  const F2 n3 = mul2(t0.hi, f2(-3.0f));
+  const DF2 a0 = df2_times(t1, nt1, t2, nz);
+  const F2 n3 = mulx2(t0.hi, f2(-3.0f), nz);
   const DF2 t03 = fast_two_sum_n(n3, fma2(t0.lo, c3, fma2(t0.hi, c3, n3)));
   const F2 nt03 = neg2(t03.hi);
-  const DF2 num = df2_plus(df2_times(a0, neg2(a0.hi), r0),
-                           df2_times(t03, nt03, df2_plus(df2_pow2(df2_times(t2, nt2, r1), c2), df2_times(t1, nt1, r2))));
-  const DF2 den = df2_plus_pos(a0, df2_times(t03, nt03, df2_plus_pos(df2_pow2(t2, c2), t1)));
+  const DF2 p0 = df2_times(a0, neg2(a0.hi), r0, nz), p1 = df2_times(t2, nt2, r1, nz), p2 = df2_times(t1, nt1, r2, nz);
+  const DF2 num = df2_plus(p0, df2_times(t03, nt03, df2_plus(df2_pow2(p1, c2), p2), nz));
+  const DF2 den = df2_plus_pos(a0, df2_times(t03, nt03, df2_plus_pos(df2_pow2(t2, c2), t1), nz));
   // num / den: a quotient from FP32's reciprocal (approximation refined by one Newton-Raphson step to about
   // half an ulp), then one correction from the remainder
   float ra, rb;
@@ -428,11 +424,11 @@ __device__ __forceinline__ DF2 weno5_combine6_df2(DF2 v0, DF2 v1, DF2 v2, DF2 d1
   F2 rc = f2(ra, rb);
   const F2 nden = neg2(den.hi);
   rc = fma2(rc, fma2(nden, rc, f2(1.0f)), rc);
-  const F2 q1 = mul2(num.hi, rc), np = mul2(q1, nden);
+  const F2 q1 = mulx2(num.hi, rc, nz), np = mulx2(q1, nden, nz);
   const F2 pe = fma2(q1, den.lo, fma2(q1, den.hi, np));
   const F2 rem = add2(add2(num.hi, np), sub2(num.lo, pe));
   DF2 G;
-  two_sum2(q1, mul2(rem, rc), G.hi, G.lo);
+  two_sum2(q1, mulx2(rem, rc, nz), G.hi, G.lo);
   // all but one t below FP32's range (indicator ratios beyond ~1e19): that stencil's value
   const float da = lo_of(den.hi), db = hi_of(den.hi);
   if (da == 0.0f || db == 0.0f) {
@@ -464,12 +460,12 @@ __device__ __forceinline__ double weno5_interface_df(double m0, double m1, doubl
   const DF2 D1 = both(df_split(v1 - v0)), D2 = both(df_split(m2 - v1)), D3 = both(df_split(v3 - m2)),
             D4 = both(df_split(v4 - v3));
   const DF2 e = both(df_split(3.0 * eps));
-  const F2 ne = neg2(e.hi);
+  const F2 ne = neg2(e.hi), nz = minus_zero2();
   DF2 a[3], b[3], c[3];
-  weno5_pair_df2(D1, D2, ne, e.lo, a[0], b[0], c[0]);
-  weno5_pair_df2(D2, D3, ne, e.lo, a[1], b[1], c[1]);
-  weno5_pair_df2(D3, D4, ne, e.lo, a[2], b[2], c[2]);
-  const DF2 G = weno5_combine6_df2(a[0], b[1], c[2], D1, D2, D3, D4);
+  weno5_pair_df2(D1, D2, ne, e.lo, nz, a[0], b[0], c[0]);
+  weno5_pair_df2(D2, D3, ne, e.lo, nz, a[1], b[1], c[1]);
+  weno5_pair_df2(D3, D4, ne, e.lo, nz, a[2], b[2], c[2]);
+  const DF2 G = weno5_combine6_df2(a[0], b[1], c[2], D1, D2, D3, D4, nz);
   return fma(df_join(lo_of(G.hi), lo_of(G.lo)), 1.0 / 6.0, m2);
 }
 

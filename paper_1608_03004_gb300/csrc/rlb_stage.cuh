@@ -420,6 +420,7 @@ __device__ void stage_tile(const StageArgs& A, const TubeDev& T, int x0, int par
   float2* phf = sm.u.c.phi[g][0];
   float2* phr = sm.u.c.phi[g][1];
   const volatile double* cst = sm.cst;
+  const rlbdev::F2 nz = rlbdev::minus_zero2();
   const float2* epsf = reinterpret_cast<const float2*>(tab + tab_epsf(Qp, Qxi));
   const int hq = Qxi / 2, upr = hq + (Qxi & 1), U = Qp * upr;
   const int u_end = (part + 1) * U / nparts;
@@ -487,7 +488,7 @@ __device__ void stage_tile(const StageArgs& A, const TubeDev& T, int x0, int par
     const int c1 = min(c + 1, GW - 1);
     const rlbdev::DF2 e2 = up(dd[c1]);
     rlbdev::DF2 vA, vB, vC;
-    rlbdev::weno5_pair_df2(e1, e2, rlbdev::f2(-ee.x), rlbdev::f2(ee.y), vA, vB, vC);
+    rlbdev::weno5_pair_df2(e1, e2, rlbdev::f2(-ee.x), rlbdev::f2(ee.y), nz, vA, vB, vC);
     svb[c] = down(vB);
     svc[c] = down(vC);
     group_sync(g);
@@ -496,7 +497,8 @@ __device__ void stage_tile(const StageArgs& A, const TubeDev& T, int x0, int par
     double Df = 0.0, Dr = 0.0;
     rlbdev::DF2 G = {rlbdev::f2(0.0f), rlbdev::f2(0.0f)};
     if (c <= TX) {
-      G = rlbdev::weno5_combine6_df2(vA, up(svb[c + 1]), up(svc[c + 2]), e1, e2, up(dd[c + 2]), up(dd[c + 3]));
+      G = rlbdev::weno5_combine6_df2(vA, up(svb[c + 1]), up(svc[c + 2]), e1, e2, up(dd[c + 2]), up(dd[c + 3]),
+                                     nz);
       phf[c] = make_float2(rlbdev::lo_of(G.hi), rlbdev::lo_of(G.lo));
       phr[c] = make_float2(rlbdev::hi_of(G.hi), rlbdev::hi_of(G.lo));
       if (c < TX) {
