@@ -301,6 +301,8 @@ rlb_status ensure_series_tables(int dev) {
   }
   RLB_CUDA(cudaFuncSetAttribute((const void*)rlb_adjoint_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)sizeof(AdjSmem)));
+  RLB_CUDA(cudaFuncSetAttribute((const void*)rlb_adjoint_cell_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)sizeof(AdjCellSmem)));
   RLB_CUDA(cudaFuncSetAttribute((const void*)rlb_init_vjp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)sizeof(InitVjpSmem)));
   g_tables_ready[dev] = true;
@@ -355,9 +357,12 @@ struct rlb_ctx {
   double* seg = nullptr;
   long long seg_cap = 0;       // states allocated
   double* adj = nullptr;       // 4 states: adjoints of F^(n+1) / F^n, F^(1), F^(2) and the F^n accumulator
-  int2* d_atiles = nullptr;
-  std::vector<int> atile_tube;
-  double* d_dlt = nullptr;     // per adjoint tile: dL/dlog(tau)
+  int2* d_atiles = nullptr;    // adjoint tiles of TXA cells
+  int2* d_ctiles = nullptr;    // tiles of PC cells of the per-cell kernel
+  int natiles = 0;
+  std::vector<int> ctile_tube;
+  double* d_cellv = nullptr;   // [NCELLV][nxtot]: what the per-cell kernel leaves for the row kernel
+  double* d_dlt = nullptr;     // per PC-cell tile: dL/dlog(tau)
   // slabs of a decomposed tube: their exchange blocks (tube, sides, offset in the buffer)
   std::vector<HaloDesc> halo;
   HaloDesc* d_halo = nullptr;
@@ -387,6 +392,8 @@ void free_ctx(rlb_ctx* h) {
   cudaFree(h->seg);
   cudaFree(h->adj);
   cudaFree(h->d_atiles);
+  cudaFree(h->d_ctiles);
+  cudaFree(h->d_cellv);
   cudaFree(h->d_dlt);
   cudaFree(h->d_halo);
   cudaFree(h->d_tubes);
@@ -407,18 +414,15 @@ void free_ctx(rlb_ctx* h) {
   delete h;
 }
 
-// WENO5 epsilon terms of every velocity: 3 eps ws^2 (C0, C1, C2) into out, ws = w^p_i w^xi_j / 2 (the limiter
-// acts on the weight-normalised population F_s / ws with eps = 1e-6), and e = 3 eps ws^2 as the float pair
-// (hi, lo), hi + lo = e to about 48 bits, into the 8 bytes of outf[s].
+// WENO5 epsilon term of every velocity, e = 3 eps ws^2, ws = w^p_i w^xi_j / 2 (the limiter acts on the
+// weight-normalised population F_s / ws with eps = 1e-6), into out[s], and as the float pair (hi, lo), hi + lo = e to
+// about 48 bits, into the 8 bytes of outf[s].
 void fill_eps(double* out, double* outf, int Qp, int Qxi, const double* wp, const double* wxi) {
   for (int i = 0; i < Qp; ++i)
     for (int j = 0; j < Qxi; ++j) {
       const double ws = 0.5 * wp[i] * wxi[j];
       const double e = 3.0 * rlbdev::WENO_EPS * ws * ws;
-      double* o = out + 3 * (i * Qxi + j);
-      o[0] = e * rlbdev::C0;
-      o[1] = e * rlbdev::C1;
-      o[2] = e * rlbdev::C2;
+      out[i * Qxi + j] = e;
       const float pair[2] = {(float)e, (float)(e - (double)(float)e)};
       std::memcpy(outf + i * Qxi + j, pair, sizeof(pair));
     }
@@ -1391,10 +1395,13 @@ rlb_status launch_adjoint(rlb_ctx* h, int st, int mode, const double* Fin, const
   AdjArgs A{};
   A.tubes = h->d_tubes;
   A.tiles = h->d_atiles;
+  A.ctiles = h->d_ctiles;
   A.Fin = Fin;
   A.mu = mu;
   A.out = out;
   A.acc = acc;
+  A.cellv = h->d_cellv;
+  A.nxtot = h->nxtot;
   A.tab = h->d_tab;
   A.flag = h->d_flag;
   A.dlt = h->d_dlt;
@@ -1402,27 +1409,35 @@ rlb_status launch_adjoint(rlb_ctx* h, int st, int mode, const double* Fin, const
   A.b = RK_B[st];
   A.mode = mode;
   A.split = h->asplit;
-  rlb_adjoint_kernel<<<(int)h->atile_tube.size() * h->asplit, NT, sizeof(AdjSmem), h->stream>>>(A);
+  rlb_adjoint_cell_kernel<<<(int)h->ctile_tube.size(), NT, sizeof(AdjCellSmem), h->stream>>>(A);
+  rlb_adjoint_kernel<<<h->natiles * h->asplit, NT, sizeof(AdjSmem), h->stream>>>(A);
   return cuda_status(cudaGetLastError());
 }
 
-// Tiles of TXA cells (tube after tube) and their dL/dlog(tau) accumulators.
+// Tiles of the adjoint kernels (tube after tube), their per-cell values and dL/dlog(tau) accumulators.
 rlb_status ensure_adjoint_tiles(rlb_ctx* h) {
-  if (h->d_atiles) return RLB_OK;
-  std::vector<int2> tiles;
-  for (size_t b = 0; b < h->tubes.size(); ++b)
-    for (int x0 = 0; x0 < (int)h->tubes[b].Nx; x0 += TXA) {
-      tiles.push_back(make_int2((int)b, x0));
-      h->atile_tube.push_back((int)b);
-    }
-  RLB_CUDA(cudaMalloc(&h->d_atiles, sizeof(int2) * tiles.size()));
-  RLB_CUDA(cudaMalloc(&h->d_dlt, sizeof(double) * tiles.size()));
+  if (h->d_dlt) return RLB_OK;
+  auto make = [&](int width) {
+    std::vector<int2> tiles;
+    for (size_t b = 0; b < h->tubes.size(); ++b)
+      for (int x0 = 0; x0 < (int)h->tubes[b].Nx; x0 += width) tiles.push_back(make_int2((int)b, x0));
+    return tiles;
+  };
+  const std::vector<int2> tiles = make(TXA), ctiles = make(PC);
+  h->natiles = (int)tiles.size();
+  h->ctile_tube.clear();
+  for (const int2& t : ctiles) h->ctile_tube.push_back(t.x);
+  if (!h->d_atiles) RLB_CUDA(cudaMalloc(&h->d_atiles, sizeof(int2) * tiles.size()));
+  if (!h->d_ctiles) RLB_CUDA(cudaMalloc(&h->d_ctiles, sizeof(int2) * ctiles.size()));
+  if (!h->d_cellv) RLB_CUDA(cudaMalloc(&h->d_cellv, sizeof(double) * NCELLV * h->nxtot));
   RLB_CUDA(cudaMemcpyAsync(h->d_atiles, tiles.data(), sizeof(int2) * tiles.size(), cudaMemcpyHostToDevice, h->stream));
-  RLB_CUDA(cudaStreamSynchronize(h->stream));  // the host vector goes out of scope
+  RLB_CUDA(cudaMemcpyAsync(h->d_ctiles, ctiles.data(), sizeof(int2) * ctiles.size(), cudaMemcpyHostToDevice, h->stream));
+  RLB_CUDA(cudaStreamSynchronize(h->stream));  // the host vectors go out of scope
   int occ = 1;
   RLB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, rlb_adjoint_kernel, NT, sizeof(AdjSmem)));
   const long long slots = (long long)h->nsm * std::max(occ, 1);
   if ((long long)tiles.size() < slots) h->asplit = (int)std::min<long long>(8, slots / (long long)tiles.size());
+  RLB_CUDA(cudaMalloc(&h->d_dlt, sizeof(double) * ctiles.size()));  // last: marks the set as complete
   return RLB_OK;
 }
 
@@ -1522,7 +1537,7 @@ rlb_status rlb_backward(rlb_handle h, const double* seed, double* grad_state, do
   if (!h->adj) RLB_CUDA(cudaMalloc(&h->adj, sizeof(double) * se * 4));
   double *L = h->adj, *L1 = L + se, *L2 = L1 + se, *LA = L2 + se;
   RLB_CUDA(cudaMemsetAsync(h->adj, 0, sizeof(double) * se * 4, h->stream));
-  RLB_CUDA(cudaMemsetAsync(h->d_dlt, 0, sizeof(double) * h->atile_tube.size(), h->stream));
+  RLB_CUDA(cudaMemsetAsync(h->d_dlt, 0, sizeof(double) * h->ctile_tube.size(), h->stream));
   st = packed_to_padded(h, seed, L);
   if (st != RLB_OK) return st;
   const long long nck = (h->rec_steps + every - 1) / every;
@@ -1550,13 +1565,13 @@ rlb_status rlb_backward(rlb_handle h, const double* seed, double* grad_state, do
     st = padded_to_packed(h, L, grad_state);
     if (st != RLB_OK) return st;
   }
-  std::vector<double> dl(h->atile_tube.size());
+  std::vector<double> dl(h->ctile_tube.size());
   RLB_CUDA(cudaMemcpyAsync(dl.data(), h->d_dlt, sizeof(double) * dl.size(), cudaMemcpyDeviceToHost, h->stream));
   st = check_flag(h);  // synchronises the stream
   if (st != RLB_OK) return st;
   if (grad_log_tau) {
     for (size_t b = 0; b < h->tubes.size(); ++b) grad_log_tau[b] = 0.0;
-    for (size_t t = 0; t < dl.size(); ++t) grad_log_tau[h->atile_tube[t]] += dl[t];
+    for (size_t t = 0; t < dl.size(); ++t) grad_log_tau[h->ctile_tube[t]] += dl[t];
   }
   return RLB_OK;
 }
@@ -1566,7 +1581,7 @@ rlb_status rlb_moments_vjp(rlb_handle h, const double* grad_moments, double* see
   DeviceGuard gd(h->dev);
   rlb_status st = ensure_adjoint_tiles(h);
   if (st != RLB_OK) return st;
-  rlb_moments_vjp_kernel<<<(int)h->atile_tube.size(), NT, 0, h->stream>>>(h->d_tubes, h->d_atiles, h->d_tab,
+  rlb_moments_vjp_kernel<<<h->natiles, NT, 0, h->stream>>>(h->d_tubes, h->d_atiles, h->d_tab,
                                                                           grad_moments, h->nxtot, seed);
   RLB_CUDA(cudaGetLastError());
   RLB_CUDA(cudaStreamSynchronize(h->stream));
@@ -1578,7 +1593,7 @@ rlb_status rlb_fields_vjp(rlb_handle h, const double* grad_fields, double* seed)
   DeviceGuard gd(h->dev);
   rlb_status st = ensure_adjoint_tiles(h);
   if (st != RLB_OK) return st;
-  rlb_fields_vjp_kernel<<<(int)h->atile_tube.size(), NT, 0, h->stream>>>(
+  rlb_fields_vjp_kernel<<<h->natiles, NT, 0, h->stream>>>(
       h->d_tubes, h->d_atiles, h->d_tab, static_cast<const double*>(h->F), grad_fields, h->nxtot, seed, h->d_flag);
   RLB_CUDA(cudaGetLastError());
   return check_flag(h);  // synchronises the stream
@@ -1592,7 +1607,7 @@ rlb_status rlb_init_vjp(rlb_handle h, const double* P, const double* n, const do
   DeviceGuard gd(h->dev);
   rlb_status st = ensure_adjoint_tiles(h);
   if (st != RLB_OK) return st;
-  rlb_init_vjp_kernel<<<(int)h->atile_tube.size(), NT, sizeof(InitVjpSmem), h->stream>>>(
+  rlb_init_vjp_kernel<<<h->natiles, NT, sizeof(InitVjpSmem), h->stream>>>(
       h->d_tubes, h->d_atiles, h->d_tab, P, n, v, grad_state, grad_P, grad_n, grad_v, h->d_flag);
   RLB_CUDA(cudaGetLastError());
   st = check_flag(h);

@@ -17,28 +17,33 @@
 // hhat_{q+2,k}(beta) and d hhat_{m,k}/d beta = m (k/(2k-1) hhat_{m+1,k-1} + (k+1)/(2k+3) hhat_{m+1,k+1}), the
 // projection of m xi (1 - beta xi)^-(m+1).
 //
-// An adjoint tile has TXA = 60 cells, so that the TXA + 4 interfaces whose stencils reach its cells fit
-// the 64 lanes of a velocity group.
+// One adjoint stage is two launches. rlb_adjoint_cell_kernel reduces each cell's rows to what the collision term
+// needs per cell (the rate, its beta multiple and gM); rlb_adjoint_kernel walks the rows. An adjoint tile has TXA =
+// 60 cells, so that the TXA + 4 interfaces whose stencils reach its cells fit the 64 lanes of a velocity group.
 
 constexpr int TXA = GW - 4;    // cells per adjoint tile
-constexpr int AWF = TXA + 8;   // staged F positions x0-4 .. x0+TXA+3
+constexpr int AWD = TXA + 7;   // first differences F(k) - F(k - 1), k = x0-3 .. x0+TXA+3
 constexpr int AWU = TXA + 6;   // staged adjoint positions x0-3 .. x0+TXA+2
+constexpr int PC = 16;         // cells per CTA of the per-cell kernel
+constexpr int NCELLV = 7;      // per-cell values: b dt r0, b dt r0 beta, b dt gM[5]
 
 struct AdjArgs {
   const TubeDev* tubes;
-  const int2* tiles;  // adjoint tiles (tube, first cell)
-  const double* Fin;  // forward stage input (read with halo)
-  const double* mu;   // adjoint of the stage output (read with halo)
-  double* out;        // adjoint of the stage input (mode 2, 1), or of F^n (mode 0)
-  double* acc;        // adjoint accumulated for F^n over the stages of one step
+  const int2* tiles;   // adjoint tiles (tube, first cell) of TXA cells
+  const int2* ctiles;  // per-cell kernel: tiles of PC cells
+  const double* Fin;   // forward stage input (read with halo)
+  const double* mu;    // adjoint of the stage output (read with halo)
+  double* out;         // adjoint of the stage input (mode 2, 1), or of F^n (mode 0)
+  double* acc;         // adjoint accumulated for F^n over the stages of one step
+  double* cellv;       // [NCELLV][nxtot], written by the per-cell kernel
+  long long nxtot;
   const double* tab;
   int* flag;
-  double* dlt;        // per-tile accumulators of dL/dlog(tau)
-  double a, b;        // the forward stage's Shu-Osher coefficients
-  int mode;           // 2: out = b(mu + dt J^T mu), acc = a mu; 1: the same with acc += a mu;
-                      // 0: out = acc + b(mu + dt J^T mu)
-  int split;          // CTAs per tile (<= 1: one): CTA k of a tile writes velocity rows
-                      // [k Q / split, (k + 1) Q / split) after the per-cell reductions over all rows
+  double* dlt;         // per PC-cell tile: accumulators of dL/dlog(tau)
+  double a, b;         // the forward stage's Shu-Osher coefficients
+  int mode;            // 2: out = b(mu + dt J^T mu), acc = a mu; 1: the same with acc += a mu;
+                       // 0: out = acc + b(mu + dt J^T mu)
+  int split;           // CTAs per tile: CTA k of a tile writes velocity rows [k Q / split, (k + 1) Q / split)
 };
 
 // Legendre coefficients and their beta derivatives (m = 2 .. Np+2, k <= Nv) of the tile's cells
@@ -142,56 +147,335 @@ __device__ void eq_param_grads(const double* tab, int Qp, double n, double T, do
   gb = q4 * ab;
 }
 
+// What the forward's Landau solve keeps for the way back.
+struct LandauRev {
+  double e, beta, n, T, gam, u;  // u = gamma^2
+  double iden, in3, isq;         // 1/(Txx + e), 1/(3n), 1/sqrt((T00 + Txx)^2 - 4 T0x^2)
+};
+
+// As landau_frame, keeping the reciprocals; false if non-physical.
+__device__ __forceinline__ bool landau_keep(const double mom[5], LandauRev& L) {
+  const double A = mom[2] + mom[4], B2 = 2.0 * mom[3];
+  const double disc = fma(A, A, -(B2 * B2));
+  L.isq = rlbdev::rsqrt_nr(disc);
+  L.e = 0.5 * ((mom[2] - mom[4]) + rlbdev::sqrt_nr(disc));
+  L.iden = rlbdev::rcp_nr(mom[4] + L.e);
+  L.beta = rlbdev::div_nr(mom[3], mom[4] + L.e);
+  const double g1 = fma(-L.beta, L.beta, 1.0);
+  L.gam = rlbdev::rsqrt_nr(g1);
+  L.u = rlbdev::rcp_nr(g1);
+  L.n = L.gam * fma(-L.beta, mom[1], mom[0]);
+  L.in3 = rlbdev::rcp_nr(3.0 * L.n);
+  L.T = rlbdev::div_nr(L.e, 3.0 * L.n);
+  return disc > 0.0 && L.e > 0.0 && fabs(L.beta) < 1.0 && L.n > 0.0 && L.T > 0.0;
+}
+
 // Landau solve backwards: adjoints (gn, gT, gbeta) of n, T, beta to the adjoints of the five moments.
-__device__ __forceinline__ void landau_reverse(const double mom[5], double e, double beta, double n, double T,
-                                               double gn, double gT, double gb, double gM[5]) {
-  const double gam = 1.0 / sqrt(1.0 - beta * beta);
+__device__ __forceinline__ void landau_reverse(const double mom[5], const LandauRev& L, double gn, double gT, double gb,
+                                               double gM[5]) {
   // T = e / (3n)
-  double ge = gT / (3.0 * n);
-  gn -= gT * T / n;
+  double ge = gT * L.in3;
+  gn = fma(-3.0 * gT, L.T * L.in3, gn);
   // n = gamma (N0 - beta Nx)
-  gM[0] = gn * gam;
-  gM[1] = -gn * gam * beta;
-  gb += gn * (gam * gam * beta * n - gam * mom[1]);
+  gM[0] = gn * L.gam;
+  gM[1] = -gM[0] * L.beta;
+  gb = fma(gn, L.u * L.beta * L.n - L.gam * mom[1], gb);
   // beta = T0x / (Txx + e)
-  const double den = mom[4] + e;
-  gM[3] = gb / den;
-  gM[4] = -gb * beta / den;
-  ge -= gb * beta / den;
+  gM[3] = gb * L.iden;
+  const double gd = -gM[3] * L.beta;
+  ge += gd;
   // e = ((T00 - Txx) + sqrt((T00 + Txx)^2 - 4 T0x^2)) / 2
-  const double A = mom[2] + mom[4];
-  const double sq = sqrt(A * A - 4.0 * mom[3] * mom[3]);
-  gM[2] = 0.5 * ge * (1.0 + A / sq);
-  gM[4] += 0.5 * ge * (A / sq - 1.0);
-  gM[3] -= 2.0 * ge * mom[3] / sq;
+  const double As = (mom[2] + mom[4]) * L.isq, h = 0.5 * ge;
+  gM[2] = fma(h, As, h);
+  gM[4] = gd + fma(h, As, -h);
+  gM[3] = fma(-2.0 * ge, mom[3] * L.isq, gM[3]);
+}
+
+// Coefficients of the per-cell kernel's steps in m and of xi P_k, by order (filled at compile time).
+struct LegTab {
+  double lead[NP_MAX + 1][NV_MAX + 2], own[NP_MAX + 1][NV_MAX + 2];  // power m = q + 2 to m + 1
+  double lo[NV_MAX + 1], hi[NV_MAX + 1];  // xi f: k/(2k-1) f_{k-1} + (k+1)/(2k+3) f_{k+1}
+};
+constexpr LegTab make_leg_tab() {
+  LegTab t{};
+  for (int q = 0; q <= NP_MAX; ++q)
+    for (int k = 0; k <= NV_MAX + 1; ++k) {
+      t.lead[q][k] = leg_lead(q + 2, k);
+      t.own[q][k] = leg_own(q + 2, k);
+    }
+  for (int k = 0; k <= NV_MAX; ++k) {
+    t.lo[k] = k == 0 ? 0.0 : (double)k / (double)(2 * k - 1);
+    t.hi[k] = (double)(k + 1) / (double)(2 * k + 3);
+  }
+  return t;
+}
+__constant__ LegTab c_leg = make_leg_tab();
+
+struct AdjCellSmem {
+  double red[NT / PC][5][PC];             // partial sums of the slices
+  double h[NP_MAX + 2][NV_MAX + 2][PC];   // Legendre coefficients (legendre_coeffs), powers 2 .. Np + 3
+  double ga[NP_MAX + 1][NV_MAX + 1][PC];  // g_q h_{q,k}
+  double gb[NP_MAX + 1][NV_MAX + 1][PC];  // and its beta derivative at fixed n, T
+  double B[3][NBC][PC];                   // B[i][k] and its T and beta derivatives
+  double cell[5][PC];                     // beta, g0 = n/T, T gamma, gamma^2, 1/T
+  double rate[2][PC];                     // r0, r0 beta
+  double mom[5][PC];
+  double cst[2];                          // 1, -0
+  int ok[PC];
+};
+
+// Per-cell part of an adjoint stage, PC cells per CTA: thread (c, slice) takes radial node i = slice / ns and every
+// ns-th mirror pair of its directions, ns = 16 / Qp.
+//  1. moments of the stage input; Landau frame and the first Legendre coefficients (one thread per cell); the further
+//     powers, their beta derivatives and B[i][k], dB/dT, dB/dbeta with a thread per order and cell (a serial FP64
+//     operation takes 64 cycles of its scheduler's FP64 unit whether one lane or 32 take part, so the per-cell work is
+//     spread over the CTA);
+//  2. Lam[i][k] = sum_j mu_ij r_ij w^xi_j P_k(xi_j) and S0 = sum mu (F^eq - F), S1 = sum mu xi (F^eq - F) over the
+//     slice, Lam at once contracted with B, dB/dT and dB/dbeta (dB/dn = B/n);
+//  3. the sums of the slices, then back through the Landau frame.
+// As a part of each CTA of the row kernel it was repeated `split` times on small handles. On GB300 one adjoint stage of
+// the 2048-cell, 96-velocity inverse problem took 177 us; now this kernel takes 29 (its serial per-cell steps bound
+// it) and the rows 48. 16 tubes of about 1590 cells and 72 velocities: 783 us, now 156 + 363.
+template <int NPc, int NVc>
+__device__ void adjoint_cells(const AdjArgs& A, const TubeDev& T, int tile, int x0, AdjCellSmem& sm) {
+  constexpr int NS = NT / PC;
+  const int tid = threadIdx.x, c = tid % PC, sl = tid / PC;
+  const double* tab = A.tab + T.tab;
+  const int Qp = T.Qp, Qxi = T.Qxi, Nx = T.Nx, ld = T.ld, hq = Qxi / 2;
+  const double* Fin = A.Fin + T.off;
+  const double* mu = A.mu + T.off;
+  const int x = x0 + c;
+  const bool cell = x < Nx;
+  const int ns = NS / Qp, i = sl / ns, js = sl - i * ns;
+  const bool on = cell && i < Qp;
+  if (tid == 0) {
+    sm.cst[0] = 1.0;
+    sm.cst[1] = -0.0;
+  }
+  __syncthreads();
+  const double one = *const_cast<const volatile double*>(&sm.cst[0]);
+  const double nz = *const_cast<const volatile double*>(&sm.cst[1]);
+  {
+    double S0 = 0.0, S1 = 0.0, S2 = 0.0;
+    if (on) {
+      for (int jb = js; jb < hq; jb += ns) {
+        const int jf = Qxi - 1 - jb;
+        const double ff = __ldg(Fin + (size_t)(i * Qxi + jf) * ld + x), fb = __ldg(Fin + (size_t)(i * Qxi + jb) * ld + x);
+        const double s = fma(ff, one, fb);
+        S0 = fma(s, one, S0);
+        S1 = fma(fma(-fb, one, ff), tab[TAB_XI + jf], S1);
+        S2 = fma(s, tab[tab_xi2(Qp, Qxi) + jf], S2);
+      }
+      if ((Qxi & 1) && js == 0) S0 += __ldg(Fin + (size_t)(i * Qxi + hq) * ld + x);
+    }
+    sm.red[sl][0][c] = S0;
+    sm.red[sl][1][c] = S1;
+    sm.red[sl][2][c] = S2;
+  }
+  __syncthreads();
+  // the radial sums of the slices, one thread per node, sum and cell
+  if (sl < 3 * Qp) {
+    const int r = sl / 3, q = sl - 3 * r;
+    double s = 0.0;
+    for (int k = 0; k < ns; ++k) s = fma(sm.red[r * ns + k][q][c], one, s);
+    sm.B[0][sl][c] = s;
+  }
+  __syncthreads();
+  LandauRev L{};
+  bool ok = false;
+  if (tid < PC) {
+    double mom[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int r = 0; r < Qp; ++r) {
+      const double p1 = tab[TAB_PBAR + r], p2 = tab[TAB_PBAR2 + r];
+      const double S0 = sm.B[0][3 * r][c], S1 = sm.B[0][3 * r + 1][c], S2 = sm.B[0][3 * r + 2][c];
+      mom[0] = fma(p1, S0, mom[0]);
+      mom[1] = fma(p1, S1, mom[1]);
+      mom[2] = fma(p2, S0, mom[2]);
+      mom[3] = fma(p2, S1, mom[3]);
+      mom[4] = fma(p2, S2, mom[4]);
+    }
+    ok = cell && landau_keep(mom, L) && fabs(L.beta) <= beta_limit_d(NPc);
+    if (cell && !ok) atomicOr(A.flag, 1);
+    if (ok) {
+      double h[NVc + 2];
+      legendre_first<NVc + 1>(L.beta, L.beta * L.beta, fma(-L.beta, L.beta, 1.0), h);
+#pragma unroll
+      for (int k = 0; k <= NVc + 1; ++k) sm.h[0][k][c] = h[k];
+    }
+    const double iT = ok ? 3.0 * L.n * rlbdev::rcp_nr(L.e) : 0.0;
+    const double r0 = ok ? T.inv_tau * L.gam : 0.0;
+    sm.cell[0][c] = ok ? L.beta : 0.0;
+    sm.cell[1][c] = ok ? L.n * iT : 0.0;
+    sm.cell[2][c] = ok ? L.T * L.gam : 0.0;
+    sm.cell[3][c] = ok ? L.u : 0.0;
+    sm.cell[4][c] = iT;
+    sm.rate[0][c] = r0;
+    sm.rate[1][c] = ok ? r0 * L.beta : 0.0;
+    sm.ok[c] = ok ? 1 : 0;
+#pragma unroll
+    for (int f = 0; f < 5; ++f) sm.mom[f][c] = mom[f];
+  }
+  __syncthreads();
+  const double beta = sm.cell[0][c];
+#pragma unroll 1
+  for (int q = 0; q <= NPc; ++q) {  // power q + 2 to q + 3
+    if (sl <= NVc + 1 && sm.ok[c])
+      sm.h[q + 1][sl][c] =
+          fma(c_leg.lead[q][sl], beta * sm.h[q][sl == 0 ? 1 : sl - 1][c], c_leg.own[q][sl] * sm.h[q][sl][c]);
+    __syncthreads();
+  }
+  if (sl <= NVc) {
+    double g = sm.cell[1][c];
+    const double u = sm.cell[3][c], tg = sm.cell[2][c];
+#pragma unroll
+    for (int q = 0; q <= NPc; ++q) {
+      double a = 0.0, d = 0.0;
+      if (sm.ok[c]) {
+        const double h = sm.h[q][sl][c];
+        d = c_leg.hi[sl] * sm.h[q + 1][sl + 1][c];
+        if (sl > 0) d = fma(c_leg.lo[sl], sm.h[q + 1][sl - 1][c], d);
+        a = g * h;
+        d = (g * u) * fma(-(double)(q + 2) * beta, h, d);
+      }
+      sm.ga[q][sl][c] = a;
+      sm.gb[q][sl][c] = d;
+      g *= tg;
+    }
+  }
+  __syncthreads();
+  for (int w = sl; w < Qp * (NVc + 1); w += NS) {
+    const int r = w / (NVc + 1), k = w - r * (NVc + 1);
+    double B = 0.0, BT = 0.0, Bb = 0.0;
+#pragma unroll
+    for (int q = 0; q <= NPc; ++q) {
+      const double K = tab[TAB_KW + r * (NP_MAX + 1) + q], t = K * sm.ga[q][k][c];
+      B += t;
+      BT = fma((double)(q - 1), t, BT);
+      Bb = fma(K, sm.gb[q][k][c], Bb);
+    }
+    sm.B[0][w][c] = B;
+    sm.B[1][w][c] = BT * sm.cell[4][c];
+    sm.B[2][w][c] = Bb;
+  }
+  __syncthreads();
+  {
+    double S0 = 0.0, S1 = 0.0, lam[NVc + 1];
+#pragma unroll
+    for (int k = 0; k <= NVc; ++k) lam[k] = 0.0;
+    if (on) {
+      const int o = i * (NVc + 1);
+      double B[NVc + 1];
+#pragma unroll
+      for (int k = 0; k <= NVc; ++k) B[k] = sm.B[0][o + k][c];
+      const double r0 = sm.rate[0][c], r1 = sm.rate[1][c];
+      for (int jb = js; jb < hq; jb += ns) {
+        const int jf = Qxi - 1 - jb;
+        const size_t of = (size_t)(i * Qxi + jf) * ld + x, ob = (size_t)(i * Qxi + jb) * ld + x;
+        const double ff = __ldg(Fin + of), fb = __ldg(Fin + ob), mf = __ldg(mu + of), mb = __ldg(mu + ob);
+        const double xi = tab[TAB_XI + jf];
+        const double* pw = tab + TAB_XI + Qxi + jf * (NV_MAX + 1);
+        double E = 0.0, O = 0.0;
+#pragma unroll
+        for (int k = 0; k <= NVc; ++k) {
+          if (k % 2 == 0)
+            E = fma(B[k], pw[k], E);
+          else
+            O = fma(B[k], pw[k], O);
+        }
+        const double df = fma(mf, fma(-ff, one, fma(E, one, O)), nz), db = fma(mb, fma(-fb, one, fma(-O, one, E)), nz);
+        S0 = fma(fma(df, one, db), one, S0);
+        S1 = fma(fma(-db, one, df), xi, S1);
+        const double t = fma(r1, xi, nz), me = fma(mf, one, mb), mo = fma(-mb, one, mf);
+        const double le = fma(-t, mo, fma(r0, me, nz)), lo = fma(-t, me, fma(r0, mo, nz));
+#pragma unroll
+        for (int k = 0; k <= NVc; ++k) lam[k] = fma(k % 2 == 0 ? le : lo, pw[k], lam[k]);
+      }
+      if ((Qxi & 1) && js == 0) {
+        const size_t oc = (size_t)(i * Qxi + hq) * ld + x;
+        const double* pw = tab + TAB_XI + Qxi + hq * (NV_MAX + 1);
+        const double m = __ldg(mu + oc);
+        double E = 0.0;
+#pragma unroll
+        for (int k = 0; k <= NVc; k += 2) E = fma(B[k], pw[k], E);
+        S0 = fma(m, E - __ldg(Fin + oc), S0);
+#pragma unroll
+        for (int k = 0; k <= NVc; k += 2) lam[k] = fma(m * r0, pw[k], lam[k]);
+      }
+    }
+    double pn = 0.0, pT = 0.0, pb = 0.0;
+    if (on) {
+#pragma unroll
+      for (int k = 0; k <= NVc; ++k) {
+        pn = fma(lam[k], sm.B[0][i * (NVc + 1) + k][c], pn);
+        pT = fma(lam[k], sm.B[1][i * (NVc + 1) + k][c], pT);
+        pb = fma(lam[k], sm.B[2][i * (NVc + 1) + k][c], pb);
+      }
+    }
+    sm.red[sl][0][c] = pn;
+    sm.red[sl][1][c] = pT;
+    sm.red[sl][2][c] = pb;
+    sm.red[sl][3][c] = S0;
+    sm.red[sl][4][c] = S1;
+  }
+  __syncthreads();
+  if (sl < 5) {
+    double s = 0.0;
+    for (int k = 0; k < NS; ++k) s = fma(sm.red[k][sl][c], one, s);
+    sm.h[0][sl][c] = s;
+  }
+  __syncthreads();
+  if (tid < 32) {
+    double dl = 0.0;
+    if (tid < PC && cell) {
+      double gM[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, r0 = 0.0, r1 = 0.0;
+      const double bdt = A.b * T.dt;
+      if (ok) {
+        const double S0 = sm.h[0][3][c], S1 = sm.h[0][4][c];
+        r0 = sm.rate[0][c];
+        r1 = sm.rate[1][c];
+        // d r_s / d beta = gamma^3 (beta - xi_j) / tau = r0 gamma^2 (beta - xi_j)
+        const double gn = sm.h[0][0][c] * (3.0 * L.in3), gT = sm.h[0][1][c];
+        const double gb = fma(r0 * L.u, fma(L.beta, S0, -S1), sm.h[0][2][c]);
+        double mom[5];
+#pragma unroll
+        for (int f = 0; f < 5; ++f) mom[f] = sm.mom[f][c];
+        landau_reverse(mom, L, gn, gT, gb, gM);
+        dl = -bdt * r0 * fma(-L.beta, S1, S0);
+      }
+      double* o = A.cellv + T.xoff + x;
+      o[0] = bdt * r0;
+      o[A.nxtot] = bdt * r1;
+#pragma unroll
+      for (int f = 0; f < 5; ++f) o[(2 + f) * A.nxtot] = bdt * gM[f];
+    }
+#pragma unroll
+    for (int d = PC / 2; d > 0; d >>= 1) dl += __shfl_down_sync(0xffffffffu, dl, d);
+    if (tid == 0) A.dlt[tile] += dl;
+  }
+}
+
+__global__ void __launch_bounds__(NT) rlb_adjoint_cell_kernel(AdjArgs A) {
+  extern __shared__ __align__(16) unsigned char adjc_smem_raw[];
+  AdjCellSmem& sm = *reinterpret_cast<AdjCellSmem*>(adjc_smem_raw);
+  const int2 tl = A.ctiles[blockIdx.x];
+  const TubeDev T = A.tubes[tl.x];
+  if (!T.collide) return;  // ballistic: the row kernel reads no per-cell values
+  if (T.Np == 2 && T.Nv == 5)
+    adjoint_cells<2, 5>(A, T, blockIdx.x, tl.y, sm);
+  else
+    adjoint_cells<NP_MAX, NV_MAX>(A, T, blockIdx.x, tl.y, sm);
 }
 
 struct AdjSmem {
-  union {
-    double red[NG][5][GW];  // A: partial moments
-    AdjCoef co;             // B .. B2: hhat and its beta derivative
-  } u;
-  double B[NBC][GW];        // equilibrium coefficients of the cells
-  union {
-    struct {
-      double lam[NBC][GW];  // Lam[i][k] = sum_j mu_ij r_ij w^xi_j P_k(xi_j) (radial row i summed by group i)
-      double s01[NG][2][GW];  // partial S0 = sum mu (F^eq - F), S1 = sum mu xi (F^eq - F)
-    } r;
-    struct {
-      double frow[2][NG][AWF + 1];  // staged F rows
-      double urow[2][NG][AWU + 1];  // staged adjoint rows
-      double P[NG][5][GW];          // psi_X dPhi_X/dF at the five stencil slots (memory order) of interface X
-    } c;
-  } v;
-  double cellv[3][GW];  // n, T, beta
-  double mom[5][GW];
-  double ee[GW];        // e
-  double r0[GW];        // gamma / tau (0: no collision at this cell)
-  double gM[5][GW];     // adjoint of the five moments
-  double dl[GW];        // per-cell share of dL/dlog(tau)
-  int ok[GW];
-  int srcF[AWF + 1];    // source cell of each staged F position
-  int srcU[AWU + 1];    // source cell of each staged adjoint position, -1: outside the tube (zero)
+  double drow[2][NG][AWD + 1];  // first differences of the staged F rows
+  double urow[2][NG][AWU + 1];  // staged adjoint rows
+  double P[NG][5][GW];          // psi_X dPhi_X/dF at the five stencil slots (memory order) of interface X
+  double mom[3 * QP_MAX][GW];   // per radial node: the moment weights' share, even, xi and xi^2 parts
+  double rate[2][GW];           // b dt r0, b dt r0 beta
+  double cst[13];               // constants of the rows (ADJ_CST)
+  double b;                     // the forward stage's b (a register operand)
+  int srcF[TXA + 8];            // source cell of each F position x0-4 .. x0+TXA+3
+  int srcU[AWU + 1];            // source cell of each staged adjoint position, -1: outside the tube (zero)
 };
 
 __device__ __forceinline__ int wrap_cell(int p, int Nx) {
@@ -199,43 +483,43 @@ __device__ __forceinline__ int wrap_cell(int p, int Nx) {
   return r < 0 ? r + Nx : r;
 }
 
-// Partial derivatives dPhi/dv_m (m = 0..4, wind order, v2 the upwind cell) of the WENO5 interface value
-// Phi = sum_k w_k q_k, w_k = alpha_k / sum alpha, alpha_k = d_k / (eps + beta_k)^2:
-//   dPhi/dv = sum_k w_k dq_k/dv + sum_k kappa_k dbeta_k/dv,  kappa_k = -2 w_k (q_k - Phi) / (eps + beta_k).
-__device__ void weno5_grad(const double v[5], double eps, double dP[5]) {
-  constexpr double S6 = 1.0 / 6.0;
-  const double q0 = (2.0 * v[0] - 7.0 * v[1] + 11.0 * v[2]) * S6;
-  const double q1 = (-v[1] + 5.0 * v[2] + 2.0 * v[3]) * S6;
-  const double q2 = (2.0 * v[2] + 5.0 * v[3] - v[4]) * S6;
-  const double a0 = v[0] - 2.0 * v[1] + v[2], b0 = v[0] - 4.0 * v[1] + 3.0 * v[2];
-  const double a1 = v[1] - 2.0 * v[2] + v[3], b1 = v[1] - v[3];
-  const double a2 = v[2] - 2.0 * v[3] + v[4], b2 = 3.0 * v[2] - 4.0 * v[3] + v[4];
-  const double e0 = eps + (13.0 / 12.0 * a0 * a0 + 0.25 * b0 * b0);
-  const double e1 = eps + (13.0 / 12.0 * a1 * a1 + 0.25 * b1 * b1);
-  const double e2 = eps + (13.0 / 12.0 * a2 * a2 + 0.25 * b2 * b2);
-  // alpha_k and the normalised weights, with the refined hardware reciprocal of the forward kernel
-  const double i0 = rlbdev::rcp_nr(e0), i1 = rlbdev::rcp_nr(e1), i2 = rlbdev::rcp_nr(e2);
-  const double s0 = 0.1 * i0 * i0, s1 = 0.6 * i1 * i1, s2 = 0.3 * i2 * i2;
-  const double is = rlbdev::rcp_nr(s0 + s1 + s2);
-  const double w0 = s0 * is, w1 = s1 * is, w2 = s2 * is;
-  const double Phi = w0 * q0 + w1 * q1 + w2 * q2;
-  const double k0 = -2.0 * w0 * (q0 - Phi) * i0;
-  const double k1 = -2.0 * w1 * (q1 - Phi) * i1;
-  const double k2 = -2.0 * w2 * (q2 - Phi) * i2;
-  // dbeta_k/dv = 13/6 a_k da_k/dv + 1/2 b_k db_k/dv
-  const double A0 = 13.0 / 6.0 * k0 * a0, B0 = 0.5 * k0 * b0;
-  const double A1 = 13.0 / 6.0 * k1 * a1, B1 = 0.5 * k1 * b1;
-  const double A2 = 13.0 / 6.0 * k2 * a2, B2 = 0.5 * k2 * b2;
-  dP[0] = w0 * (2.0 / 6.0) + A0 + B0;
-  dP[1] = w0 * (-7.0 / 6.0) + w1 * (-1.0 / 6.0) - 2.0 * A0 - 4.0 * B0 + A1 + B1;
-  dP[2] = w0 * (11.0 / 6.0) + w1 * (5.0 / 6.0) + w2 * (2.0 / 6.0) + A0 + 3.0 * B0 - 2.0 * A1 + A2 + 3.0 * B2;
-  dP[3] = w1 * (2.0 / 6.0) + w2 * (5.0 / 6.0) + A1 - B1 - 2.0 * A2 - 4.0 * B2;
-  dP[4] = w2 * (-1.0 / 6.0) + A2 + B2;
+// Gradient of the WENO5 interface value with respect to its five samples, from the differences d1..d4 in wind order
+// (their common sign does not matter): with Phi = v2 + G(d), dPhi/dv_m = g_m - g_{m+1} + [m = 2], g_l = dG/dd_l, g_0 =
+// g_5 = 0. Returns 1.5 g_l (1.5 = 6/4): 6 G = sum_k w_k r_k, w_k = (c_k / v_k^2) / sum, (c_k) = (1, 6, 3), and
+//   d(6G)/dv_k = 2 w_k (6G - r_k) / v_k,  v_k = x a + y b + e with a, b half the partials of the quadratic form,
+// so that g_l collects -2 w_0, 5 w_0 + w_1, 2 w_1 + 4 w_2, -w_2 and 4 z_k a_k, z_k = w_k (6G - r_k) / v_k, over 6. 66 FP64
+// operations; written on samples with every partial formed on its own it took about 130.
+// k: the constants, in registers (ADJ_CST from shared memory: FP64 operations with an immediate operand, additions and
+// multiplications issue every 19 cycles instead of 16; all-immediate, the row kernel took 11 % longer).
+enum { C_ONE, C_NZ, C_55, C_25, C_4, C_10, C_6, C_3, C_2, C_H, C_Q, C_125, C_15, ADJ_CST };
+__device__ __forceinline__ void weno5_grad(double d1, double d2, double d3, double d4, double e,
+                                           const volatile double* k, double (&g)[4]) {
+  const double one = k[C_ONE], nz = k[C_NZ], c55 = k[C_55], c25 = k[C_25], c4 = k[C_4], c10 = k[C_10];
+  const double t1 = fma(c55, d1, nz), t2 = fma(c55, d2, nz), t3 = fma(c55, d3, nz), t4 = fma(c55, d4, nz);
+  const double s2 = fma(c25, d2, nz), s3 = fma(c25, d3, nz);
+  const double ax0 = fma(c4, d1, -t2), ay0 = fma(c10, d2, -t1);  // 4x^2 - 11xy + 10y^2 of (d1, d2)
+  const double ax1 = fma(c4, d2, -s3), ay1 = fma(c4, d3, -s2);   // 4x^2 - 5xy + 4y^2 of (d2, d3)
+  const double ax2 = fma(c10, d3, -t4), ay2 = fma(c4, d4, -t3);  // 10x^2 - 11xy + 4y^2 of (d3, d4)
+  const double i0 = rlbdev::rcp_nr(fma(d1, ax0, fma(d2, ay0, e)), one);
+  const double i1 = rlbdev::rcp_nr(fma(d2, ax1, fma(d3, ay1, e)), one);
+  const double i2 = rlbdev::rcp_nr(fma(d3, ax2, fma(d4, ay2, e)), one);
+  const double q0 = fma(i0, i0, nz), q1 = fma(k[C_6], fma(i1, i1, nz), nz), q2 = fma(k[C_3], fma(i2, i2, nz), nz);
+  const double is = rlbdev::rcp_nr(fma(fma(q0, one, q1), one, q2), one);
+  const double w0 = fma(q0, is, nz), w1 = fma(q1, is, nz), w2 = fma(q2, is, nz);
+  const double c2 = k[C_2];
+  const double r0 = fma(c2, s2, -fma(c2, d1, nz)), r1 = fma(c2, d3, d2), r2 = fma(c4, d3, -d4);
+  const double G = fma(w0, r0, fma(w1, r1, fma(w2, r2, nz)));
+  const double z0 = fma(fma(w0, i0, nz), fma(-r0, one, G), nz), z1 = fma(fma(w1, i1, nz), fma(-r1, one, G), nz),
+               z2 = fma(fma(w2, i2, nz), fma(-r2, one, G), nz);
+  const double ch = k[C_H], cq = k[C_Q];
+  g[0] = fma(z0, ax0, -fma(ch, w0, nz));
+  g[1] = fma(z0, ay0, fma(z1, ax1, fma(cq, w1, fma(k[C_125], w0, nz))));
+  g[2] = fma(z1, ay1, fma(z2, ax2, fma(ch, w1, w2)));
+  g[3] = fma(z2, ay2, -fma(cq, w2, nz));
 }
 
-template <int NPc, int NVc>
-__device__ void adjoint_tile(const AdjArgs& A, const TubeDev& T, int tile, int x0, int part, int nparts,
-                             AdjSmem& sm) {
+// What bounds it: the FP64 pipe (92 % busy on a batch that fills the GPU): 100 FP64 operations per node.
+__device__ void adjoint_rows(const AdjArgs& A, const TubeDev& T, int x0, int part, int nparts, AdjSmem& sm) {
   const int tid = threadIdx.x, c = tid % GW, g = tid / GW;
   const double* tab = A.tab + T.tab;
   const int Qp = T.Qp, Qxi = T.Qxi, Q = Qp * Qxi, Nx = T.Nx, ld = T.ld;
@@ -246,7 +530,7 @@ __device__ void adjoint_tile(const AdjArgs& A, const TubeDev& T, int tile, int x
   const int x = x0 + c;
   const bool cell = (c < TXA) && (x < Nx);
   const bool periodic = T.bc == RLB_BC_PERIODIC;
-  for (int k = tid; k < AWF; k += NT) {
+  for (int k = tid; k < TXA + 8; k += NT) {
     const int p = x0 - 4 + k;
     sm.srcF[k] = periodic ? wrap_cell(p, Nx) : min(max(p, 0), Nx - 1);
   }
@@ -254,162 +538,89 @@ __device__ void adjoint_tile(const AdjArgs& A, const TubeDev& T, int tile, int x
     const int p = x0 - 3 + k;
     sm.srcU[k] = periodic ? wrap_cell(p, Nx) : ((p >= 0 && p < Nx) ? p : -1);
   }
-  if (g == 0) {
-#pragma unroll
-    for (int f = 0; f < 5; ++f) sm.gM[f][c] = 0.0;
-    sm.r0[c] = 0.0;
-    sm.dl[c] = 0.0;
-    sm.cellv[2][c] = 0.0;
+  if (tid < ADJ_CST) {
+    constexpr double v[ADJ_CST] = {1.0, -0.0, 5.5, 2.5, 4.0, 10.0, 6.0, 3.0, 2.0, 0.5, 0.25, 1.25, 1.5};
+    sm.cst[tid] = v[tid];
+    if (tid == 0) sm.b = A.b;
   }
   if (T.collide) {
-    // A. moments of the forward stage input (as the forward kernel sums them)
-    double m0 = 0, m1 = 0, m2 = 0, m3 = 0, m4 = 0;
-    if (cell) {
-      for (int j = g; j < Qxi; j += NG) {
-        double a = 0.0, b = 0.0;
-        for (int i = 0; i < Qp; ++i) {
-          const double f = __ldg(Fin + (size_t)(i * Qxi + j) * ld + x);
-          a = fma(f, tab[TAB_PBAR + i], a);
-          b = fma(f, tab[TAB_PBAR2 + i], b);
-        }
-        const double xi = tab[TAB_XI + j];
-        m0 += a;
-        m1 = fma(a, xi, m1);
-        m2 += b;
-        m3 = fma(b, xi, m3);
-        m4 = fma(b * xi, xi, m4);
-      }
-    }
-    sm.u.red[g][0][c] = m0;
-    sm.u.red[g][1][c] = m1;
-    sm.u.red[g][2][c] = m2;
-    sm.u.red[g][3][c] = m3;
-    sm.u.red[g][4][c] = m4;
-    __syncthreads();
-    // B. Landau frame, then hhat, d hhat/d beta and the equilibrium coefficients
-    double mom[5] = {0, 0, 0, 0, 0}, e = 1.0, beta = 0.0, n = 1.0, Tt = 1.0;
-    bool ok = false;
-    if (g == 0 && cell) {
-#pragma unroll
-      for (int f = 0; f < 5; ++f) mom[f] = (sm.u.red[0][f][c] + sm.u.red[1][f][c]) + (sm.u.red[2][f][c] + sm.u.red[3][f][c]);
-      ok = landau(mom, e, beta, n, Tt);
-      if (!ok) atomicOr(A.flag, 1);
-    }
-    __syncthreads();  // the union now holds the coefficient scratch
+    // the cell's rate, and gM contracted with the moment weights of radial node i = g: pbar (gM0 + xi gM1) +
+    // pbar^2 (gM2 + xi gM3 + xi^2 gM4) by powers of xi
+    const double* v = A.cellv + T.xoff + x;
     if (g == 0) {
-      sm.cellv[0][c] = n;
-      sm.cellv[1][c] = Tt;
-      sm.cellv[2][c] = ok ? beta : 0.0;
-#pragma unroll
-      for (int f = 0; f < 5; ++f) sm.mom[f][c] = mom[f];
-      sm.ee[c] = e;
-      sm.ok[c] = ok ? 1 : 0;
-      sm.r0[c] = ok ? T.inv_tau / sqrt(1.0 - beta * beta) : 0.0;
+      sm.rate[0][c] = cell ? v[0] : 0.0;
+      sm.rate[1][c] = cell ? v[A.nxtot] : 0.0;
     }
-    __syncthreads();
-    tile_coeffs_d<NPc, NVc>(tab, Qp, &sm.cellv[0][0], sm.ok, sm.u.co, sm.B, A.flag);
-    // R. per cell: Lam[i][k] (group i sums radial row i) and the partial sums S0, S1
-    {
-      double lam[NVc + 1], B[NVc + 1];
-#pragma unroll
-      for (int k = 0; k <= NVc; ++k) lam[k] = 0.0;
-      double S0 = 0.0, S1 = 0.0;
-      if (cell && g < Qp && sm.ok[c]) {
-#pragma unroll
-        for (int k = 0; k <= NVc; ++k) B[k] = sm.B[g * (NV_MAX + 1) + k][c];
-        const double r0 = sm.r0[c], bt = sm.cellv[2][c];
-        for (int j = 0; j < Qxi; ++j) {
-          const size_t o = (size_t)(g * Qxi + j) * ld + x;
-          const double m = __ldg(mu + o), f = __ldg(Fin + o);
-          const double xi = tab[TAB_XI + j];
-          const double* pw = tab + TAB_XI + Qxi + j * (NV_MAX + 1);
-          double feq = 0.0;
-#pragma unroll
-          for (int k = 0; k <= NVc; ++k) feq = fma(B[k], pw[k], feq);
-          const double d = m * (feq - f);
-          S0 += d;
-          S1 = fma(d, xi, S1);
-          const double mr = m * r0 * fma(-bt, xi, 1.0);
-#pragma unroll
-          for (int k = 0; k <= NVc; ++k) lam[k] = fma(mr, pw[k], lam[k]);
-        }
+    if (g < Qp) {
+      double m0 = 0.0, m1 = 0.0, m2 = 0.0;
+      if (cell) {
+        const double p1 = tab[TAB_PBAR + g], p2 = tab[TAB_PBAR2 + g];
+        m0 = fma(p1, v[2 * A.nxtot], p2 * v[4 * A.nxtot]);
+        m1 = fma(p1, v[3 * A.nxtot], p2 * v[5 * A.nxtot]);
+        m2 = p2 * v[6 * A.nxtot];
       }
-      if (g < QP_MAX) {
-#pragma unroll
-        for (int k = 0; k <= NVc; ++k) sm.v.r.lam[g * (NV_MAX + 1) + k][c] = lam[k];
-      }
-      sm.v.r.s01[g][0][c] = S0;
-      sm.v.r.s01[g][1][c] = S1;
-    }
-    __syncthreads();
-    // B2. per cell: gradients of the collision term with respect to n, T, beta, then to the moments
-    if (g == 0 && cell && sm.ok[c]) {
-      const double n_ = sm.cellv[0][c], T_ = sm.cellv[1][c], b_ = sm.cellv[2][c], r0 = sm.r0[c];
-      const double S0 = (sm.v.r.s01[0][0][c] + sm.v.r.s01[1][0][c]) + (sm.v.r.s01[2][0][c] + sm.v.r.s01[3][0][c]);
-      const double S1 = (sm.v.r.s01[0][1][c] + sm.v.r.s01[1][1][c]) + (sm.v.r.s01[2][1][c] + sm.v.r.s01[3][1][c]);
-      double gn, gT, gb;
-      eq_param_grads<NPc, NVc>(tab, Qp, n_, T_, b_, sm.u.co, c, sm.v.r.lam, gn, gT, gb);
-      // d r_s / d beta = gamma^3 (beta - xi_j) / tau = r0 gamma^2 (beta - xi_j)
-      gb += r0 / (1.0 - b_ * b_) * (b_ * S0 - S1);
-      double m5[5], gM[5];
-#pragma unroll
-      for (int f = 0; f < 5; ++f) m5[f] = sm.mom[f][c];
-      landau_reverse(m5, sm.ee[c], b_, n_, T_, gn, gT, gb, gM);
-#pragma unroll
-      for (int f = 0; f < 5; ++f) sm.gM[f][c] = gM[f];
-      sm.dl[c] = -A.b * T.dt * r0 * fma(-b_, S1, S0);
+      sm.mom[3 * g][c] = m0;
+      sm.mom[3 * g + 1][c] = m1;
+      sm.mom[3 * g + 2][c] = m2;
     }
   }
-  __syncthreads();  // srcF/srcU, gM, r0 ready; the union is free for the row buffers
-  if (tid == 0 && part == 0) {
-    double s = 0.0;
-    for (int k = 0; k < TXA; ++k) s += sm.dl[k];
-    A.dlt[tile] += s;
-  }
+  __syncthreads();
 
-  // C. rows: transposed WENO5 flux differences, collision terms, Runge-Kutta combination
-  const double a = A.a, b = A.b, dt = T.dt, inv_dx = 1.0 / T.dx;
-  const double bt = sm.cellv[2][c], r0 = sm.r0[c];
-  double* P0 = sm.v.c.P[g][0];
+  // rows: transposed WENO5 flux differences, collision terms, Runge-Kutta combination
+  const double a = A.a, cpsi = A.b * T.dt * (2.0 / 3.0) / T.dx;  // 4/6 of b dt / dx, with weno5_grad's 6/4
+  double* P0 = sm.P[g][0];
   int buf = 0;
   const int r_end = (part + 1) * Q / nparts;
-  for (int s0 = part * Q / nparts; s0 < r_end; s0 += NG, buf ^= 1) {
-    const int s = s0 + g;
-    const bool rv = s < r_end;
-    const int i = rv ? s / Qxi : 0, j = rv ? s - i * Qxi : 0;
-    double* fr = sm.v.c.frow[buf][g];
-    double* ur = sm.v.c.urow[buf][g];
-    if (rv) {
+  for (int s = part * Q / nparts + g; s < r_end; s += NG, buf ^= 1) {  // uniform over the group
+    const int i = s / Qxi, j = s - i * Qxi;
+    double* dr = sm.drow[buf][g];
+    double* ur = sm.urow[buf][g];
+    const volatile double* cst = sm.cst;
+    const double one = cst[C_ONE], nz = cst[C_NZ];
+    {
+      // difference k lies between positions k and k + 1 of srcF; each lane loads position c + 1 and takes position c
+      // from the lane below
       const double* fs = Fin + (size_t)s * ld;
+      const double v = __ldg(fs + sm.srcF[c + 1]);
+      double w = __shfl_up_sync(0xffffffffu, v, 1);
+      if ((c & 31) == 0) w = __ldg(fs + sm.srcF[c]);
+      dr[c] = fma(-w, one, v);
+      if (c < AWD - GW) dr[GW + c] = __ldg(fs + sm.srcF[GW + 1 + c]) - __ldg(fs + sm.srcF[GW + c]);
       const double* us = mu + (size_t)s * ld;
-      for (int k = c; k < AWF; k += GW) fr[k] = __ldg(fs + sm.srcF[k]);
       for (int k = c; k < AWU; k += GW) {
         const int q = sm.srcU[k];
         ur[k] = q >= 0 ? __ldg(us + q) : 0.0;
       }
     }
+    const double prev = (cell && A.mode != 2) ? acc[(size_t)s * ld + x] : 0.0;  // needed at the row's end only
     group_sync(g);
     const double xi = tab[TAB_XI + j];
-    const bool fwd = xi > 0.0;
-    if (rv) {
-      // lane c: interface X = x0 - 1 + c (wind toward +x) or x0 - 2 + c (toward -x); its stencil is staged at
-      // fr[c .. c+4] in memory order and mu(X), mu(X-1) at ur[c+2], ur[c+1] (resp. ur[c+1], ur[c])
-      const double psi = xi * inv_dx * (fwd ? ur[c + 2] - ur[c + 1] : ur[c + 1] - ur[c]);
-      double v[5], dP[5];
+    const bool fwd = 2 * j + 1 > Qxi;  // xi_j > 0, decided without an FP64 comparison
+    if (2 * j + 1 != Qxi) {
+      // lane c: interface X = x0 - 1 + c (wind toward +x) or x0 - 2 + c (toward -x); its stencil's differences are
+      // dr[c .. c+3] in memory order and mu(X), mu(X-1) are ur[c+2], ur[c+1] (resp. ur[c+1], ur[c])
+      const int lo = fwd ? c + 1 : c;
+      const double psi = fma(fma(xi, cpsi, nz), fma(-ur[lo], one, ur[lo + 1]), nz);
+      const double e = tab[tab_eps(Qxi) + s];
+      double h[4];
+      weno5_grad(dr[fwd ? c : c + 3], dr[fwd ? c + 1 : c + 2], dr[fwd ? c + 2 : c + 1], dr[fwd ? c + 3 : c], e, cst, h);
+      P0[(fwd ? 0 : 4) * GW + c] = fma(-psi, h[0], nz);
+      P0[(fwd ? 1 : 3) * GW + c] = fma(psi, fma(-h[1], one, h[0]), nz);
+      P0[2 * GW + c] = fma(psi, fma(fma(-h[2], one, h[1]), one, cst[C_15]), nz);
+      P0[(fwd ? 3 : 1) * GW + c] = fma(psi, fma(-h[3], one, h[2]), nz);
+      P0[(fwd ? 4 : 0) * GW + c] = fma(psi, h[3], nz);
+    } else {
 #pragma unroll
-      for (int m = 0; m < 5; ++m) v[m] = fwd ? fr[c + m] : fr[c + 4 - m];
-      const double eps = tab[tab_eps(Qxi) + 3 * s] * (1.0 / (3.0 * rlbdev::C0));
-      weno5_grad(v, eps, dP);
-#pragma unroll
-      for (int m = 0; m < 5; ++m) P0[(fwd ? m : 4 - m) * GW + c] = psi * dP[m];
+      for (int m = 0; m < 5; ++m) P0[m * GW + c] = 0.0;
     }
     group_sync(g);
-    if (rv && cell) {
+    if (cell) {
       // cell y = x0 + c gathers slot m of interface lane c + 4 - m; the open boundary's ghost positions
       // (copies of the edge cells) add theirs to the edge cells
-      double w = 0.0;
-#pragma unroll
-      for (int m = 0; m < 5; ++m) w += P0[m * GW + c + 4 - m];
+      double w = fma(P0[c + 4], one, P0[GW + c + 3]);
+      w = fma(P0[2 * GW + c + 2], one, w);
+      w = fma(P0[3 * GW + c + 1], one, w);
+      w = fma(P0[4 * GW + c], one, w);
       if (!periodic && (x == 0 || x == Nx - 1)) {
         for (int side = 0; side < 2; ++side) {
           if ((side == 0 && x != 0) || (side == 1 && x != Nx - 1)) continue;
@@ -424,38 +635,29 @@ __device__ void adjoint_tile(const AdjArgs& A, const TubeDev& T, int tile, int x
         }
       }
       const double m_ = ur[c + 3];
-      if (r0 != 0.0) {
-        const double pb = tab[TAB_PBAR + i], pb2 = tab[TAB_PBAR2 + i];
-        w = fma(-r0 * fma(-bt, xi, 1.0), m_, w);
-        w = fma(pb, fma(xi, sm.gM[1][c], sm.gM[0][c]), w);
-        w = fma(pb2, fma(xi, fma(xi, sm.gM[4][c], sm.gM[3][c]), sm.gM[2][c]), w);
+      if (T.collide) {
+        w = fma(fma(sm.rate[1][c], xi, -sm.rate[0][c]), m_, w);
+        w = fma(fma(sm.mom[3 * i + 2][c], xi, sm.mom[3 * i + 1][c]), xi, fma(sm.mom[3 * i][c], one, w));
       }
-      const double val = b * fma(dt, w, m_);
+      const double val = fma(sm.b, m_, w);
       const size_t o = (size_t)s * ld + x;
-      if (A.mode == 2) {
-        out[o] = val;
-        acc[o] = a * m_;
-      } else if (A.mode == 1) {
-        out[o] = val;
-        acc[o] = fma(a, m_, acc[o]);
+      if (A.mode == 0) {
+        out[o] = fma(prev, one, val);
       } else {
-        out[o] = acc[o] + val;
+        out[o] = val;
+        acc[o] = fma(a, m_, prev);
       }
     }
   }
 }
 
-__global__ void __launch_bounds__(NT) rlb_adjoint_kernel(AdjArgs A) {
+__global__ void __launch_bounds__(NT, 2) rlb_adjoint_kernel(AdjArgs A) {
   extern __shared__ __align__(16) unsigned char adj_smem_raw[];
   AdjSmem& sm = *reinterpret_cast<AdjSmem*>(adj_smem_raw);
-  const int K = A.split > 1 ? A.split : 1;
-  const int t = blockIdx.x / K, part = blockIdx.x - t * K;
+  const int t = blockIdx.x / A.split, part = blockIdx.x - t * A.split;
   const int2 tl = A.tiles[t];
   const TubeDev T = A.tubes[tl.x];
-  if (T.Np == 2 && T.Nv == 5)
-    adjoint_tile<2, 5>(A, T, t, tl.y, part, K, sm);
-  else
-    adjoint_tile<NP_MAX, NV_MAX>(A, T, t, tl.y, part, K, sm);
+  adjoint_rows(A, T, tl.y, part, A.split, sm);
 }
 
 // Seed of the state from the adjoint of the five moments of each cell: dL/dF_s = sum_a c_a(s) dL/dM_a.

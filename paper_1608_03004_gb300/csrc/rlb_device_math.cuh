@@ -15,6 +15,15 @@ __device__ __forceinline__ double rcp_nr(double d) {
   return fma(x0, fma(e, e, e), x0);
 }
 
+// The same with 1 in a register that the compiler does not know, for loops bound by the FP64 pipe (an immediate operand
+// costs three of its cycles).
+__device__ __forceinline__ double rcp_nr(double d, double one) {
+  double x0;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x0) : "d"(d));
+  const double e = fma(-d, x0, one);
+  return fma(x0, fma(e, e, e), x0);
+}
+
 // 1/sqrt(x) for positive, normal x: the hardware approximation of rsqrt.approx.ftz.f64 refined by one step of
 // third order, y1 = y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2 (the binomial series of (1 - e)^(-1/2)): five FP64
 // operations and no branch, where 1.0 / sqrt(x) takes about 35.

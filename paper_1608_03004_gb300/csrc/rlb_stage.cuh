@@ -136,8 +136,8 @@ __host__ __device__ constexpr double beta_limit_d(int NPc) { return NPc <= 2 ? 0
 // here about 2 operations for each of 18 and 46 steps). FP64 operations bound every kernel that calls this. With the
 // series, the FP32 steps of 128 uneven moving tubes kept the FP64 pipe 85 % busy; on GB300 they went from 4.42 to 2.43
 // ms, the FP32 stress tube's (half its gas in motion) from 6.5 to 5.2 ms, the 400-cell FP64 tube's from 89 to 54 us.
-template <int NM, int KV>
-__device__ __forceinline__ void legendre_coeffs(double beta, double b2, double g1, double (&h)[NM][KV + 1]) {
+template <int KV>
+__device__ __forceinline__ void legendre_first(double beta, double b2, double g1, double (&h)[KV + 1]) {
   double C[KV + 2];
   {
     // K = KV + 2 + 54 / -log2((1 - s)/(1 + s)), (1 - s)/(1 + s) = beta^2 / (1 + s)^2 (beta = 0: K = KV + 2)
@@ -156,22 +156,29 @@ __device__ __forceinline__ void legendre_coeffs(double beta, double b2, double g
   for (int k = KV; k >= 1; --k) C[k - 1] = fma(g_leg[k], b2 * C[k + 1], C[k]);
   const double inv = rlbdev::rcp_nr(C[0]);
   double bk = inv, sk = 1.0;  // beta^k / c_0; (2k+1) s_k
-  h[0][0] = 1.0;
+  h[0] = 1.0;
 #pragma unroll
   for (int k = 1; k <= KV; ++k) {
     bk *= beta;
     sk *= (double)(k + 1) / (double)(2 * k + 1);
-    h[0][k] = ((2 * k + 1) * sk) * (bk * C[k]);
+    h[k] = ((2 * k + 1) * sk) * (bk * C[k]);
   }
+}
+// Coefficients of the step from the power m to m + 1 at order k: h' = lead beta h[k == 0 ? 1 : k - 1] + own h[k].
+__host__ __device__ constexpr double leg_lead(int m, int k) {
+  return k == 0 ? (m - 2) / 3.0 : (double)((k + m - 1) * (2 * k + 1)) / (double)(2 * k - 1);
+}
+__host__ __device__ constexpr double leg_own(int m, int k) { return k == 0 ? m : m - 1 - k; }
+
+template <int NM, int KV>
+__device__ __forceinline__ void legendre_coeffs(double beta, double b2, double g1, double (&h)[NM][KV + 1]) {
+  legendre_first<KV>(beta, b2, g1, h[0]);
 #pragma unroll
   for (int q = 1; q < NM; ++q) {
     const int m = q + 1;  // from m to m + 1
-    h[q][0] = fma((m - 2) / 3.0, beta * h[q - 1][1], (double)m * h[q - 1][0]);
 #pragma unroll
-    for (int k = 1; k <= KV; ++k) {
-      const double lead = (double)((k + m - 1) * (2 * k + 1)) / (double)(2 * k - 1);
-      h[q][k] = fma(lead, beta * h[q - 1][k - 1], (double)(m - 1 - k) * h[q - 1][k]);
-    }
+    for (int k = 0; k <= KV; ++k)
+      h[q][k] = fma(leg_lead(m, k), beta * h[q - 1][k == 0 ? 1 : k - 1], leg_own(m, k) * h[q - 1][k]);
   }
 }
 
