@@ -428,6 +428,40 @@ void fill_eps(double* out, double* outf, int Qp, int Qxi, const double* wp, cons
     }
 }
 
+// Round the radial factors KW[i][q] (TAB_KW) so that the equilibrium keeps the moments it must: with p = pbar and p^2
+// as the kernels hold them, sum_i p_i KW[i][q] 2 (q+1)! is 1 at q = 1 and sum_i p_i^2 KW[i][q] 2 (q+1)! is 3 at q = 2 (N^0 =
+// n, T^00 = 3 n T), else 0. Each entry stays within one unit of its nearest double; of those roundings the one
+// with the smallest residual is taken. The collision applies F^eq in every stage, so what the residual leaves adds up
+// over a run: with entries rounded to nearest the residual of T^00 is 1.2e-15 at Qp = 3.
+void balance_radial(double* T, const double* pb, int Qp, int Np) {
+  long double f = 2.0L;
+  for (int q = 0; q <= Np; ++q) {
+    f *= q + 1;
+    double best[QP_MAX], near[QP_MAX], w = -1.0;
+    int n = 1;
+    for (int i = 0; i < Qp; ++i) {
+      near[i] = T[TAB_KW + i * (NP_MAX + 1) + q];
+      n *= 3;
+    }
+    for (int t = 0; t < n; ++t) {
+      double k[QP_MAX];
+      long double m1 = 0.0L, m2 = 0.0L;
+      for (int i = 0, r = t; i < Qp; ++i, r /= 3) {
+        k[i] = r % 3 == 0 ? near[i] : std::nextafter(near[i], r % 3 == 1 ? -1e300 : 1e300);
+        m1 += (long double)pb[i] * k[i];
+        m2 += (long double)(pb[i] * pb[i]) * k[i];
+      }
+      const double res = (double)std::max(std::fabs(m1 * f - (q == 1 ? 1.0L : 0.0L)),
+                                          std::fabs(m2 * f - (q == 2 ? 3.0L : 0.0L)) / 3.0L);
+      if (w < 0.0 || res < w) {
+        w = res;
+        std::copy(k, k + Qp, best);
+      }
+    }
+    for (int i = 0; i < Qp; ++i) T[TAB_KW + i * (NP_MAX + 1) + q] = best[i];
+  }
+}
+
 // The FP64 tables of one tube (layout in rlb_internal.h): quadrature nodes and weights, the radial factors
 // K[i][q], w^xi_j P_k(xi_j), the per-stage b dt xi_j / dx and the WENO5 epsilon terms. pb, wp, xi, wxi receive
 // the quadrature (Qp and Qxi entries). Returns false if a quadrature rule cannot be built.
@@ -452,6 +486,7 @@ bool fill_tube_tables(const rlb_tube& t, double* pb, double* wp, double* xi, dou
       T[TAB_KW + i * (NP_MAX + 1) + q] = (double)(wp[i] * acc / f);
     }
   }
+  balance_radial(T, pb, t.Qp, t.Np);
   for (int j = 0; j < t.Qxi; ++j) {
     T[TAB_XI + j] = xi[j];
     T[tab_xi2(t.Qp, t.Qxi) + j] = xi[j] * xi[j];
