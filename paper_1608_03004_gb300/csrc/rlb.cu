@@ -283,8 +283,8 @@ rlb_status ensure_series_tables(int dev) {
   double leg[LEG_MAX + 1];
   for (int k = 0; k <= LEG_MAX; ++k) leg[k] = -(double)(k * (k + 2)) / (double)((2 * k + 1) * (2 * k + 3));
   RLB_CUDA(cudaMemcpyToSymbol(g_leg, leg, sizeof(leg)));
-  const void* fp64[3] = {(const void*)rlb_stage_kernel<0>, (const void*)rlb_stage_kernel<1>,
-                         (const void*)rlb_stage_kernel<2>};
+  const void* fp64[4] = {(const void*)rlb_stage_kernel<0>, (const void*)rlb_stage_kernel<1>,
+                         (const void*)rlb_stage_kernel<2>, (const void*)rlb_stage_kernel<SCHED_CLUSTER>};
   const void* rp[6] = {(const void*)rlb_stage_rp_kernel<float, 0>, (const void*)rlb_stage_rp_kernel<float, 1>,
                        (const void*)rlb_stage_rp_kernel<float, 2>, (const void*)rlb_stage_rp_kernel<__nv_bfloat16, 0>,
                        (const void*)rlb_stage_rp_kernel<__nv_bfloat16, 1>,
@@ -804,6 +804,27 @@ rlb_status rlb_init_riemann(rlb_handle* out, const rlb_tube* tubes, int32_t ntub
 
 namespace {
 
+// One FP64 stage with one CTA per work item. The items of a split tile are a thread-block cluster that shares the
+// tile's per-cell work.
+rlb_status launch_tiles(const StageArgs& A, size_t smem, cudaStream_t stream) {
+  if (A.split <= 1) {
+    rlb_stage_kernel<0><<<A.ntiles, NT, smem, stream>>>(A);
+    return cuda_status(cudaGetLastError());
+  }
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)A.split;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(A.ntiles * A.split));
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cuda_status(cudaLaunchKernelEx(&cfg, rlb_stage_kernel<SCHED_CLUSTER>, A));
+}
+
 // One stage st of the current step as one launch on `stream`, with work counter ctr (counter schedule).
 rlb_status launch_stage(rlb_ctx* h, cudaStream_t stream, int st, int* ctr) {
   const void* in[3] = {h->F, h->F1, h->F2};
@@ -834,7 +855,7 @@ rlb_status launch_stage(rlb_ctx* h, cudaStream_t stream, int st, int* ctr) {
     A.counter = ctr;
     A.split = split;
     if (sched == RLB_SCHED_TILE)
-      rlb_stage_kernel<0><<<grid, NT, h->stage_smem, stream>>>(A);
+      return launch_tiles(A, h->stage_smem, stream);
     else if (sched == RLB_SCHED_STRIDE)
       rlb_stage_kernel<1><<<grid, NT, h->stage_smem, stream>>>(A);
     else
@@ -1421,8 +1442,7 @@ rlb_status launch_stage_ptrs(rlb_ctx* h, int st, const double* Fn, const double*
   A.schedule = RLB_SCHED_TILE;
   A.counter = h->d_counters;
   A.split = eff_split(h);
-  rlb_stage_kernel<0><<<h->ntiles * A.split, NT, h->stage_smem, h->stream>>>(A);
-  return cuda_status(cudaGetLastError());
+  return launch_tiles(A, h->stage_smem, h->stream);
 }
 
 rlb_status launch_adjoint(rlb_ctx* h, int st, int mode, const double* Fin, const double* mu, double* out,

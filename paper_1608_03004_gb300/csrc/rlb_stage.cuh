@@ -243,22 +243,24 @@ __device__ __forceinline__ void store_cell_coeffs(bool ok, double beta, double b
     for (int k = 0; k <= NVc; ++k) cs.ge[q][k][c] = ge[q][k];
 }
 
+// B[i][k] of cell c from its ge[q][k].
+template <int NPc>
+__device__ __forceinline__ double row_coeff(const double* tab, int i, const double (*ge)[NV_MAX + 1][GW], int k, int c) {
+  const double* KW = tab + TAB_KW + i * (NP_MAX + 1);
+  double B = KW[0] * ge[0][k][c];
+#pragma unroll
+  for (int q = 1; q <= NPc; ++q) B = fma(KW[q], ge[q][k][c], B);
+  return B;
+}
+
 // Fill B[i (NVc+1) + k][c] (radial rows i < Qp) for the TX cells of a tile from cs.ge: group g builds radial row
 // i = g. Coefficients of w^xi_j P_k(xi_j).
 template <int NPc, int NVc>
 __device__ __forceinline__ void build_rows(const double* tab, int Qp, const CoefSmem& cs, double (*Bs)[GW]) {
   const int c = threadIdx.x % GW, i = threadIdx.x / GW;
   if (c >= TX || i >= Qp) return;
-  double KW[NPc + 1];
 #pragma unroll
-  for (int q = 0; q <= NPc; ++q) KW[q] = tab[TAB_KW + i * (NP_MAX + 1) + q];
-#pragma unroll
-  for (int k = 0; k <= NVc; ++k) {
-    double B = KW[0] * cs.ge[0][k][c];
-#pragma unroll
-    for (int q = 1; q <= NPc; ++q) B = fma(KW[q], cs.ge[q][k][c], B);
-    Bs[i * (NVc + 1) + k][c] = B;
-  }
+  for (int k = 0; k <= NVc; ++k) Bs[i * (NVc + 1) + k][c] = row_coeff<NPc>(tab, i, cs.ge, k, c);
 }
 
 // Orders up to which the stage kernel evaluates the equilibrium as a polynomial in xi (two Horner chains in xi^2) from
@@ -314,7 +316,124 @@ constexpr size_t stage_smem_bytes(int brows) { return offsetof(StageSmem, B) + (
 // that the compiler cannot fold (read from shared memory).
 __device__ __forceinline__ double add_r(double a, double b, double one) { return fma(a, one, b); }
 
+// Phase B of one cell: the five moments from the groups' radial sums, Landau frame, Legendre coefficients into
+// sm.u.a.coef and the collision rate into sm.rate (zeros for a cell past the tube's end or a non-physical one).
 template <int NPc, int NVc>
+__device__ __forceinline__ void cell_phase(const StageArgs& A, const TubeDev& T, const double* tab, bool cell, int c,
+                                           StageSmem& sm) {
+  double beta = 0.0, b2 = 0.0, g1 = 1.0, gam = 1.0, g0 = 0.0, tg = 1.0;
+  bool ok = false;
+  if (cell) {
+    double mom[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int i = 0; i < QP_MAX; ++i) {
+      if (i < T.Qp) {
+        double Si[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+          Si[q] = (sm.u.a.red[0][3 * i + q][c] + sm.u.a.red[1][3 * i + q][c]) +
+                  (sm.u.a.red[2][3 * i + q][c] + sm.u.a.red[3][3 * i + q][c]);
+        const double p1 = tab[TAB_PBAR + i], p2 = tab[TAB_PBAR2 + i];
+        mom[0] = fma(p1, Si[0], mom[0]);
+        mom[1] = fma(p1, Si[1], mom[1]);
+        mom[2] = fma(p2, Si[0], mom[2]);
+        mom[3] = fma(p2, Si[1], mom[3]);
+        mom[4] = fma(p2, Si[2], mom[4]);
+      }
+    }
+    ok = landau_frame(mom, beta, b2, g1, gam, g0, tg);
+    if (ok && A.warn != nullptr && stiff(T, beta)) atomicOr(A.warn, RLB_WARN_STIFF);
+    ok = ok && fabs(beta) <= beta_limit(NPc);
+    if (!ok) atomicOr(A.flag, 1);
+  }
+  store_cell_coeffs<NPc, NVc>(ok, beta, b2, g1, g0, tg, sm.u.a.coef, c);
+  // b dt gamma / tau and its beta multiple: the stage's collision rate is r0 - r1 xi_j
+  const double r0 = ok ? (A.b * T.dt) * (T.inv_tau * gam) : 0.0;
+  sm.rate[0][c] = r0;
+  sm.rate[1][c] = ok ? r0 * beta : 0.0;
+}
+
+// Thread-block clusters: barrier over the CTAs of the cluster (release / acquire), and a store to the same place of the
+// shared memory of CTA `rank` of the cluster.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_store(double* p, int rank, double v) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(r), "d"(v) : "memory");
+}
+
+// Moments, Landau frame and equilibrium coefficients of a tile shared by the nparts CTAs that split its velocity rows
+// (one cluster): CTA `part` takes every cell of its share through phases A and B with the operations and the order of
+// summation of the unshared path, and stores the results to all of them. Small handles only: the per-cell work was
+// repeated in each of up to 8 CTAs, and with FP64 at 2 lanes per SM and clock that was two thirds of a stage.
+template <int NPc, int NVc>
+__device__ __forceinline__ void cluster_coeffs(const StageArgs& A, const TubeDev& T, int x0, int part, int nparts,
+                                               StageSmem& sm) {
+  const int tid = threadIdx.x;
+  const double* tab = A.tab + T.tab;
+  const int Qp = T.Qp, Qxi = T.Qxi, Nx = T.Nx, ld = T.ld, hq = Qxi / 2;
+  const double* Fin = A.Fin + T.off;
+  const int share = (TX + nparts - 1) / nparts, c0 = part * share;  // cells c0 .. c0 + share - 1 of the tile
+  const int lg = share <= 8 ? 3 : (share <= 16 ? 4 : 5), cc = tid & ((1 << lg) - 1), c = c0 + cc;
+  const bool own = cc < share && c < TX, cell = own && x0 + c < Nx;
+  const double one = *const_cast<const volatile double*>(&sm.cst[0]);
+  // A. one slice (every NG-th mirror pair) of one radial node per thread
+  for (int w = tid >> lg; w < NG * Qp; w += NT >> lg) {
+    const int gs = w & (NG - 1), i = w / NG;
+    double S0 = 0.0, S1 = 0.0, S2 = 0.0;
+    if (cell) {
+      const double* r = Fin + (size_t)(i * Qxi) * ld + x0 + c;
+#pragma unroll 2
+      for (int jb = gs; jb < hq; jb += NG) {
+        const int jf = Qxi - 1 - jb;
+        const double ff = __ldg(r + (size_t)jf * ld), fb = __ldg(r + (size_t)jb * ld);
+        const double sum = add_r(fb, ff, one), dif = fma(-fb, one, ff);
+        S0 = add_r(sum, S0, one);
+        S1 = fma(dif, tab[TAB_XI + jf], S1);
+        S2 = fma(sum, tab[tab_xi2(Qp, Qxi) + jf], S2);
+      }
+      if ((Qxi & 1) && gs == (hq % NG)) S0 += __ldg(r + (size_t)hq * ld);
+    }
+    if (own) {
+      sm.u.a.red[gs][3 * i][c] = S0;
+      sm.u.a.red[gs][3 * i + 1][c] = S1;
+      sm.u.a.red[gs][3 * i + 2][c] = S2;
+    }
+  }
+  __syncthreads();
+  // B. per cell, on one warp (a different scheduler in neighbouring CTAs)
+  if ((tid >> 5) == (part & 3) && (tid & 31) < share && c0 + (tid & 31) < TX)
+    cell_phase<NPc, NVc>(A, T, tab, x0 + c0 + (tid & 31) < Nx, c0 + (tid & 31), sm);
+  __syncthreads();
+  if (own) {
+    for (int w = tid >> lg; w < Qp * (NVc + 1); w += NT >> lg) {
+      const int i = w / (NVc + 1), k = w - i * (NVc + 1);
+      sm.B[w][c] = row_coeff<NPc>(tab, i, sm.u.a.coef.ge, k, c);
+    }
+  }
+  __syncthreads();
+  if constexpr (NVc <= NV_MONO) {
+    if (own && (tid >> lg) < Qp) legendre_to_monomial<NVc>(&sm.B[(tid >> lg) * (NVc + 1)][c], GW);
+    __syncthreads();
+  }
+  cluster_sync();  // every CTA of the cluster runs: its shared memory can be written
+  if (own) {
+    const int rows = Qp * (NVc + 1);
+    for (int w = tid >> lg; w < rows + 2; w += NT >> lg) {
+      double* p = w < rows ? &sm.B[w][c] : &sm.rate[w - rows][c];
+      const double v = *p;
+      for (int r = 0; r < nparts; ++r)
+        if (r != part) cluster_store(p, r, v);
+    }
+  }
+  cluster_sync();  // all shares are in place, and no CTA is written to after it
+}
+
+// COOP: the nparts CTAs of a tile are one thread-block cluster and share phases A and B.
+template <int NPc, int NVc, bool COOP>
 __device__ void stage_tile(const StageArgs& A, const TubeDev& T, int x0, int part, int nparts, StageSmem& sm) {
   constexpr bool MONO = NVc <= NV_MONO;
   const int tid = threadIdx.x, c = tid % GW, g = tid / GW;
@@ -335,7 +454,9 @@ __device__ void stage_tile(const StageArgs& A, const TubeDev& T, int x0, int par
   }
   __syncthreads();
 
-  if (T.collide) {
+  if (COOP && T.collide) {
+    cluster_coeffs<NPc, NVc>(A, T, x0, part, nparts, sm);
+  } else if (T.collide) {
     // A. moments of the stage input. The groups split the mirror pairs of directions (xi_jf = -xi_jb > 0) and
     //    keep, per radial node i, S0 = sum_j F_ij, S1 = sum_j F_ij xi_j and S2 = sum_j F_ij xi_j^2 from the sum
     //    s = F(xi) + F(-xi) and difference d = F(xi) - F(-xi) of each pair (S0 += s, S1 += d xi, S2 += s xi^2):
@@ -373,38 +494,7 @@ __device__ void stage_tile(const StageArgs& A, const TubeDev& T, int x0, int par
     for (int k = 0; k < 3 * QP_MAX; ++k) sm.u.a.red[g][k][c] = S[k];
     __syncthreads();
     // B. Landau frame and Legendre coefficients (one thread per cell), then the equilibrium coefficients
-    if (g == 0) {
-      double beta = 0.0, b2 = 0.0, g1 = 1.0, gam = 1.0, g0 = 0.0, tg = 1.0;
-      bool ok = false;
-      if (cell) {
-        double mom[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-        for (int i = 0; i < QP_MAX; ++i) {
-          if (i < Qp) {
-            double Si[3];
-#pragma unroll
-            for (int q = 0; q < 3; ++q)
-              Si[q] = (sm.u.a.red[0][3 * i + q][c] + sm.u.a.red[1][3 * i + q][c]) +
-                      (sm.u.a.red[2][3 * i + q][c] + sm.u.a.red[3][3 * i + q][c]);
-            const double p1 = tab[TAB_PBAR + i], p2 = tab[TAB_PBAR2 + i];
-            mom[0] = fma(p1, Si[0], mom[0]);
-            mom[1] = fma(p1, Si[1], mom[1]);
-            mom[2] = fma(p2, Si[0], mom[2]);
-            mom[3] = fma(p2, Si[1], mom[3]);
-            mom[4] = fma(p2, Si[2], mom[4]);
-          }
-        }
-        ok = landau_frame(mom, beta, b2, g1, gam, g0, tg);
-        if (ok && A.warn != nullptr && stiff(T, beta)) atomicOr(A.warn, RLB_WARN_STIFF);
-        ok = ok && fabs(beta) <= beta_limit(NPc);
-        if (!ok) atomicOr(A.flag, 1);
-      }
-      store_cell_coeffs<NPc, NVc>(ok, beta, b2, g1, g0, tg, sm.u.a.coef, c);
-      // b dt gamma / tau and its beta multiple: the stage's collision rate is r0 - r1 xi_j
-      const double r0 = ok ? (A.b * T.dt) * (T.inv_tau * gam) : 0.0;
-      sm.rate[0][c] = r0;
-      sm.rate[1][c] = ok ? r0 * beta : 0.0;
-    }
+    if (g == 0) cell_phase<NPc, NVc>(A, T, tab, cell, c, sm);
     __syncthreads();
     build_rows<NPc, NVc>(tab, Qp, sm.u.a.coef, sm.B);
     if constexpr (MONO) {
@@ -574,19 +664,21 @@ __device__ void stage_tile(const StageArgs& A, const TubeDev& T, int x0, int par
 // register operands and Horner equilibria, 34.8 once no conversion instruction was left in the rows (df_split,
 // df_join). The relaxation-time sweep: 3.62, 2.89, 2.67. 80 registers for 3 CTAs per SM: two CTAs with 128 registers ran
 // 8 % slower on the stress tube, four with 64 registers 1 % faster there and 3 % slower on the sweep.
-// SCHED is the launch's schedule (compile time, so that the one-CTA-per-tile kernel carries no tile loop).
+// SCHED is the launch's schedule (compile time, so that the one-CTA-per-tile kernel carries no tile loop);
+// SCHED_CLUSTER: one CTA per item, the items of a tile being one thread-block cluster.
+constexpr int SCHED_CLUSTER = 3;
 template <int SCHED>
 __global__ void __launch_bounds__(NT, 3) rlb_stage_kernel(StageArgs A) {
   extern __shared__ __align__(16) unsigned char stage_smem_raw[];
   StageSmem& sm = *reinterpret_cast<StageSmem*>(stage_smem_raw);
   const int K = A.split > 1 ? A.split : 1;
-  for_each_tile(A.ntiles * K, SCHED, A.counter, [&](int item) {
+  for_each_tile(A.ntiles * K, SCHED == SCHED_CLUSTER ? 0 : SCHED, A.counter, [&](int item) {
     const int t = item / K, part = item - t * K;
     const int2 tl = A.tiles[t];
     const TubeDev T = A.tubes[tl.x];
     if (T.Np == 2 && T.Nv == 5)
-      stage_tile<2, 5>(A, T, tl.y, part, K, sm);
+      stage_tile<2, 5, SCHED == SCHED_CLUSTER>(A, T, tl.y, part, K, sm);
     else
-      stage_tile<NP_MAX, NV_MAX>(A, T, tl.y, part, K, sm);
+      stage_tile<NP_MAX, NV_MAX, SCHED == SCHED_CLUSTER>(A, T, tl.y, part, K, sm);
   });
 }
