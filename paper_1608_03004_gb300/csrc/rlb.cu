@@ -138,7 +138,7 @@ __device__ void init_tile(const InitArgs& A, const TubeDev& T, int x0, InitSmem&
       const double g1 = fma(-v, v, 1.0), gam = 1.0 / sqrt(g1), Tt = P / n;
       const bool ok = P > 0.0 && n > 0.0 && fabs(v) <= beta_limit(NPc);
       if (cell && !ok) atomicOr(A.flag, 1);
-      store_cell_coeffs<NPc, NVc>(cell && ok, v, v * v, g1, n / Tt, Tt * gam, sm.coef, c);
+      store_cell_coeffs<NPc, NVc>(tab, cell && ok, v, v * v, g1, n / Tt, Tt * gam, sm.coef, c);
     }
     __syncthreads();
     if (pass == 1 && sm.tie == 0) break;  // uniform over the CTA
@@ -428,40 +428,6 @@ void fill_eps(double* out, double* outf, int Qp, int Qxi, const double* wp, cons
     }
 }
 
-// Round the radial factors KW[i][q] (TAB_KW) so that the equilibrium keeps the moments it must: with p = pbar and p^2
-// as the kernels hold them, sum_i p_i KW[i][q] 2 (q+1)! is 1 at q = 1 and sum_i p_i^2 KW[i][q] 2 (q+1)! is 3 at q = 2 (N^0 =
-// n, T^00 = 3 n T), else 0. Each entry stays within one unit of its nearest double; of those roundings the one
-// with the smallest residual is taken. The collision applies F^eq in every stage, so what the residual leaves adds up
-// over a run: with entries rounded to nearest the residual of T^00 is 1.2e-15 at Qp = 3.
-void balance_radial(double* T, const double* pb, int Qp, int Np) {
-  long double f = 2.0L;
-  for (int q = 0; q <= Np; ++q) {
-    f *= q + 1;
-    double best[QP_MAX], near[QP_MAX], w = -1.0;
-    int n = 1;
-    for (int i = 0; i < Qp; ++i) {
-      near[i] = T[TAB_KW + i * (NP_MAX + 1) + q];
-      n *= 3;
-    }
-    for (int t = 0; t < n; ++t) {
-      double k[QP_MAX];
-      long double m1 = 0.0L, m2 = 0.0L;
-      for (int i = 0, r = t; i < Qp; ++i, r /= 3) {
-        k[i] = r % 3 == 0 ? near[i] : std::nextafter(near[i], r % 3 == 1 ? -1e300 : 1e300);
-        m1 += (long double)pb[i] * k[i];
-        m2 += (long double)(pb[i] * pb[i]) * k[i];
-      }
-      const double res = (double)std::max(std::fabs(m1 * f - (q == 1 ? 1.0L : 0.0L)),
-                                          std::fabs(m2 * f - (q == 2 ? 3.0L : 0.0L)) / 3.0L);
-      if (w < 0.0 || res < w) {
-        w = res;
-        std::copy(k, k + Qp, best);
-      }
-    }
-    for (int i = 0; i < Qp; ++i) T[TAB_KW + i * (NP_MAX + 1) + q] = best[i];
-  }
-}
-
 // The FP64 tables of one tube (layout in rlb_internal.h): quadrature nodes and weights, the radial factors
 // K[i][q], w^xi_j P_k(xi_j), the per-stage b dt xi_j / dx and the WENO5 epsilon terms. pb, wp, xi, wxi receive
 // the quadrature (Qp and Qxi entries). Returns false if a quadrature rule cannot be built.
@@ -479,14 +445,15 @@ bool fill_tube_tables(const rlb_tube& t, double* pb, double* wp, double* xi, dou
         for (int u = 1; u <= q; ++u) C = C * (l - q + u) / u;
         acc += C * rlbq::laguerre1(l, pb[i]);
       }
-      if (q % 2) acc = -acc;
-      T[TAB_K + i * (NP_MAX + 1) + q] = (double)acc;
-      long double f = 4.0L;  // 4 (q + 1)!
-      for (int u = 2; u <= q + 1; ++u) f *= u;
-      T[TAB_KW + i * (NP_MAX + 1) + q] = (double)(wp[i] * acc / f);
+      T[TAB_K + i * (NP_MAX + 1) + q] = (double)((q % 2) ? -acc : acc);
     }
   }
-  balance_radial(T, pb, t.Qp, t.Np);
+  long double KW[QP_MAX * (NP_MAX + 1)];
+  if (!rlbq::radial_factors(t.Qp, t.Np, KW)) return false;
+  const double* c = RADIAL_SCALE[t.Qp == 3 ? 0 : t.Np - 1];
+  for (int q = 0; q <= NP_MAX; ++q) T[TAB_KC + q] = c[q];
+  for (int i = 0; i < t.Qp; ++i)
+    for (int q = 0; q <= t.Np; ++q) T[TAB_KW + i * (NP_MAX + 1) + q] = (double)(KW[i * (t.Np + 1) + q] / c[q]);
   for (int j = 0; j < t.Qxi; ++j) {
     T[TAB_XI + j] = xi[j];
     T[tab_xi2(t.Qp, t.Qxi) + j] = xi[j] * xi[j];

@@ -334,8 +334,9 @@ __device__ void adjoint_cells(const AdjArgs& A, const TubeDev& T, int tile, int 
         const double h = sm.h[q][sl][c];
         d = c_leg.hi[sl] * sm.h[q + 1][sl + 1][c];
         if (sl > 0) d = fma(c_leg.lo[sl], sm.h[q + 1][sl - 1][c], d);
-        a = g * h;
-        d = (g * u) * fma(-(double)(q + 2) * beta, h, d);
+        const double gq = g * tab[TAB_KC + q];
+        a = gq * h;
+        d = (gq * u) * fma(-(double)(q + 2) * beta, h, d);
       }
       sm.ga[q][sl][c] = a;
       sm.gb[q][sl][c] = d;

@@ -13,6 +13,9 @@ bool gauss_legendre(int n, double* x, double* w);
 bool gauss_laguerre1(int n, double* x, double* w);
 double laguerre1(int l, double x);  // L^(1)_l(x)
 double legendre(int k, double x);   // P_k(x)
+// w^p_i (-1)^q sum_{l=q}^{Np} C(l,q) L^(1)_l(pbar_i) / (4 (q+1)!) at KW[i (Np + 1) + q], n radial nodes, evaluated at
+// the nodes in extended precision
+bool radial_factors(int n, int Np, long double* KW);
 }  // namespace rlbq
 
 namespace rlb {
@@ -51,8 +54,8 @@ struct TubeDev {
 //   [3 QP_MAX, 3 QP_MAX + QP_MAX (NP_MAX+1))   K[i][q] = (-1)^q sum_{l=q}^{Np} C(l,q) L^(1)_l(pbar_i)
 //                                               at [i (NP_MAX+1) + q]: the radial factor multiplying
 //                                               s^(q+2) hhat_{q+2,k} in the truncated equilibrium
-//   then w^p_i K[i][q] / (4 (q+1)!) at [i (NP_MAX+1) + q]: the same with the factors that the per-cell
-//                                               coefficients take out (legendre_coeffs)
+//   then KW[i][q] = w^p_i K[i][q] / (4 (q+1)! c_q) at [i (NP_MAX+1) + q]: the same with the factors that the
+//                                               per-cell coefficients take out (legendre_coeffs), and c_q (NP_MAX+1)
 //   then xi_j (Qxi), then w^xi_j P_k(xi_j) at [j (NV_MAX+1) + k] (Qxi (NV_MAX+1)), zero for k > Nv,
 //   then b_st dt xi_j / dx at [st Qxi + j] for the three Runge-Kutta stages, b = (1, 1/4, 2/3),
 //   then per velocity s = i Qxi + j the WENO5 epsilon term e = 3 eps ws^2, ws = w^p_i w^xi_j / 2 (the limiter acts on
@@ -65,7 +68,16 @@ constexpr int TAB_PBAR2 = QP_MAX;
 constexpr int TAB_WP = 2 * QP_MAX;
 constexpr int TAB_K = 3 * QP_MAX;
 constexpr int TAB_KW = TAB_K + QP_MAX * (NP_MAX + 1);
-constexpr int TAB_XI = TAB_KW + QP_MAX * (NP_MAX + 1);
+constexpr int TAB_KC = TAB_KW + QP_MAX * (NP_MAX + 1);
+constexpr int TAB_XI = TAB_KC + NP_MAX + 1;
+// Scales c_q of the radial factors by (Qp, Np) = (3, 2), (4, 2), (4, 3): the collision applies the equilibrium in every
+// stage, so the rounding of these few constants is the part of its error that adds up over a run. Divided by c_q the
+// entries of one q all lie within 4e-18 of doubles (found by a search over k / 2^17), where the entries themselves
+// round by up to 1e-16; the per-cell factors g_q carry c_q.
+constexpr double RADIAL_SCALE[3][NP_MAX + 1] = {
+    {1.5519180297851562, 1.469573974609375, 1.5150070190429688, 1.0},
+    {1.5099411010742188, 1.9296340942382812, 1.1760940551757812, 1.0},
+    {1.0521774291992188, 1.4824142456054688, 1.3223495483398438, 1.790069580078125}};
 __host__ __device__ inline int tab_pw(int Qxi) { return TAB_XI + Qxi; }
 __host__ __device__ inline int tab_cxi(int Qxi) { return TAB_XI + Qxi + Qxi * (NV_MAX + 1); }
 __host__ __device__ inline int tab_eps(int Qxi) { return tab_cxi(Qxi) + 3 * Qxi; }

@@ -182,20 +182,21 @@ __device__ __forceinline__ void legendre_coeffs(double beta, double b2, double g
   }
 }
 
-// The same times the per-cell factors of the equilibrium: ge[q][k] = g_q h[q][k], so that
+// The same times the per-cell factors of the equilibrium: ge[q][k] = c_q g_q h[q][k] (c_q: TAB_KC), so that
 //   F^eq_ij = sum_k B[i][k] w^xi_j P_k(xi_j),  B[i][k] = sum_q TAB_KW[i][q] ge[q][k]
 // (Eq. (feqtrunc): Laguerre generating function for the radial projection, Legendre projection of each
 // (1 - beta xi)^-m for the angular one; B = n/(4T^3) w^p_i sum_q s^(q+2) K[i][q] hhat_{q+2,k}, s = T/gamma, so
 // that g_q = (n/T) (T gamma)^q).
 template <int NPc, int NVc>
-__device__ __forceinline__ void cell_coeffs(double beta, double b2, double g1, double g0, double tg,
+__device__ __forceinline__ void cell_coeffs(const double* tab, double beta, double b2, double g1, double g0, double tg,
                                             double (&ge)[NPc + 1][NVc + 1]) {
   legendre_coeffs<NPc + 1, NVc>(beta, b2, g1, ge);
   double g = g0;
 #pragma unroll
   for (int q = 0; q <= NPc; ++q) {
+    const double gq = g * tab[TAB_KC + q];
 #pragma unroll
-    for (int k = 0; k <= NVc; ++k) ge[q][k] *= g;
+    for (int k = 0; k <= NVc; ++k) ge[q][k] *= gq;
     g *= tg;
   }
 }
@@ -226,11 +227,11 @@ struct CoefSmem {
 
 // Per-cell coefficients of one cell into column c of cs.ge (all zero for a non-physical cell).
 template <int NPc, int NVc>
-__device__ __forceinline__ void store_cell_coeffs(bool ok, double beta, double b2, double g1, double g0, double tg,
+__device__ __forceinline__ void store_cell_coeffs(const double* tab, bool ok, double beta, double b2, double g1, double g0, double tg,
                                                   CoefSmem& cs, int c) {
   double ge[NPc + 1][NVc + 1];
   if (ok) {
-    cell_coeffs<NPc, NVc>(beta, b2, g1, g0, tg, ge);
+    cell_coeffs<NPc, NVc>(tab, beta, b2, g1, g0, tg, ge);
   } else {
 #pragma unroll
     for (int q = 0; q <= NPc; ++q)
@@ -346,7 +347,7 @@ __device__ __forceinline__ void cell_phase(const StageArgs& A, const TubeDev& T,
     ok = ok && fabs(beta) <= beta_limit(NPc);
     if (!ok) atomicOr(A.flag, 1);
   }
-  store_cell_coeffs<NPc, NVc>(ok, beta, b2, g1, g0, tg, sm.u.a.coef, c);
+  store_cell_coeffs<NPc, NVc>(tab, ok, beta, b2, g1, g0, tg, sm.u.a.coef, c);
   // b dt gamma / tau and its beta multiple: the stage's collision rate is r0 - r1 xi_j
   const double r0 = ok ? (A.b * T.dt) * (T.inv_tau * gam) : 0.0;
   sm.rate[0][c] = r0;

@@ -122,11 +122,11 @@ __device__ __forceinline__ void cell_coeffs_rp(const TubeDev* Tg, const double* 
 #pragma unroll
       for (int q = 0; q <= NPc; ++q) {
         f *= q + 1;
-        ge[q][0] = f * g;
+        ge[q][0] = f * (g * tab[TAB_KC + q]);
         g *= tg;
       }
     } else {
-      cell_coeffs<NPc, NVc>(beta, b2, g1, g0, tg, ge);
+      cell_coeffs<NPc, NVc>(tab, beta, b2, g1, g0, tg, ge);
     }
   }
 #pragma unroll
