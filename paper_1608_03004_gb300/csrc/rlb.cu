@@ -29,8 +29,10 @@
 #include <cstddef>
 #include <complex>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <mutex>
+#include <queue>
 #include <type_traits>
 #include <new>
 #include <utility>
@@ -160,38 +162,83 @@ __global__ void __launch_bounds__(NT) rlb_init_kernel(InitArgs A) {
     init_tile<S, NP_MAX, NV_MAX>(A, T, tl.y, sm);
 }
 
+// FP64 view of a stored population without a conversion instruction, which would occupy the FP64 pipe (subnormal FP32
+// populations read as zero).
+__device__ __forceinline__ double ld_w(const double* p) { return __ldg(p); }
+__device__ __forceinline__ double ld_w(const float* p) { return rlbdev::df_widen(__ldg(p)); }
+__device__ __forceinline__ double ld_w(const __nv_bfloat16* p) {
+  return rlbdev::df_widen(__uint_as_float((unsigned)__ldg(reinterpret_cast<const unsigned short*>(p)) << 16));
+}
+
 // Fields of every cell: the five moments summed over F in FP64, or, with M != NULL, read from M for tubes with
 // collisions (reduced storage: the stage kernel leaves the FP64 moments of its output there, so F need not be
-// read again; ballistic tubes keep no moments and are summed), then the Landau frame.
+// read again; ballistic tubes keep no moments and are summed), then the Landau frame. The sums are those of the FP64
+// stage kernel's phase A: four groups split the mirror pairs of directions, 2.5 FP64 operations per population,
+// register operands. On GB300, FP64 sweep (31.7 M populations): 336 us with one thread per cell walking all rows, 182 us
+// so; the 400-cell tube 17.5 -> 9 us.
 template <typename S>
-__global__ void __launch_bounds__(GW) rlb_fields_kernel(const TubeDev* tubes, const int2* tiles, const void* Fv,
-                                                         const double* tabs, double* out, long long nxtot,
-                                                         int* flag, const double* M = nullptr) {
-  const S* F = static_cast<const S*>(Fv);
+__global__ void __launch_bounds__(NT) rlb_fields_kernel(const TubeDev* tubes, const int2* tiles, const void* Fv,
+                                                        const double* tabs, double* out, long long nxtot, int* flag,
+                                                        const double* M = nullptr) {
+  __shared__ double red[NG][3 * QP_MAX][GW];
+  __shared__ double cst[1];
   const int2 tl = tiles[blockIdx.x];
   const TubeDev T = tubes[tl.x];
-  const int c = threadIdx.x, x = tl.y + c;
-  if (c >= TX || x >= T.Nx) return;
+  const int c = threadIdx.x % GW, g = threadIdx.x / GW, x = tl.y + c;
+  const bool cell = c < TX && x < T.Nx, kept = M != nullptr && T.collide;
   const double* tab = tabs + T.tab;
-  const S* f = F + T.off + x;
+  if (!kept) {
+    if (threadIdx.x == 0) cst[0] = 1.0;
+    __syncthreads();
+    const double one = *const_cast<const volatile double*>(&cst[0]);
+    const int Qp = T.Qp, Qxi = T.Qxi, hq = Qxi / 2;
+    const S* f = static_cast<const S*>(Fv) + T.off + x;
+    double s[3 * QP_MAX];
+#pragma unroll
+    for (int k = 0; k < 3 * QP_MAX; ++k) s[k] = 0.0;
+    if (cell) {
+      for (int jb = g; jb < hq; jb += NG) {
+        const int jf = Qxi - 1 - jb;
+        const double xi = tab[TAB_XI + jf], xi2 = tab[tab_xi2(Qp, Qxi) + jf];
+#pragma unroll
+        for (int i = 0; i < QP_MAX; ++i) {
+          if (i < Qp) {
+            const double ff = ld_w(f + (size_t)(i * Qxi + jf) * T.ld), fb = ld_w(f + (size_t)(i * Qxi + jb) * T.ld);
+            const double sum = add_r(fb, ff, one);
+            s[3 * i] = add_r(sum, s[3 * i], one);
+            s[3 * i + 1] = fma(fma(-fb, one, ff), xi, s[3 * i + 1]);
+            s[3 * i + 2] = fma(sum, xi2, s[3 * i + 2]);
+          }
+        }
+      }
+      if ((Qxi & 1) && g == (hq % NG)) {
+#pragma unroll
+        for (int i = 0; i < QP_MAX; ++i)
+          if (i < Qp) s[3 * i] += ld_w(f + (size_t)(i * Qxi + hq) * T.ld);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 3 * QP_MAX; ++k) red[g][k][c] = s[k];
+    __syncthreads();
+  }
+  if (g != 0 || !cell) return;
   double mom[5] = {0, 0, 0, 0, 0};
-  if (M != nullptr && T.collide) {
+  if (kept) {
 #pragma unroll
     for (int k = 0; k < 5; ++k) mom[k] = M[k * nxtot + T.xoff + x];
-  }
-  for (int j = 0; j < ((M != nullptr && T.collide) ? 0 : T.Qxi); ++j) {
-    double a = 0.0, b = 0.0;
+  } else {
     for (int i = 0; i < T.Qp; ++i) {
-      const double v = ld_d<S>(f + (size_t)(i * T.Qxi + j) * T.ld);
-      a = fma(v, tab[TAB_PBAR + i], a);
-      b = fma(v, tab[TAB_PBAR2 + i], b);
+      double s[3];
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        s[q] = (red[0][3 * i + q][c] + red[1][3 * i + q][c]) + (red[2][3 * i + q][c] + red[3][3 * i + q][c]);
+      const double p1 = tab[TAB_PBAR + i], p2 = tab[TAB_PBAR2 + i];
+      mom[0] = fma(p1, s[0], mom[0]);
+      mom[1] = fma(p1, s[1], mom[1]);
+      mom[2] = fma(p2, s[0], mom[2]);
+      mom[3] = fma(p2, s[1], mom[3]);
+      mom[4] = fma(p2, s[2], mom[4]);
     }
-    const double xi = tab[TAB_XI + j];
-    mom[0] += a;
-    mom[1] = fma(a, xi, mom[1]);
-    mom[2] += b;
-    mom[3] = fma(b, xi, mom[3]);
-    mom[4] = fma(b * xi, xi, mom[4]);
   }
   double e, beta, n, Tt;
   if (!landau(mom, e, beta, n, Tt)) atomicOr(flag, 1);
@@ -506,6 +553,40 @@ rlb_status validate(const rlb_tube* t) {
   return RLB_OK;
 }
 
+// Work items per tile of the FP64 stage kernel. The velocity rows of a tile are split over several CTAs where that
+// shortens the launch: for each split the tiles, in their order, are handed to `slots` resident CTAs as they come
+// free, an item costing its rows plus a fixed part worth ROW0 rows (the per-cell chain, barriers and start-up: 12 to 16
+// us on GB300, where a CTA takes 0.6 us per row), and the split with the earliest end is taken. Handles of
+// many times the slots are never split. Against "split only what cannot fill the slots": 13 uneven tubes, 545
+// tiles of 16 to 288 rows for 456 slots, 137 -> 115 us per stage.
+int choose_split(const std::vector<rlb_tube>& tubes, const std::vector<int2>& tiles, int slots) {
+  constexpr int ROW0 = 20;
+  const long long n = (long long)tiles.size();
+  if (n >= 8LL * slots) return 1;
+  int best = 1;
+  double best_end = -1.0;
+  for (int s = 1; s <= SPLIT_MAX; ++s) {
+    std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+    double end = 0.0;
+    for (const int2& t : tiles)
+      for (int k = 0; k < s; ++k) {
+        double at = 0.0;
+        if ((long long)free_at.size() >= slots) {
+          at = free_at.top();
+          free_at.pop();
+        }
+        at += ROW0 + (double)tubes[t.x].Qp * tubes[t.x].Qxi / s;
+        end = std::max(end, at);
+        free_at.push(at);
+      }
+    if (best_end < 0.0 || end < best_end) {
+      best_end = end;
+      best = s;
+    }
+  }
+  return best;
+}
+
 rlb_status create(rlb_handle* out, const rlb_tube* tubes, int32_t ntubes, const double* xleft, void* stream,
                   rlb_ctx** hp) {
   if (!out || !tubes || ntubes < 1) return RLB_EINVAL;
@@ -652,10 +733,7 @@ rlb_status create(rlb_handle* out, const rlb_tube* tubes, int32_t ntubes, const 
     RLB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&h->occupancy, rlb_stage_rp_kernel<__nv_bfloat16, 1>, RP_NT,
                                                            rp_smem_bytes(h->brows)));
   if (h->occupancy < 1) h->occupancy = 1;
-  // a handle whose tiles cannot fill the resident slots splits each tile's velocity rows over several CTAs
-  const long long slots = (long long)h->nsm * h->occupancy;
-  if (h->storage == RLB_STORAGE_F64 && h->ntiles < slots)
-    h->split = (int)std::min<long long>(SPLIT_MAX, slots / h->ntiles);
+  if (h->storage == RLB_STORAGE_F64) h->split = choose_split(h->tubes, tiles, h->nsm * h->occupancy);
   return RLB_OK;
 }
 
@@ -673,10 +751,10 @@ rlb_status check_flag(rlb_ctx* h) {
 // written from outside the step (initial condition, rlb_set_state).
 rlb_status refresh_moments(rlb_ctx* h) {
   if (h->storage == RLB_STORAGE_F32)
-    rlb_fields_kernel<float><<<h->ntiles, GW, 0, h->stream>>>(h->d_tubes, h->d_tiles, h->F, h->d_tab, h->M,
+    rlb_fields_kernel<float><<<h->ntiles, NT, 0, h->stream>>>(h->d_tubes, h->d_tiles, h->F, h->d_tab, h->M,
                                                                h->nxtot, h->d_flag);
   else if (h->storage == RLB_STORAGE_BF16)
-    rlb_fields_kernel<__nv_bfloat16><<<h->ntiles, GW, 0, h->stream>>>(h->d_tubes, h->d_tiles, h->F, h->d_tab,
+    rlb_fields_kernel<__nv_bfloat16><<<h->ntiles, NT, 0, h->stream>>>(h->d_tubes, h->d_tiles, h->F, h->d_tab,
                                                                        h->M, h->nxtot, h->d_flag);
   return cuda_status(cudaGetLastError());
 }
@@ -1068,13 +1146,13 @@ rlb_status rlb_moments(rlb_handle h, double* out, int32_t out_on_device) {
     dst = h->d_fields;
   }
   if (h->storage == RLB_STORAGE_F64)
-    rlb_fields_kernel<double><<<h->ntiles, GW, 0, h->stream>>>(h->d_tubes, h->d_tiles, h->F, h->d_tab, dst,
+    rlb_fields_kernel<double><<<h->ntiles, NT, 0, h->stream>>>(h->d_tubes, h->d_tiles, h->F, h->d_tab, dst,
                                                                 h->nxtot, h->d_flag);
   else if (h->storage == RLB_STORAGE_F32)
-    rlb_fields_kernel<float><<<h->ntiles, GW, 0, h->stream>>>(h->d_tubes, h->d_tiles, h->F, h->d_tab, dst,
+    rlb_fields_kernel<float><<<h->ntiles, NT, 0, h->stream>>>(h->d_tubes, h->d_tiles, h->F, h->d_tab, dst,
                                                                h->nxtot, h->d_flag, h->M);
   else
-    rlb_fields_kernel<__nv_bfloat16><<<h->ntiles, GW, 0, h->stream>>>(h->d_tubes, h->d_tiles, h->F, h->d_tab, dst,
+    rlb_fields_kernel<__nv_bfloat16><<<h->ntiles, NT, 0, h->stream>>>(h->d_tubes, h->d_tiles, h->F, h->d_tab, dst,
                                                                        h->nxtot, h->d_flag, h->M);
   RLB_CUDA(cudaGetLastError());
   if (!out_on_device)
