@@ -495,12 +495,14 @@ bool fill_tube_tables(const rlb_tube& t, double* pb, double* wp, double* xi, dou
       T[TAB_K + i * (NP_MAX + 1) + q] = (double)((q % 2) ? -acc : acc);
     }
   }
-  long double KW[QP_MAX * (NP_MAX + 1)];
-  if (!rlbq::radial_factors(t.Qp, t.Np, KW)) return false;
   const double* c = RADIAL_SCALE[t.Qp == 3 ? 0 : t.Np - 1];
-  for (int q = 0; q <= NP_MAX; ++q) T[TAB_KC + q] = c[q];
-  for (int i = 0; i < t.Qp; ++i)
-    for (int q = 0; q <= t.Np; ++q) T[TAB_KW + i * (NP_MAX + 1) + q] = (double)(KW[i * (t.Np + 1) + q] / c[q]);
+  long double f = 4.0L;  // 4 (q + 1)!
+  for (int q = 0; q <= NP_MAX; ++q) {
+    f *= q + 1;
+    T[TAB_KC + q] = c[q];
+    for (int i = 0; i < t.Qp; ++i)
+      T[TAB_KW + i * (NP_MAX + 1) + q] = (double)((long double)wp[i] * T[TAB_K + i * (NP_MAX + 1) + q] / (f * c[q]));
+  }
   for (int j = 0; j < t.Qxi; ++j) {
     T[TAB_XI + j] = xi[j];
     T[tab_xi2(t.Qp, t.Qxi) + j] = xi[j] * xi[j];

@@ -155,6 +155,19 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
 
+// d rounded to the nearest float, ties to even, by integer operations on its bits: a conversion instruction occupies
+// the FP64 pipe. |d| below 2^-126 gives zero.
+__device__ __forceinline__ float round_f32(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  const int e = (int)((hi >> 20) & 0x7FFu);
+  const unsigned sgn = hi & 0x80000000u;
+  if (e < 897) return __uint_as_float(sgn);
+  if (e >= 1151) return __uint_as_float(sgn | 0x7F800000u | (e == 2047 && ((hi & 0xFFFFFu) | lo) ? 1u : 0u));
+  const unsigned m = (((hi & 0x7FFFFFFFu) - (896u << 20)) << 3) | (lo >> 29), rest = lo << 3;
+  const unsigned up = rest > 0x80000000u || (rest == 0x80000000u && (m & 1u)) ? 1u : 0u;
+  return __uint_as_float(sgn | (m + up));  // a carry into the exponent is the right value, up to infinity
+}
+
 // acc += f (whi + wlo)
 __device__ __forceinline__ void df_add_prod(DF& acc, float f, float whi, float wlo) {
   const float p = __fmul_rn(f, whi);
@@ -360,6 +373,13 @@ __device__ __forceinline__ double df_join(float hi, float lo) {
   const unsigned add = (unsigned)__float2int_rn(__fmul_rn(l, __uint_as_float((top - ep) << 23))) + (down << 29);
   const unsigned wh = (p & 0x80000000u) | (((p & 0x7FFFFFFFu) >> 3) + (896u << 20)), wl = (p << 29) + add;
   return __hiloint2double((int)(wh + (wl < add ? 1u : 0u)), (int)wl);
+}
+
+// hi + lo of any double-float, as one double: normalised first (TwoSum), then joined.
+__device__ __forceinline__ double df_sum(float hi, float lo) {
+  float s, t;
+  two_sum(hi, lo, s, t);
+  return df_join(s, t);
 }
 
 // Indicators v_A, v_B, v_C of the pairs (x, y) = (d_j, d_{j+1}) in wind order, e the epsilon term:

@@ -13,9 +13,7 @@ bool gauss_legendre(int n, double* x, double* w);
 bool gauss_laguerre1(int n, double* x, double* w);
 double laguerre1(int l, double x);  // L^(1)_l(x)
 double legendre(int k, double x);   // P_k(x)
-// w^p_i (-1)^q sum_{l=q}^{Np} C(l,q) L^(1)_l(pbar_i) / (4 (q+1)!) at KW[i (Np + 1) + q], n radial nodes, evaluated at
-// the nodes in extended precision
-bool radial_factors(int n, int Np, long double* KW);
+
 }  // namespace rlbq
 
 namespace rlb {
@@ -71,13 +69,13 @@ constexpr int TAB_KW = TAB_K + QP_MAX * (NP_MAX + 1);
 constexpr int TAB_KC = TAB_KW + QP_MAX * (NP_MAX + 1);
 constexpr int TAB_XI = TAB_KC + NP_MAX + 1;
 // Scales c_q of the radial factors by (Qp, Np) = (3, 2), (4, 2), (4, 3): the collision applies the equilibrium in every
-// stage, so the rounding of these few constants is the part of its error that adds up over a run. Divided by c_q the
-// entries of one q all lie within 4e-18 of doubles (found by a search over k / 2^17), where the entries themselves
-// round by up to 1e-16; the per-cell factors g_q carry c_q.
+// stage, so the rounding of these few constants is the part of its error that adds up over a run. The products
+// w^p_i K[i][q] / (4 (q+1)!) of the tables' entries, divided by c_q, all lie within 5e-18 of doubles (found by a search
+// over k / 2^17), where they round by up to 1e-16 themselves; the per-cell factors g_q carry c_q.
 constexpr double RADIAL_SCALE[3][NP_MAX + 1] = {
-    {1.5519180297851562, 1.469573974609375, 1.5150070190429688, 1.0},
-    {1.5099411010742188, 1.9296340942382812, 1.1760940551757812, 1.0},
-    {1.0521774291992188, 1.4824142456054688, 1.3223495483398438, 1.790069580078125}};
+    {1.0260772705078125, 1.1634902954101562, 1.6391983032226562, 1.0},
+    {1.3723526000976562, 1.0144424438476562, 1.7607879638671875, 1.0},
+    {1.1395034790039062, 1.322998046875, 1.6575088500976562, 1.1712188720703125}};
 __host__ __device__ inline int tab_pw(int Qxi) { return TAB_XI + Qxi; }
 __host__ __device__ inline int tab_cxi(int Qxi) { return TAB_XI + Qxi + Qxi * (NV_MAX + 1); }
 __host__ __device__ inline int tab_eps(int Qxi) { return tab_cxi(Qxi) + 3 * Qxi; }

@@ -135,34 +135,6 @@ bool gauss_laguerre1(int n, double* x, double* w) {
   return true;
 }
 
-bool radial_factors(int n, int Np, long double* KW) {
-  std::vector<double> x(n), w(n);
-  if (!gauss_laguerre1(n, x.data(), w.data())) return false;
-  for (int i = 0; i < n; ++i) {
-    long double z = x[i], ln, ln1, l0, l1;
-    for (int it = 0; it < 4; ++it) {  // Newton steps beyond double precision: x L_n' = n L_n - (n + 1) L_{n-1}
-      laguerre1_pair(n, z, ln, ln1);
-      laguerre1_pair(n - 1, z, l0, l1);
-      z -= ln * z / (n * ln - (n + 1.0L) * l0);
-    }
-    laguerre1_pair(n + 1, z, ln, ln1);
-    const long double wz = z / ((n + 1.0L) * ln * ln);
-    long double f = 4.0L;
-    for (int q = 0; q <= Np; ++q) {
-      if (q > 0) f *= q + 1;
-      long double acc = 0.0L;
-      for (int l = q; l <= Np; ++l) {
-        long double C = 1.0L;
-        for (int u = 1; u <= q; ++u) C = C * (l - q + u) / u;
-        laguerre1_pair(l, z, ln, ln1);
-        acc += C * ln;
-      }
-      KW[i * (Np + 1) + q] = wz * (q % 2 ? -acc : acc) / f;
-    }
-  }
-  return true;
-}
-
 double laguerre1(int l, double x) {
   long double ln, ln1;
   laguerre1_pair(l, x, ln, ln1);

@@ -140,9 +140,9 @@ template <int KV>
 __device__ __forceinline__ void legendre_first(double beta, double b2, double g1, double (&h)[KV + 1]) {
   double C[KV + 2];
   {
-    // K = KV + 2 + 54 / -log2((1 - s)/(1 + s)), (1 - s)/(1 + s) = beta^2 / (1 + s)^2 (beta = 0: K = KV + 2)
+    // K = KV + 1 + 54 / -log2((1 - s)/(1 + s)), (1 - s)/(1 + s) = beta^2 / (1 + s)^2 (beta = 0: K = KV + 1)
     const float lr = 2.0f * __log2f(1.0f + sqrtf((float)g1)) - __log2f((float)b2);
-    const int K = min(KV + 2 + (int)(54.0f / lr), LEG_MAX);
+    const int K = min(KV + 1 + (int)(54.0f / lr), LEG_MAX);
     double c1 = 1.0, c2 = 0.0;  // c_k, c_{k+1}
     for (int k = K; k > KV + 1; --k) {
       const double c0 = fma(g_leg[k], b2 * c2, c1);
@@ -177,27 +177,26 @@ __device__ __forceinline__ void legendre_coeffs(double beta, double b2, double g
   for (int q = 1; q < NM; ++q) {
     const int m = q + 1;  // from m to m + 1
 #pragma unroll
-    for (int k = 0; k <= KV; ++k)
-      h[q][k] = fma(leg_lead(m, k), beta * h[q - 1][k == 0 ? 1 : k - 1], leg_own(m, k) * h[q - 1][k]);
+    for (int k = 0; k <= KV; ++k) {
+      const double b = beta * h[q - 1][k == 0 ? 1 : k - 1];
+      h[q][k] = leg_own(m, k) == 0.0   ? leg_lead(m, k) * b
+                : leg_lead(m, k) == 0.0 ? leg_own(m, k) * h[q - 1][k]
+                                        : fma(leg_lead(m, k), b, leg_own(m, k) * h[q - 1][k]);
+    }
   }
 }
 
-// The same times the per-cell factors of the equilibrium: ge[q][k] = c_q g_q h[q][k] (c_q: TAB_KC), so that
-//   F^eq_ij = sum_k B[i][k] w^xi_j P_k(xi_j),  B[i][k] = sum_q TAB_KW[i][q] ge[q][k]
+// Per-cell factors of the equilibrium: with g[q] = c_q (n/T) (T gamma)^q (c_q: TAB_KC) and h of legendre_coeffs,
+//   F^eq_ij = sum_k B[i][k] w^xi_j P_k(xi_j),  B[i][k] = sum_q (TAB_KW[i][q] g[q]) h[q][k]
 // (Eq. (feqtrunc): Laguerre generating function for the radial projection, Legendre projection of each
-// (1 - beta xi)^-m for the angular one; B = n/(4T^3) w^p_i sum_q s^(q+2) K[i][q] hhat_{q+2,k}, s = T/gamma, so
-// that g_q = (n/T) (T gamma)^q).
-template <int NPc, int NVc>
-__device__ __forceinline__ void cell_coeffs(const double* tab, double beta, double b2, double g1, double g0, double tg,
-                                            double (&ge)[NPc + 1][NVc + 1]) {
-  legendre_coeffs<NPc + 1, NVc>(beta, b2, g1, ge);
-  double g = g0;
+// (1 - beta xi)^-m for the angular one; B = n/(4T^3) w^p_i sum_q s^(q+2) K[i][q] hhat_{q+2,k}, s = T/gamma).
+template <int NPc>
+__device__ __forceinline__ void cell_factors(const double* tab, double g0, double tg, double (&g)[NPc + 1]) {
+  double t = g0;
 #pragma unroll
   for (int q = 0; q <= NPc; ++q) {
-    const double gq = g * tab[TAB_KC + q];
-#pragma unroll
-    for (int k = 0; k <= NVc; ++k) ge[q][k] *= gq;
-    g *= tg;
+    g[q] = t * tab[TAB_KC + q];
+    t *= tg;
   }
 }
 
@@ -222,46 +221,52 @@ __device__ __forceinline__ bool landau_frame(const double mom[5], double& beta, 
 }
 
 struct CoefSmem {
-  double ge[NP_MAX + 1][NV_MAX + 1][GW];  // cell_coeffs of the tile's cells
+  double h[NP_MAX + 1][NV_MAX + 1][GW];  // Legendre coefficients of the tile's cells
+  double g[NP_MAX + 1][GW];              // and their factors
 };
 
-// Per-cell coefficients of one cell into column c of cs.ge (all zero for a non-physical cell).
+// Coefficients and factors of one cell into column c of cs (all zero for a non-physical cell).
 template <int NPc, int NVc>
 __device__ __forceinline__ void store_cell_coeffs(const double* tab, bool ok, double beta, double b2, double g1, double g0, double tg,
                                                   CoefSmem& cs, int c) {
-  double ge[NPc + 1][NVc + 1];
+  double h[NPc + 1][NVc + 1], g[NPc + 1];
   if (ok) {
-    cell_coeffs<NPc, NVc>(tab, beta, b2, g1, g0, tg, ge);
+    legendre_coeffs<NPc + 1, NVc>(beta, b2, g1, h);
+    cell_factors<NPc>(tab, g0, tg, g);
   } else {
 #pragma unroll
-    for (int q = 0; q <= NPc; ++q)
+    for (int q = 0; q <= NPc; ++q) {
+      g[q] = 0.0;
 #pragma unroll
-      for (int k = 0; k <= NVc; ++k) ge[q][k] = 0.0;
+      for (int k = 0; k <= NVc; ++k) h[q][k] = 0.0;
+    }
   }
 #pragma unroll
-  for (int q = 0; q <= NPc; ++q)
+  for (int q = 0; q <= NPc; ++q) {
+    cs.g[q][c] = g[q];
 #pragma unroll
-    for (int k = 0; k <= NVc; ++k) cs.ge[q][k][c] = ge[q][k];
+    for (int k = 0; k <= NVc; ++k) cs.h[q][k][c] = h[q][k];
+  }
 }
 
-// B[i][k] of cell c from its ge[q][k].
+// B[i][k] of cell c.
 template <int NPc>
-__device__ __forceinline__ double row_coeff(const double* tab, int i, const double (*ge)[NV_MAX + 1][GW], int k, int c) {
+__device__ __forceinline__ double row_coeff(const double* tab, int i, const CoefSmem& cs, int k, int c) {
   const double* KW = tab + TAB_KW + i * (NP_MAX + 1);
-  double B = KW[0] * ge[0][k][c];
+  double B = (KW[0] * cs.g[0][c]) * cs.h[0][k][c];
 #pragma unroll
-  for (int q = 1; q <= NPc; ++q) B = fma(KW[q], ge[q][k][c], B);
+  for (int q = 1; q <= NPc; ++q) B = fma(KW[q] * cs.g[q][c], cs.h[q][k][c], B);
   return B;
 }
 
-// Fill B[i (NVc+1) + k][c] (radial rows i < Qp) for the TX cells of a tile from cs.ge: group g builds radial row
+// Fill B[i (NVc+1) + k][c] (radial rows i < Qp) for the TX cells of a tile from cs: group g builds radial row
 // i = g. Coefficients of w^xi_j P_k(xi_j).
 template <int NPc, int NVc>
 __device__ __forceinline__ void build_rows(const double* tab, int Qp, const CoefSmem& cs, double (*Bs)[GW]) {
   const int c = threadIdx.x % GW, i = threadIdx.x / GW;
   if (c >= TX || i >= Qp) return;
 #pragma unroll
-  for (int k = 0; k <= NVc; ++k) Bs[i * (NVc + 1) + k][c] = row_coeff<NPc>(tab, i, cs.ge, k, c);
+  for (int k = 0; k <= NVc; ++k) Bs[i * (NVc + 1) + k][c] = row_coeff<NPc>(tab, i, cs, k, c);
 }
 
 // Orders up to which the stage kernel evaluates the equilibrium as a polynomial in xi (two Horner chains in xi^2) from
@@ -412,7 +417,7 @@ __device__ __forceinline__ void cluster_coeffs(const StageArgs& A, const TubeDev
   if (own) {
     for (int w = tid >> lg; w < Qp * (NVc + 1); w += NT >> lg) {
       const int i = w / (NVc + 1), k = w - i * (NVc + 1);
-      sm.B[w][c] = row_coeff<NPc>(tab, i, sm.u.a.coef.ge, k, c);
+      sm.B[w][c] = row_coeff<NPc>(tab, i, sm.u.a.coef, k, c);
     }
   }
   __syncthreads();

@@ -111,22 +111,21 @@ __device__ __forceinline__ void cell_coeffs_rp(const TubeDev* Tg, const double* 
   if (ok && flag != nullptr && stiff(*Tg, beta)) atomicOr(flag + 1, RLB_WARN_STIFF);
   ok = ok && fabs(beta) <= beta_limit(NPc);
   if (!ok && flag) atomicOr(flag, 1);
-  double ge[NPc + 1][NVc + 1];
+  double h[NPc + 1][NVc + 1], g[NPc + 1];
 #pragma unroll
-  for (int q = 0; q <= NPc; ++q)
+  for (int q = 0; q <= NPc; ++q) {
+    g[q] = 0.0;
 #pragma unroll
-    for (int k = 0; k <= NVc; ++k) ge[q][k] = 0.0;
+    for (int k = 0; k <= NVc; ++k) h[q][k] = 0.0;
+  }
   if (ok) {
+    cell_factors<NPc>(tab, g0, tg, g);
     if (beta == 0.0) {
-      double g = g0, f = 1.0;  // h[q][0] = (q + 1)! at rest
+      double f = 1.0;  // h[q][0] = (q + 1)! at rest
 #pragma unroll
-      for (int q = 0; q <= NPc; ++q) {
-        f *= q + 1;
-        ge[q][0] = f * (g * tab[TAB_KC + q]);
-        g *= tg;
-      }
+      for (int q = 0; q <= NPc; ++q) h[q][0] = f *= q + 1;
     } else {
-      cell_coeffs<NPc, NVc>(tab, beta, b2, g1, g0, tg, ge);
+      legendre_coeffs<NPc + 1, NVc>(beta, b2, g1, h);
     }
   }
 #pragma unroll
@@ -134,19 +133,19 @@ __device__ __forceinline__ void cell_coeffs_rp(const TubeDev* Tg, const double* 
     if (i < Qp) {
       double KW[NPc + 1];
 #pragma unroll
-      for (int q = 0; q <= NPc; ++q) KW[q] = tab[TAB_KW + i * (NP_MAX + 1) + q];
+      for (int q = 0; q <= NPc; ++q) KW[q] = tab[TAB_KW + i * (NP_MAX + 1) + q] * g[q];
 #pragma unroll
       for (int k = 0; k <= NVc; ++k) {
-        double B = KW[0] * ge[0][k];
+        double B = KW[0] * h[0][k];
 #pragma unroll
-        for (int q = 1; q <= NPc; ++q) B = fma(KW[q], ge[q][k], B);
-        w.B[rp_brow(i, k, Qp, NVc + 1) * RP_WT + col] = (float)B;
+        for (int q = 1; q <= NPc; ++q) B = fma(KW[q], h[q][k], B);
+        w.B[rp_brow(i, k, Qp, NVc + 1) * RP_WT + col] = rlbdev::round_f32(B);
       }
     }
   }
   const double r0 = ok ? bdt_itau * gam : 0.0;
-  rt0 = (float)r0;
-  rt1 = ok ? (float)(r0 * beta) : 0.0f;
+  rt0 = rlbdev::round_f32(r0);
+  rt1 = ok ? rlbdev::round_f32(r0 * beta) : 0.0f;
 }
 
 // One velocity row as a lane holds it: its RP_C cells xl .. xl+3 (xl = x0 - RP_C + RP_C lane, so that lane 0
@@ -548,7 +547,7 @@ __device__ void warp_tile_rp(const StageArgsRP& A, const TubeDev& T, int x0, con
 #pragma unroll
         for (int f = 0; f < 5; ++f) {
           const float2 m = M[f * RP_WT + RP_C * lane + q];
-          A.Mout[f * A.nxtot + T.xoff + xl + q] = (double)m.x + (double)m.y;
+          A.Mout[f * A.nxtot + T.xoff + xl + q] = rlbdev::df_sum(m.x, m.y);
         }
       }
   }
