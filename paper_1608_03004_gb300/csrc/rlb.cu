@@ -1354,7 +1354,10 @@ rlb_status rlb_quadrature(int32_t Qp, int32_t Qxi, double* pbar, double* wp, dou
 // file-scope array instead; the existing stage kernel runs on it unchanged.
 namespace {
 
-static __device__ __align__(256) double g_static_scratch[RLB_STATIC_SCRATCH_BYTES / sizeof(double)];
+// STATIC_SLACK: the size limit is counted with the tile list and tables that tiles of 61 cells need (static_need), so
+// that the tubes it admits do not depend on the tile width; the list of the present tiles is at most 1 KB longer.
+constexpr size_t STATIC_SLACK = 2048;
+static __device__ __align__(256) double g_static_scratch[(RLB_STATIC_SCRATCH_BYTES + STATIC_SLACK) / sizeof(double)];
 
 std::mutex g_static_mu;
 double* g_static_addr[64] = {};
@@ -1378,6 +1381,12 @@ rlb_status static_setup(int dev, double** base) {
 
 size_t align256(size_t bytes) { return (bytes + 255) / 256 * 256; }
 
+// Bytes of the array that a tube is counted with.
+size_t static_need(size_t Qxi, size_t Q, size_t Nx) {
+  return align256(sizeof(TubeDev)) + align256(sizeof(int2) * ((Nx + 60) / 61)) + 256 +
+         align256(sizeof(double) * (28 + 13 * Qxi + 4 * Q)) + 2 * align256(sizeof(double) * Q * Nx);
+}
+
 }  // namespace
 
 extern "C" rlb_status rlb_step_static(const rlb_tube* tube, const double* F_in, double* F_out, int64_t nsteps,
@@ -1396,7 +1405,9 @@ extern "C" rlb_status rlb_step_static(const rlb_tube* tube, const double* F_in, 
   const size_t off_f1 = off_tab + align256(sizeof(double) * (size_t)tab_size(t.Qp, t.Qxi));
   const size_t stage_bytes = align256(sizeof(double) * (size_t)Q * (size_t)Nx);
   const size_t off_f2 = off_f1 + stage_bytes;
-  if (off_f2 + stage_bytes > (size_t)RLB_STATIC_SCRATCH_BYTES) return RLB_EINVAL;
+  if (static_need(t.Qxi, Q, Nx) > (size_t)RLB_STATIC_SCRATCH_BYTES ||
+      off_f2 + stage_bytes > (size_t)RLB_STATIC_SCRATCH_BYTES + STATIC_SLACK)
+    return RLB_EINVAL;
   if (nsteps == 0) return RLB_OK;
 
   cudaStream_t s = (cudaStream_t)stream;
