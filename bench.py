@@ -778,7 +778,7 @@ def run_gradient(args, specs, desc, rank, world, emit=True):
     backward_ms = sum(e[2].elapsed_time(e[3]) for e in ev)
     total_ms, record_ms, backward_ms = reduce_max_over_ranks([total_ms, record_ms, backward_ms], world)
     # the reverse sweep recomputes the recorded forward launches (unless the record kept the stage inputs),
-    # then runs 3 GRAD_STEPS adjoint launches
+    # then runs 3 GRAD_STEPS adjoint stages (two launches each)
     recompute_ms = record_ms if args.every < GRAD_STEPS else 0.0  # a kept record leaves nothing to recompute
     adj_launch_ms = max(backward_ms - recompute_ms, 1e-9) / (3 * GRAD_STEPS * args.steps)
 
@@ -836,7 +836,7 @@ def run_gradient(args, specs, desc, rank, world, emit=True):
                 "steps": e2e_steps, "api": "adjoint.run_fields (torch.autograd) from pinned host fields, "
                                           "gradients read back"},
         "clocks": clk,
-        "gpu_launches": 9 * GRAD_STEPS + 3,
+        "gpu_launches": 12 * GRAD_STEPS + 3,  # record, recompute: 3 per step; adjoint: 3 stages of 2 kernels
     }
     if not emit:
         return line
