@@ -9,11 +9,9 @@
 //   B. solves the Landau-frame eigenproblem T^mu_nu u^nu = -e u^mu for e, v, n and builds the per-cell
 //      coefficients of the truncated equilibrium of Eq. (feqtrunc);
 //   C. lets each of its four 64-thread groups walk mirror pairs of directions (xi_j, -xi_j) of one radial
-//      node: stages a row (tile + 3-cell halo, boundary condition folded into the load) in shared memory with
-//      its first differences and their squares, evaluates the WENO5 smoothness indicators once per pair of
-//      adjacent differences, combines three pairs into each of the 62 interface values and writes
-//      F_out = a F^n + b (F_in + dt L(F_in)), L = advection + Anderson-Witting collision (Eq. (Boltz)); the
-//      even and odd Legendre parts of the equilibrium serve both rows of a pair.
+//      node, both rows at once: first differences, WENO5 indicators once per pair of adjacent differences, three pairs
+//      combined into each of the 61 interface values, and F_out = a F^n + b (F_in + dt L(F_in)), L = advection +
+//      Anderson-Witting collision (Eq. (Boltz)); the parts of the equilibrium even and odd in xi serve both rows.
 // Tiles that cannot fill the GPU are split over several CTAs by velocity rows (StageArgs::split). The FP64
 // path is FP64 throughout; on GB300 the FP64 pipe (about 2 DFMA per SM per clock) bounds it, so the
 // arithmetic is arranged to spend as few FP64 instructions per velocity-node update as possible. The FP64
@@ -162,12 +160,11 @@ __global__ void __launch_bounds__(NT) rlb_init_kernel(InitArgs A) {
     init_tile<S, NP_MAX, NV_MAX>(A, T, tl.y, sm);
 }
 
-// FP64 view of a stored population without a conversion instruction, which would occupy the FP64 pipe (subnormal FP32
-// populations read as zero).
+// FP64 view of a stored population without a conversion instruction, which would occupy the FP64 pipe.
 __device__ __forceinline__ double ld_w(const double* p) { return __ldg(p); }
-__device__ __forceinline__ double ld_w(const float* p) { return rlbdev::df_widen(__ldg(p)); }
+__device__ __forceinline__ double ld_w(const float* p) { return rlbdev::widen_f32(__ldg(p)); }
 __device__ __forceinline__ double ld_w(const __nv_bfloat16* p) {
-  return rlbdev::df_widen(__uint_as_float((unsigned)__ldg(reinterpret_cast<const unsigned short*>(p)) << 16));
+  return rlbdev::widen_f32(__uint_as_float((unsigned)__ldg(reinterpret_cast<const unsigned short*>(p)) << 16));
 }
 
 // Fields of every cell: the five moments summed over F in FP64, or, with M != NULL, read from M for tubes with

@@ -352,6 +352,20 @@ __device__ __forceinline__ double df_widen(float f) {
   return ef == 0u ? 0.0 : w;
 }
 
+// The double equal to any float (subnormals, infinities and NaN too), by integer operations.
+__device__ __forceinline__ double widen_f32(float f) {
+  const unsigned b = __float_as_uint(f), sgn = b & 0x80000000u;
+  unsigned ef = (b >> 23) & 0xFFu, m = b & 0x7FFFFFu;
+  if (ef == 255u) {
+    ef = 1151u;  // the double's exponent field is 2047
+  } else if (ef == 0u) {
+    if (m == 0u) return __hiloint2double((int)sgn, 0);
+    const int s = __clz(m) - 8;  // normalise: the leading bit to bit 23
+    return __hiloint2double((int)(sgn | ((unsigned)(897 - s) << 20) | (((m << s) >> 3) & 0xFFFFFu)), (int)((m << s) << 29));
+  }
+  return __hiloint2double((int)(sgn | ((ef + 896u) << 20) | (m >> 3)), (int)(m << 29));
+}
+
 // hi + lo of a normalised double-float (|lo| <= ulp(hi)/2) as one double, rounded at its 53rd bit: an addition on the
 // bits of hi widened, in place of an FP64 operation that widens lo on its own. Where lo points toward zero, the float
 // next to hi is widened and lo is added to 2^29 units of that double's last place, so that the sum never leaves the

@@ -414,7 +414,15 @@ __device__ __forceinline__ void cluster_coeffs(const StageArgs& A, const TubeDev
   if ((tid >> 5) == (part & 3) && (tid & 31) < share && c0 + (tid & 31) < TX)
     cell_phase<NPc, NVc>(A, T, tab, x0 + c0 + (tid & 31) < Nx, c0 + (tid & 31), sm);
   __syncthreads();
-  if (own) {
+  // B[i][k], a thread per radial row where the share fills the warps (the factors KW g once per row: 2 % of a launch on
+  // 13 uneven tubes), else a thread per coefficient
+  if (own && share > 8) {
+    if ((tid >> lg) < Qp) {
+#pragma unroll
+      for (int k = 0; k <= NVc; ++k)
+        sm.B[(tid >> lg) * (NVc + 1) + k][c] = row_coeff<NPc>(tab, tid >> lg, sm.u.a.coef, k, c);
+    }
+  } else if (own) {
     for (int w = tid >> lg; w < Qp * (NVc + 1); w += NT >> lg) {
       const int i = w / (NVc + 1), k = w - i * (NVc + 1);
       sm.B[w][c] = row_coeff<NPc>(tab, i, sm.u.a.coef, k, c);
