@@ -52,11 +52,9 @@ struct AdjCoef {
   double dh[NP_MAX + 1][NV_MAX + 1][GW];
 };
 
-// hhat and d hhat/d beta of the tile's cells, one thread per cell; cells with ok == 0 keep zeros. With
-// Bs != nullptr, group i then builds the equilibrium coefficients B[i][k] as the forward does. Ends with a barrier.
+// hhat and d hhat/d beta of the tile's cells, one thread per cell; cells with ok == 0 keep zeros. Ends with a barrier.
 template <int NPc, int NVc>
-__device__ void tile_coeffs_d(const double* tab, int Qp, const double* cellv /* n, T, beta: [3][GW] */,
-                              int* ok, AdjCoef& co, double (*Bs)[GW], int* flag) {
+__device__ void tile_coeffs_d(const double* cellv /* n, T, beta: [3][GW] */, int* ok, AdjCoef& co, int* flag) {
   const int c = threadIdx.x % GW, g = threadIdx.x / GW;
   if (g == 0 && c < TXA) {
     const double beta = cellv[2 * GW + c];
@@ -86,30 +84,6 @@ __device__ void tile_coeffs_d(const double* tab, int Qp, const double* cellv /* 
       for (int m = 0; m <= NPc; ++m)
 #pragma unroll
         for (int k = 0; k <= NVc; ++k) co.hh[m][k][c] = co.dh[m][k][c] = 0.0;
-    }
-  }
-  __syncthreads();
-  if (Bs != nullptr && c < TXA) {
-    const int i = g;
-    double B[NVc + 1];
-#pragma unroll
-    for (int k = 0; k <= NVc; ++k) B[k] = 0.0;
-    if (i < Qp && ok[c]) {
-      const double n = cellv[c], T = cellv[GW + c], beta = cellv[2 * GW + c];
-      const double s = T * sqrt(1.0 - beta * beta);
-      const double pref = n / (4.0 * T * T * T) * tab[TAB_WP + i];
-      double sq = s * s;
-#pragma unroll
-      for (int q = 0; q <= NPc; ++q) {
-        const double G = pref * sq * tab[TAB_K + i * (NP_MAX + 1) + q];
-#pragma unroll
-        for (int k = 0; k <= NVc; ++k) B[k] = fma(G, co.hh[q][k][c], B[k]);
-        sq *= s;
-      }
-    }
-    if (i < QP_MAX) {
-#pragma unroll
-      for (int k = 0; k <= NVc; ++k) Bs[i * (NV_MAX + 1) + k][c] = B[k];
     }
   }
   __syncthreads();
@@ -787,7 +761,7 @@ __device__ void init_vjp_tile(const TubeDev& T, const double* tab, int x0, const
     sm.ok[c] = ok ? 1 : 0;
   }
   __syncthreads();
-  tile_coeffs_d<NPc, NVc>(tab, T.Qp, &sm.cellv[0][0], sm.ok, sm.co, nullptr, flag);
+  tile_coeffs_d<NPc, NVc>(&sm.cellv[0][0], sm.ok, sm.co, flag);
   // Lam[i][k] = sum_j dL/dF_ij w^xi_j P_k(xi_j), radial row i summed by group i
   if (g < QP_MAX) {
     double lam[NVc + 1];
