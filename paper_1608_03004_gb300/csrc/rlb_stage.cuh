@@ -206,14 +206,24 @@ __device__ __forceinline__ void cell_factors(const double* tab, double g0, doubl
 // FP64 operations instead of 150. Returns false if non-physical.
 __device__ __forceinline__ bool landau_frame(const double mom[5], double& beta, double& b2, double& g1, double& gam,
                                              double& g0, double& tg) {
-  const double A = mom[2] + mom[4], B2 = 2.0 * mom[3];
-  const double disc = fma(A, A, -(B2 * B2));
-  const double e = 0.5 * ((mom[2] - mom[4]) + rlbdev::sqrt_nr(disc));
-  beta = rlbdev::div_nr(mom[3], mom[4] + e);
-  b2 = beta * beta;
-  g1 = fma(-beta, beta, 1.0);
-  gam = rlbdev::rsqrt_nr(g1);
-  const double n = gam * fma(-beta, mom[1], mom[0]);
+  const double A = mom[2] + mom[4];
+  double disc = 1.0, e, n;
+  if (((unsigned long long)__double_as_longlong(mom[3]) << 1) == 0ull) {
+    // at rest (T0x = 0, exactly so wherever the state is symmetric in xi): sqrt(A^2) = |A|, beta = 0
+    e = 0.5 * ((mom[2] - mom[4]) + fabs(A));
+    beta = b2 = 0.0;
+    g1 = gam = 1.0;
+    n = mom[0];
+  } else {
+    const double B2 = 2.0 * mom[3];
+    disc = fma(A, A, -(B2 * B2));
+    e = 0.5 * ((mom[2] - mom[4]) + rlbdev::sqrt_nr(disc));
+    beta = rlbdev::div_nr(mom[3], mom[4] + e);
+    b2 = beta * beta;
+    g1 = fma(-beta, beta, 1.0);
+    gam = rlbdev::rsqrt_nr(g1);
+    n = gam * fma(-beta, mom[1], mom[0]);
+  }
   const double n3 = 3.0 * n;
   g0 = n3 * (n * rlbdev::rcp_nr(e));
   tg = (e * rlbdev::rcp_nr(n3)) * gam;
