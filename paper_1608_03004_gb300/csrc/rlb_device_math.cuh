@@ -156,12 +156,19 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 }
 
 // d rounded to the nearest float, ties to even, by integer operations on its bits: a conversion instruction occupies
-// the FP64 pipe. |d| below 2^-126 gives zero.
+// the FP64 pipe. As a conversion does, it keeps FP32's subnormals (coefficients of a thin gas lie there).
 __device__ __forceinline__ float round_f32(double d) {
   const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
   const int e = (int)((hi >> 20) & 0x7FFu);
   const unsigned sgn = hi & 0x80000000u;
-  if (e < 897) return __uint_as_float(sgn);
+  if (e < 897) {  // below 2^-126: units of 2^-149 (e < 873: below half of one)
+    if (e < 873) return __uint_as_float(sgn);
+    const unsigned long long sig = ((unsigned long long)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo;
+    const int s = 926 - e;  // 30 .. 53
+    const unsigned q = (unsigned)(sig >> s);
+    const unsigned long long rest = sig << (64 - s), half = 1ull << 63;
+    return __uint_as_float(sgn | (q + (rest > half || (rest == half && (q & 1u)) ? 1u : 0u)));
+  }
   if (e >= 1151) return __uint_as_float(sgn | 0x7F800000u | (e == 2047 && ((hi & 0xFFFFFu) | lo) ? 1u : 0u));
   const unsigned m = (((hi & 0x7FFFFFFFu) - (896u << 20)) << 3) | (lo >> 29), rest = lo << 3;
   const unsigned up = rest > 0x80000000u || (rest == 0x80000000u && (m & 1u)) ? 1u : 0u;
