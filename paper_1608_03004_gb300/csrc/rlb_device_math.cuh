@@ -396,11 +396,12 @@ __device__ __forceinline__ double df_join(float hi, float lo) {
   return __hiloint2double((int)(wh + (wl < add ? 1u : 0u)), (int)wl);
 }
 
-// hi + lo of any double-float, as one double: normalised first (TwoSum), then joined.
+// hi + lo of any double-float, as one double: normalised first (TwoSum), then joined. A sum below 2^-126 is exact in
+// its high part, and df_join would drop it.
 __device__ __forceinline__ double df_sum(float hi, float lo) {
   float s, t;
   two_sum(hi, lo, s, t);
-  return df_join(s, t);
+  return ((__float_as_uint(s) >> 23) & 0xFFu) == 0u ? widen_f32(s) : df_join(s, t);
 }
 
 // Indicators v_A, v_B, v_C of the pairs (x, y) = (d_j, d_{j+1}) in wind order, e the epsilon term:

@@ -8,6 +8,7 @@ __global__ void small_kernel(int which, const double* a, const double* b, double
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   if (which == 0) out[i] = (double)rlbdev::round_f32(a[i]);
+  if (which == 1) out[i] = rlbdev::df_sum((float)a[i], (float)b[i]);
 }
 
 extern "C" int sv_eval(int which, const double* a, const double* b, double* out, int n) {

@@ -89,3 +89,21 @@ def test_thin_gas_relaxes_to_its_equilibrium(storage, Qp, exp, v):
     got, tol = relax(storage, Qp, 2.0**exp, v)
     ref, _ = relax(storage, Qp, 1.0, v)
     assert np.all(np.abs(got - ref) <= tol), (got, ref, tol)
+
+
+def test_sum_of_a_double_float_keeps_subnormals(shim):
+    """hi + lo, exact in FP64: within its last place for a normal high part, exact below 2^-126."""
+    rng = np.random.default_rng(8)
+    u = rng.integers(-(2**23), 2**23, 20000) * 2.0**-149  # subnormal, and zero
+    hi = np.concatenate([u, [0.0, -0.0, 2.0**-149, -(2.0**-149), 2.0**-126 - 2.0**-149], 2.0**-126 * rng.uniform(1, 4, 5000)])
+    hi = hi.astype(np.float32).astype(np.float64)
+    lo = rng.integers(-4, 5, hi.size) * 2.0**-149
+    np.testing.assert_allclose(shim(1, hi, lo), hi + lo, rtol=2.0**-52, atol=0)
+
+
+@pytest.mark.parametrize("Qp,exp,v", [(3, -128, 0.0), (3, -128, 0.3), (3, -124, 0.02), (3, -120, 0.0), (4, -120, 0.0)])
+def test_moments_below_the_normal_range(Qp, exp, v):
+    """The moments that a step leaves for the next one (N^0 below 2^-126, or the N^x and T^0x of a slow gas)."""
+    got, tol = relax(rb.STORAGE_F32, Qp, 2.0**exp, v)
+    ref, _ = relax(rb.STORAGE_F32, Qp, 1.0, v)
+    assert np.all(np.abs(got - ref) <= tol), (got, ref, tol)
