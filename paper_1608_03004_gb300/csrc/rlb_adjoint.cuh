@@ -131,7 +131,7 @@ struct LandauRev {
 __device__ __forceinline__ bool landau_keep(const double mom[5], LandauRev& L) {
   const double A = mom[2] + mom[4], B2 = 2.0 * mom[3];
   const double disc = fma(A, A, -(B2 * B2));
-  L.isq = rlbdev::rsqrt_nr(disc);
+  L.isq = rlbdev::rsqrt_any(disc);
   L.e = 0.5 * ((mom[2] - mom[4]) + rlbdev::sqrt_nr(disc));
   L.iden = rlbdev::rcp_nr(mom[4] + L.e);
   L.beta = rlbdev::div_nr(mom[3], mom[4] + L.e);

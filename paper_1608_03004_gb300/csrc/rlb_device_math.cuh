@@ -34,9 +34,15 @@ __device__ __forceinline__ double rsqrt_nr(double x) {
   return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
+// rsqrt_nr for subnormal x too, which the hardware approximation would take as zero: scaled by 2^106.
+__device__ __forceinline__ double rsqrt_any(double x) {
+  if ((unsigned)__double2hiint(x) >= 0x100000u) return rsqrt_nr(x);
+  return rsqrt_nr(x * 0x1p106) * 0x1p53;
+}
+
 // sqrt(x) for x >= 0 (0 gives 0): x rsqrt(x) and one Newton-Raphson correction from the remainder x - s^2.
 __device__ __forceinline__ double sqrt_nr(double x) {
-  const double y = rsqrt_nr(x), s = x * y;
+  const double y = rsqrt_any(x), s = x * y;
   const double r = fma(fma(-s, s, x), 0.5 * y, s);
   return x == 0.0 ? 0.0 : r;
 }

@@ -9,6 +9,7 @@ __global__ void small_kernel(int which, const double* a, const double* b, double
   if (i >= n) return;
   if (which == 0) out[i] = (double)rlbdev::round_f32(a[i]);
   if (which == 1) out[i] = rlbdev::df_sum((float)a[i], (float)b[i]);
+  if (which == 2) out[i] = rlbdev::sqrt_nr(a[i]);
 }
 
 extern "C" int sv_eval(int which, const double* a, const double* b, double* out, int n) {
