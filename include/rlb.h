@@ -233,9 +233,12 @@ rlb_status rlb_quadrature(int32_t Qp, int32_t Qxi, double *pbar, double *wp, dou
  *   order:        tile order, RLB_ORDER_COST (most expensive tubes first, the default) or RLB_ORDER_INTERLEAVE
  *                 (tubes interleaved tile by tile).
  *   split:        work items per tile of the FP64 stage kernel: item k advances velocity rows [k Q / split,
- *                 (k + 1) Q / split) of the tile after reducing its moments over all rows. 0 (the default)
- *                 chooses: one item per tile when the tiles fill the GPU's resident CTA slots, else
- *                 min(8, slots / tiles). 1 <= split <= 8 fixes it. Handles with reduced storage use one.
+ *                 (k + 1) Q / split) of the tile. With RLB_SCHED_TILE the items of a tile are a thread-block
+ *                 cluster and share its moments and coefficients; the persistent schedules repeat them in each
+ *                 item. 0 (the default) chooses: with RLB_SCHED_TILE the split that ends a launch earliest, by
+ *                 handing the tiles to the GPU's resident CTA slots in order (1 from 8 times the slots on); with
+ *                 the others one item per tile when the tiles fill the slots, else min(8, slots / tiles).
+ *                 1 <= split <= 8 fixes it for every schedule. Handles with reduced storage use one.
  */
 enum { RLB_SCHED_TILE = 0, RLB_SCHED_STRIDE = 1, RLB_SCHED_COUNTER = 2 };
 enum { RLB_ORDER_COST = 0, RLB_ORDER_INTERLEAVE = 1 };
@@ -253,9 +256,10 @@ rlb_status rlb_set_launch(rlb_handle h, const rlb_launch *cfg);
 
 /*
  * rlb_autotune - time every launch shape (schedules x ctas_per_sm in {occupancy, 1, 2} x both tile orders x
- *   graph on/off x split automatic or 1 where the automatic choice is not 1) for trial_steps steps on the handle's own tubes and state, keep the fastest. The state is
- *   saved first and restored after every trial, so the handle's state is unchanged on return. best and
- *   best_ms_per_step (either may be NULL) receive the choice and its time per step. Synchronous.
+ *   graph on/off x split automatic or 1 where the schedule's automatic choice is not 1) for trial_steps steps on
+ *   the handle's own tubes and state, keep the fastest. The state is saved first and restored after every
+ *   trial, so the handle's state is unchanged on return. best and best_ms_per_step (either may be NULL) receive
+ *   the choice and its time per step. Synchronous.
  */
 rlb_status rlb_autotune(rlb_handle h, int32_t trial_steps, rlb_launch *best, double *best_ms_per_step);
 

@@ -384,8 +384,9 @@ struct rlb_ctx {
   // launch shape, CUDA graph of graph_steps steps, work counters of the counter schedule
   rlb_launch cfg = {RLB_SCHED_TILE, 0, 0, RLB_ORDER_COST, 0};
   int occupancy = 1;           // resident CTAs per SM of the stage kernel
-  int split = 1;               // automatic FP64 stage work items per tile (several when the tiles cannot fill
-                               // the GPU); rlb_launch.split overrides it
+  int split = 1;               // automatic FP64 stage work items per tile, one-CTA-per-tile schedule (choose_split)
+  int psplit = 1;              // the same for the persistent schedules (several only when the tiles cannot fill the
+                               // GPU); rlb_launch.split overrides both
   int asplit = 1;              // adjoint work items per adjoint tile
   int nsm = 1;
   cudaStream_t gstream = nullptr;
@@ -418,10 +419,14 @@ namespace {
 constexpr int GRAPH_MAX = 64;  // longest captured graph, in steps
 constexpr int SPLIT_MAX = 8;   // most work items per tile
 
-// Work items per tile of the FP64 stage kernel for the handle's launch shape.
-int eff_split(const rlb_ctx* h) {
+// Work items per tile of the FP64 stage kernel for a launch with this schedule. The items of a persistent launch each
+// repeat their tile's moments and coefficients, so its automatic split stays 1 once the tiles fill the resident slots.
+// On GB300, stride schedule, 500 tiles of 384 rows: 1.94 ms per step with choose_split's 5 items per tile, 1.47 with
+// one (the cluster launch, which shares that work: 1.15 and 1.39); 1000 tiles of 96 rows: 0.88 and 0.69.
+int eff_split(const rlb_ctx* h, int schedule) {
   if (h->storage != RLB_STORAGE_F64) return 1;
-  return h->cfg.split > 0 ? h->cfg.split : h->split;
+  if (h->cfg.split > 0) return h->cfg.split;
+  return schedule == RLB_SCHED_TILE ? h->split : h->psplit;
 }
 
 void free_ctx(rlb_ctx* h) {
@@ -732,7 +737,11 @@ rlb_status create(rlb_handle* out, const rlb_tube* tubes, int32_t ntubes, const 
     RLB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&h->occupancy, rlb_stage_rp_kernel<__nv_bfloat16, 1>, RP_NT,
                                                            rp_smem_bytes(h->brows)));
   if (h->occupancy < 1) h->occupancy = 1;
-  if (h->storage == RLB_STORAGE_F64) h->split = choose_split(h->tubes, tiles, h->nsm * h->occupancy);
+  if (h->storage == RLB_STORAGE_F64) {
+    const int slots = h->nsm * h->occupancy;
+    h->split = choose_split(h->tubes, tiles, slots);
+    if (h->ntiles < slots) h->psplit = std::min(SPLIT_MAX, slots / h->ntiles);
+  }
   return RLB_OK;
 }
 
@@ -874,7 +883,7 @@ rlb_status launch_stage(rlb_ctx* h, cudaStream_t stream, int st, int* ctr) {
   const void* in[3] = {h->F, h->F1, h->F2};
   void* out[3] = {h->F1, h->F2, h->F};
   const int sched = h->cfg.schedule;
-  const int split = eff_split(h);
+  const int split = eff_split(h, sched);
   // work items: tiles (times the split) of the FP64 kernel, groups of RP_WARPS warp tiles otherwise
   const int items = h->storage == RLB_STORAGE_F64 ? h->ntiles * split : (h->nwt + RP_WARPS - 1) / RP_WARPS;
   const int grid = sched == RLB_SCHED_TILE
@@ -1103,9 +1112,10 @@ rlb_status rlb_autotune(rlb_handle h, int32_t trial_steps, rlb_launch* best, dou
   rlb_status st = cuda_status(e);
   const int scheds[7][2] = {{RLB_SCHED_TILE, 0}, {RLB_SCHED_STRIDE, 0}, {RLB_SCHED_STRIDE, 1}, {RLB_SCHED_STRIDE, 2},
                             {RLB_SCHED_COUNTER, 0}, {RLB_SCHED_COUNTER, 1}, {RLB_SCHED_COUNTER, 2}};
-  const int nsplit = (h->storage == RLB_STORAGE_F64 && h->split > 1) ? 2 : 1;  // automatic, and 1 if different
   for (int order = 0; order < 2 && st == RLB_OK; ++order)
-    for (int k = 0; k < 7 && st == RLB_OK; ++k)
+    for (int k = 0; k < 7 && st == RLB_OK; ++k) {
+      const int automatic = scheds[k][0] == RLB_SCHED_TILE ? h->split : h->psplit;
+      const int nsplit = (h->storage == RLB_STORAGE_F64 && automatic > 1) ? 2 : 1;  // automatic, and 1 if different
       for (int graph = 0; graph < 2 && st == RLB_OK; ++graph)
         for (int sp = 0; sp < nsplit && st == RLB_OK; ++sp) {
           const rlb_launch c = {scheds[k][0], scheds[k][1], graph ? trial_steps : 0, order, sp};
@@ -1124,6 +1134,7 @@ rlb_status rlb_autotune(rlb_handle h, int32_t trial_steps, rlb_launch* best, dou
           }
           if (st == RLB_OK) st = cuda_status(restore());
         }
+    }
   if (st == RLB_OK) st = rlb_set_launch(h, &win);
   else rlb_set_launch(h, &start);
   if (t0) cudaEventDestroy(t0);
@@ -1496,7 +1507,7 @@ rlb_status launch_stage_ptrs(rlb_ctx* h, int st, const double* Fn, const double*
   A.ntiles = h->ntiles;
   A.schedule = RLB_SCHED_TILE;
   A.counter = h->d_counters;
-  A.split = eff_split(h);
+  A.split = eff_split(h, RLB_SCHED_TILE);
   return launch_tiles(A, h->stage_smem, h->stream);
 }
 
