@@ -27,10 +27,8 @@
 #include <cstddef>
 #include <complex>
 #include <cstring>
-#include <functional>
 #include <map>
 #include <mutex>
-#include <queue>
 #include <type_traits>
 #include <new>
 #include <utility>
@@ -39,6 +37,7 @@
 #include "../../include/rlb.h"
 #include "rlb_device_math.cuh"
 #include "rlb_internal.h"
+#include "rlb_schedule.h"
 
 using namespace rlb;
 
@@ -417,7 +416,6 @@ struct rlb_ctx {
 namespace {
 
 constexpr int GRAPH_MAX = 64;  // longest captured graph, in steps
-constexpr int SPLIT_MAX = 8;   // most work items per tile
 
 // Work items per tile of the FP64 stage kernel for a launch with this schedule. The items of a persistent launch each
 // repeat their tile's moments and coefficients, so its automatic split stays 1 once the tiles fill the resident slots.
@@ -557,38 +555,15 @@ rlb_status validate(const rlb_tube* t) {
   return RLB_OK;
 }
 
-// Work items per tile of the FP64 stage kernel. The velocity rows of a tile are split over several CTAs where that
-// shortens the launch: for each split the tiles, in their order, are handed to `slots` resident CTAs as they come
-// free, an item costing its rows plus a fixed part worth ROW0 rows (the per-cell chain, barriers and start-up: 12 to 16
-// us on GB300, where a CTA takes 0.6 us per row), and the split with the earliest end is taken. Handles of
-// many times the slots are never split. Against "split only what cannot fill the slots": 13 uneven tubes, 545
-// tiles of 16 to 288 rows for 456 slots, 137 -> 115 us per stage.
-int choose_split(const std::vector<rlb_tube>& tubes, const std::vector<int2>& tiles, int slots) {
-  constexpr int ROW0 = 20;
-  const long long n = (long long)tiles.size();
-  if (n >= 8LL * slots) return 1;
-  int best = 1;
-  double best_end = -1.0;
-  for (int s = 1; s <= SPLIT_MAX; ++s) {
-    std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
-    double end = 0.0;
-    for (const int2& t : tiles)
-      for (int k = 0; k < s; ++k) {
-        double at = 0.0;
-        if ((long long)free_at.size() >= slots) {
-          at = free_at.top();
-          free_at.pop();
-        }
-        at += ROW0 + (double)tubes[t.x].Qp * tubes[t.x].Qxi / s;
-        end = std::max(end, at);
-        free_at.push(at);
-      }
-    if (best_end < 0.0 || end < best_end) {
-      best_end = end;
-      best = s;
-    }
+// The tiles of a launch as runs of equally many velocity rows.
+std::vector<TileRun> tile_runs(const std::vector<rlb_tube>& tubes, const std::vector<int2>& tiles) {
+  std::vector<TileRun> runs;
+  for (const int2& t : tiles) {
+    const double rows = (double)tubes[t.x].Qp * tubes[t.x].Qxi;
+    if (runs.empty() || runs.back().rows != rows) runs.push_back({rows, 0});
+    ++runs.back().tiles;
   }
-  return best;
+  return runs;
 }
 
 rlb_status create(rlb_handle* out, const rlb_tube* tubes, int32_t ntubes, const double* xleft, void* stream,
@@ -739,7 +714,7 @@ rlb_status create(rlb_handle* out, const rlb_tube* tubes, int32_t ntubes, const 
   if (h->occupancy < 1) h->occupancy = 1;
   if (h->storage == RLB_STORAGE_F64) {
     const int slots = h->nsm * h->occupancy;
-    h->split = choose_split(h->tubes, tiles, slots);
+    h->split = choose_split(tile_runs(h->tubes, tiles), slots);
     if (h->ntiles < slots) h->psplit = std::min(SPLIT_MAX, slots / h->ntiles);
   }
   return RLB_OK;
