@@ -495,13 +495,17 @@ bool fill_tube_tables(const rlb_tube& t, double* pb, double* wp, double* xi, dou
       T[TAB_K + i * (NP_MAX + 1) + q] = (double)((q % 2) ? -acc : acc);
     }
   }
-  const double* c = RADIAL_SCALE[t.Qp == 3 ? 0 : t.Np - 1];
+  const int orders = t.Qp == 3 ? 0 : t.Np - 1;
+  const double* c = RADIAL_SCALE[orders];
   long double f = 4.0L;  // 4 (q + 1)!
   for (int q = 0; q <= NP_MAX; ++q) {
     f *= q + 1;
     T[TAB_KC + q] = c[q];
-    for (int i = 0; i < t.Qp; ++i)
+    T[TAB_KCA + q] = RADIAL_ADJ[orders].c[q];
+    for (int i = 0; i < t.Qp; ++i) {
       T[TAB_KW + i * (NP_MAX + 1) + q] = (double)((long double)wp[i] * T[TAB_K + i * (NP_MAX + 1) + q] / (f * c[q]));
+      T[TAB_KWA + i * (NP_MAX + 1) + q] = RADIAL_ADJ[orders].k[i][q];
+    }
   }
   for (int j = 0; j < t.Qxi; ++j) {
     T[TAB_XI + j] = xi[j];

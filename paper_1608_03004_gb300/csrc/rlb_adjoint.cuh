@@ -308,7 +308,7 @@ __device__ void adjoint_cells(const AdjArgs& A, const TubeDev& T, int tile, int 
         const double h = sm.h[q][sl][c];
         d = c_leg.hi[sl] * sm.h[q + 1][sl + 1][c];
         if (sl > 0) d = fma(c_leg.lo[sl], sm.h[q + 1][sl - 1][c], d);
-        const double gq = g * tab[TAB_KC + q];
+        const double gq = g * tab[TAB_KCA + q];
         a = gq * h;
         d = (gq * u) * fma(-(double)(q + 2) * beta, h, d);
       }
@@ -323,7 +323,7 @@ __device__ void adjoint_cells(const AdjArgs& A, const TubeDev& T, int tile, int 
     double B = 0.0, BT = 0.0, Bb = 0.0;
 #pragma unroll
     for (int q = 0; q <= NPc; ++q) {
-      const double K = tab[TAB_KW + r * (NP_MAX + 1) + q], t = K * sm.ga[q][k][c];
+      const double K = tab[TAB_KWA + r * (NP_MAX + 1) + q], t = K * sm.ga[q][k][c];
       B += t;
       BT = fma((double)(q - 1), t, BT);
       Bb = fma(K, sm.gb[q][k][c], Bb);

@@ -54,6 +54,7 @@ struct TubeDev {
 //                                               s^(q+2) hhat_{q+2,k} in the truncated equilibrium
 //   then KW[i][q] = w^p_i K[i][q] / (4 (q+1)! c_q) at [i (NP_MAX+1) + q]: the same with the factors that the
 //                                               per-cell coefficients take out (legendre_coeffs), and c_q (NP_MAX+1)
+//   then both again as the adjoint takes them (RADIAL_ADJ)
 //   then xi_j (Qxi), then w^xi_j P_k(xi_j) at [j (NV_MAX+1) + k] (Qxi (NV_MAX+1)), zero for k > Nv,
 //   then b_st dt xi_j / dx at [st Qxi + j] for the three Runge-Kutta stages, b = (1, 1/4, 2/3),
 //   then per velocity s = i Qxi + j the WENO5 epsilon term e = 3 eps ws^2, ws = w^p_i w^xi_j / 2 (the limiter acts on
@@ -67,7 +68,9 @@ constexpr int TAB_WP = 2 * QP_MAX;
 constexpr int TAB_K = 3 * QP_MAX;
 constexpr int TAB_KW = TAB_K + QP_MAX * (NP_MAX + 1);
 constexpr int TAB_KC = TAB_KW + QP_MAX * (NP_MAX + 1);
-constexpr int TAB_XI = TAB_KC + NP_MAX + 1;
+constexpr int TAB_KWA = TAB_KC + NP_MAX + 1;
+constexpr int TAB_KCA = TAB_KWA + QP_MAX * (NP_MAX + 1);
+constexpr int TAB_XI = TAB_KCA + NP_MAX + 1;
 // Scales c_q of the radial factors by (Qp, Np) = (3, 2), (4, 2), (4, 3): the collision applies the equilibrium in every
 // stage, so the rounding of these few constants is the part of its error that adds up over a run. The products
 // w^p_i K[i][q] / (4 (q+1)!) of the tables' entries, divided by c_q, all lie within 5e-18 of doubles (found by a search
@@ -76,6 +79,31 @@ constexpr double RADIAL_SCALE[3][NP_MAX + 1] = {
     {1.0260772705078125, 1.1634902954101562, 1.6391983032226562, 1.0},
     {1.3723526000976562, 1.0144424438476562, 1.7607879638671875, 1.0},
     {1.1395034790039062, 1.322998046875, 1.6575088500976562, 1.1712188720703125}};
+// The adjoint's radial factors, (c_q; K[i][q]) for the same three orders: K[i][q] c_q is w^p_i K[i][q] / (4 (q+1)!) of the
+// exact rule within 3 units of 2^-53. They are doubles next to those values, found by a search over c_q = k / 2^12, whose
+// sums with the doubles of pbar_i and pbar_i^2 meet the conditions under which the equilibrium keeps N^0 and T^00, each
+// order to 5e-18 (three nodes: 1.5e-18). The gradient in log(tau) is a sum of collision terms that cancel to 1e-5 of
+// themselves, and a bias of the equilibrium in these moments is what is left of it: with the factors above, which leave
+// 6e-17 (three nodes) to 2e-16 (four), that gradient of a 2048-cell inverse problem was 1.1e-11 to 3.2e-10 off (against
+// extended precision, six inputs), with these 2.7e-12 to 5.8e-11.
+struct RadialAdj {
+  double c[NP_MAX + 1], k[QP_MAX][NP_MAX + 1];
+};
+constexpr RadialAdj RADIAL_ADJ[3] = {
+    {{1.7470703125, 1.785888671875, 1.6513671875, 1.0},
+     {{0.22698812067910754, -0.09579887087265786, 0.00936379671476203},
+      {-0.09845901057459167, 0.11533854013180392, -0.014346168879678392},
+      {0.014567591963678652, -0.019539669259146054, 0.0049823721649163615}}},
+    {{1.872314453125, 1.01171875, 1.6484375, 1.0},
+     {{0.19708849068139514, -0.18492861394231702, 0.011819021642336381},
+      {-0.062493369050982246, 0.1999439223017031, -0.017001741456455655},
+      {-0.004967235280486029, -0.006673444758233741, 0.004180521551315315},
+      {0.003896693125884858, -0.00834186360115231, 0.0010021982628039565}}},
+    {{1.790283203125, 1.7490234375, 1.568359375, 1.353759765625},
+     {{0.24211096224870726, -0.16223286611923352, 0.032964828719821135, -0.001983228517689746},
+      {-0.1345696218644599, 0.2219254185983264, -0.057373046895087085, 0.0038137765996400785},
+      {0.03552370267295469, -0.06637888242299789, 0.027634091072212492, -0.002243680786495522},
+      {-0.0034223320248824344, 0.006686329943905031, -0.003225872896946547, 0.0004131327045451898}}}};
 __host__ __device__ inline int tab_pw(int Qxi) { return TAB_XI + Qxi; }
 __host__ __device__ inline int tab_cxi(int Qxi) { return TAB_XI + Qxi + Qxi * (NV_MAX + 1); }
 __host__ __device__ inline int tab_eps(int Qxi) { return tab_cxi(Qxi) + 3 * Qxi; }
