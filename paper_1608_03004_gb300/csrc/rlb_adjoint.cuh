@@ -447,7 +447,7 @@ struct AdjSmem {
   double P[NG][5][GW];          // psi_X dPhi_X/dF at the five stencil slots (memory order) of interface X
   double mom[3 * QP_MAX][GW];   // per radial node: the moment weights' share, even, xi and xi^2 parts
   double rate[2][GW];           // b dt r0, b dt r0 beta
-  double cst[13];               // constants of the rows (ADJ_CST)
+  double cst[rlbdev::ADJ_CST];  // constants of the rows (grad_constant)
   double b;                     // the forward stage's b (a register operand)
   int srcF[TXA + 8];            // source cell of each F position x0-4 .. x0+TXA+3
   int srcU[AWU + 1];            // source cell of each staged adjoint position, -1: outside the tube (zero)
@@ -456,41 +456,6 @@ struct AdjSmem {
 __device__ __forceinline__ int wrap_cell(int p, int Nx) {
   const int r = p % Nx;
   return r < 0 ? r + Nx : r;
-}
-
-// Gradient of the WENO5 interface value with respect to its five samples, from the differences d1..d4 in wind order
-// (their common sign does not matter): with Phi = v2 + G(d), dPhi/dv_m = g_m - g_{m+1} + [m = 2], g_l = dG/dd_l, g_0 =
-// g_5 = 0. Returns 1.5 g_l (1.5 = 6/4): 6 G = sum_k w_k r_k, w_k = (c_k / v_k^2) / sum, (c_k) = (1, 6, 3), and
-//   d(6G)/dv_k = 2 w_k (6G - r_k) / v_k,  v_k = x a + y b + e with a, b half the partials of the quadratic form,
-// so that g_l collects -2 w_0, 5 w_0 + w_1, 2 w_1 + 4 w_2, -w_2 and 4 z_k a_k, z_k = w_k (6G - r_k) / v_k, over 6. 66 FP64
-// operations; written on samples with every partial formed on its own it took about 130.
-// k: the constants, in registers (ADJ_CST from shared memory: FP64 operations with an immediate operand, additions and
-// multiplications issue every 19 cycles instead of 16; all-immediate, the row kernel took 11 % longer).
-enum { C_ONE, C_NZ, C_55, C_25, C_4, C_10, C_6, C_3, C_2, C_H, C_Q, C_125, C_15, ADJ_CST };
-__device__ __forceinline__ void weno5_grad(double d1, double d2, double d3, double d4, double e,
-                                           const volatile double* k, double (&g)[4]) {
-  const double one = k[C_ONE], nz = k[C_NZ], c55 = k[C_55], c25 = k[C_25], c4 = k[C_4], c10 = k[C_10];
-  const double t1 = fma(c55, d1, nz), t2 = fma(c55, d2, nz), t3 = fma(c55, d3, nz), t4 = fma(c55, d4, nz);
-  const double s2 = fma(c25, d2, nz), s3 = fma(c25, d3, nz);
-  const double ax0 = fma(c4, d1, -t2), ay0 = fma(c10, d2, -t1);  // 4x^2 - 11xy + 10y^2 of (d1, d2)
-  const double ax1 = fma(c4, d2, -s3), ay1 = fma(c4, d3, -s2);   // 4x^2 - 5xy + 4y^2 of (d2, d3)
-  const double ax2 = fma(c10, d3, -t4), ay2 = fma(c4, d4, -t3);  // 10x^2 - 11xy + 4y^2 of (d3, d4)
-  const double i0 = rlbdev::rcp_nr(fma(d1, ax0, fma(d2, ay0, e)), one);
-  const double i1 = rlbdev::rcp_nr(fma(d2, ax1, fma(d3, ay1, e)), one);
-  const double i2 = rlbdev::rcp_nr(fma(d3, ax2, fma(d4, ay2, e)), one);
-  const double q0 = fma(i0, i0, nz), q1 = fma(k[C_6], fma(i1, i1, nz), nz), q2 = fma(k[C_3], fma(i2, i2, nz), nz);
-  const double is = rlbdev::rcp_nr(fma(fma(q0, one, q1), one, q2), one);
-  const double w0 = fma(q0, is, nz), w1 = fma(q1, is, nz), w2 = fma(q2, is, nz);
-  const double c2 = k[C_2];
-  const double r0 = fma(c2, s2, -fma(c2, d1, nz)), r1 = fma(c2, d3, d2), r2 = fma(c4, d3, -d4);
-  const double G = fma(w0, r0, fma(w1, r1, fma(w2, r2, nz)));
-  const double z0 = fma(fma(w0, i0, nz), fma(-r0, one, G), nz), z1 = fma(fma(w1, i1, nz), fma(-r1, one, G), nz),
-               z2 = fma(fma(w2, i2, nz), fma(-r2, one, G), nz);
-  const double ch = k[C_H], cq = k[C_Q];
-  g[0] = fma(z0, ax0, -fma(ch, w0, nz));
-  g[1] = fma(z0, ay0, fma(z1, ax1, fma(cq, w1, fma(k[C_125], w0, nz))));
-  g[2] = fma(z1, ay1, fma(z2, ax2, fma(ch, w1, w2)));
-  g[3] = fma(z2, ay2, -fma(cq, w2, nz));
 }
 
 // What bounds it: the FP64 pipe (92 % busy on a batch that fills the GPU): 100 FP64 operations per node.
@@ -513,9 +478,8 @@ __device__ void adjoint_rows(const AdjArgs& A, const TubeDev& T, int x0, int par
     const int p = x0 - 3 + k;
     sm.srcU[k] = periodic ? wrap_cell(p, Nx) : ((p >= 0 && p < Nx) ? p : -1);
   }
-  if (tid < ADJ_CST) {
-    constexpr double v[ADJ_CST] = {1.0, -0.0, 5.5, 2.5, 4.0, 10.0, 6.0, 3.0, 2.0, 0.5, 0.25, 1.25, 1.5};
-    sm.cst[tid] = v[tid];
+  if (tid < rlbdev::ADJ_CST) {
+    sm.cst[tid] = rlbdev::grad_constant(tid);
     if (tid == 0) sm.b = A.b;
   }
   if (T.collide) {
@@ -551,7 +515,7 @@ __device__ void adjoint_rows(const AdjArgs& A, const TubeDev& T, int x0, int par
     double* dr = sm.drow[buf][g];
     double* ur = sm.urow[buf][g];
     const volatile double* cst = sm.cst;
-    const double one = cst[C_ONE], nz = cst[C_NZ];
+    const double one = cst[rlbdev::C_ONE], nz = cst[rlbdev::C_NZ];
     {
       // difference k lies between positions k and k + 1 of srcF; each lane loads position c + 1 and takes position c
       // from the lane below
@@ -578,10 +542,11 @@ __device__ void adjoint_rows(const AdjArgs& A, const TubeDev& T, int x0, int par
       const double psi = fma(fma(xi, cpsi, nz), fma(-ur[lo], one, ur[lo + 1]), nz);
       const double e = tab[tab_eps(Qxi) + s];
       double h[4];
-      weno5_grad(dr[fwd ? c : c + 3], dr[fwd ? c + 1 : c + 2], dr[fwd ? c + 2 : c + 1], dr[fwd ? c + 3 : c], e, cst, h);
+      rlbdev::weno5_grad(dr[fwd ? c : c + 3], dr[fwd ? c + 1 : c + 2], dr[fwd ? c + 2 : c + 1], dr[fwd ? c + 3 : c], e,
+                         cst, h);
       P0[(fwd ? 0 : 4) * GW + c] = fma(-psi, h[0], nz);
       P0[(fwd ? 1 : 3) * GW + c] = fma(psi, fma(-h[1], one, h[0]), nz);
-      P0[2 * GW + c] = fma(psi, fma(fma(-h[2], one, h[1]), one, cst[C_15]), nz);
+      P0[2 * GW + c] = fma(psi, fma(fma(-h[2], one, h[1]), one, cst[rlbdev::C_15]), nz);
       P0[(fwd ? 3 : 1) * GW + c] = fma(psi, fma(-h[3], one, h[2]), nz);
       P0[(fwd ? 4 : 0) * GW + c] = fma(psi, h[3], nz);
     } else {

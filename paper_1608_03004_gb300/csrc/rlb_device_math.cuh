@@ -528,4 +528,44 @@ __device__ __forceinline__ double weno5_interface_df(double m0, double m1, doubl
   return fma(df_join(lo_of(G.hi), lo_of(G.lo)), 1.0 / 6.0, m2);
 }
 
+// ---------------------------------------------------------------------------------------------------------
+// Gradient of the WENO5 interface value with respect to its five samples, from the differences d1..d4 in wind order
+// (their common sign does not matter): with Phi = v2 + G(d), dPhi/dv_m = g_m - g_{m+1} + [m = 2], g_l = dG/dd_l, g_0 =
+// g_5 = 0. Returns 1.5 g_l (1.5 = 6/4): 6 G = sum_k w_k r_k, w_k = (c_k / v_k^2) / sum, (c_k) = (1, 6, 3), and
+//   d(6G)/dv_k = 2 w_k (6G - r_k) / v_k,  v_k = x a + y b + e with a, b half the partials of the quadratic form,
+// so that g_l collects -2 w_0, 5 w_0 + w_1, 2 w_1 + 4 w_2, -w_2 and 4 z_k a_k, z_k = w_k (6G - r_k) / v_k, over 6. 66 FP64
+// operations; written on samples with every partial formed on its own it took about 130.
+// k: the constants, in registers (ADJ_CST from shared memory: FP64 operations with an immediate operand, additions and
+// multiplications issue every 19 cycles instead of 16; all-immediate, the row kernel took 11 % longer).
+enum { C_ONE, C_NZ, C_55, C_25, C_4, C_10, C_6, C_3, C_2, C_H, C_Q, C_125, C_15, ADJ_CST };
+__device__ __forceinline__ double grad_constant(int i) {
+  constexpr double v[ADJ_CST] = {1.0, -0.0, 5.5, 2.5, 4.0, 10.0, 6.0, 3.0, 2.0, 0.5, 0.25, 1.25, 1.5};
+  return v[i];
+}
+__device__ __forceinline__ void weno5_grad(double d1, double d2, double d3, double d4, double e,
+                                           const volatile double* k, double (&g)[4]) {
+  const double one = k[C_ONE], nz = k[C_NZ], c55 = k[C_55], c25 = k[C_25], c4 = k[C_4], c10 = k[C_10];
+  const double t1 = fma(c55, d1, nz), t2 = fma(c55, d2, nz), t3 = fma(c55, d3, nz), t4 = fma(c55, d4, nz);
+  const double s2 = fma(c25, d2, nz), s3 = fma(c25, d3, nz);
+  const double ax0 = fma(c4, d1, -t2), ay0 = fma(c10, d2, -t1);  // 4x^2 - 11xy + 10y^2 of (d1, d2)
+  const double ax1 = fma(c4, d2, -s3), ay1 = fma(c4, d3, -s2);   // 4x^2 - 5xy + 4y^2 of (d2, d3)
+  const double ax2 = fma(c10, d3, -t4), ay2 = fma(c4, d4, -t3);  // 10x^2 - 11xy + 4y^2 of (d3, d4)
+  const double i0 = rcp_nr(fma(d1, ax0, fma(d2, ay0, e)), one);
+  const double i1 = rcp_nr(fma(d2, ax1, fma(d3, ay1, e)), one);
+  const double i2 = rcp_nr(fma(d3, ax2, fma(d4, ay2, e)), one);
+  const double q0 = fma(i0, i0, nz), q1 = fma(k[C_6], fma(i1, i1, nz), nz), q2 = fma(k[C_3], fma(i2, i2, nz), nz);
+  const double is = rcp_nr(fma(fma(q0, one, q1), one, q2), one);
+  const double w0 = fma(q0, is, nz), w1 = fma(q1, is, nz), w2 = fma(q2, is, nz);
+  const double c2 = k[C_2];
+  const double r0 = fma(c2, s2, -fma(c2, d1, nz)), r1 = fma(c2, d3, d2), r2 = fma(c4, d3, -d4);
+  const double G = fma(w0, r0, fma(w1, r1, fma(w2, r2, nz)));
+  const double z0 = fma(fma(w0, i0, nz), fma(-r0, one, G), nz), z1 = fma(fma(w1, i1, nz), fma(-r1, one, G), nz),
+               z2 = fma(fma(w2, i2, nz), fma(-r2, one, G), nz);
+  const double ch = k[C_H], cq = k[C_Q];
+  g[0] = fma(z0, ax0, -fma(ch, w0, nz));
+  g[1] = fma(z0, ay0, fma(z1, ax1, fma(cq, w1, fma(k[C_125], w0, nz))));
+  g[2] = fma(z1, ay1, fma(z2, ax2, fma(ch, w1, w2)));
+  g[3] = fma(z2, ay2, -fma(cq, w2, nz));
+}
+
 }  // namespace rlbdev
