@@ -32,8 +32,9 @@
  *    and in xi, so Eq. (mom_feq) recovers it exactly only with Np >= 2, Nv >= 2 and a polar rule exact to
  *    degree Nv + 2 (section "Riemann problem" gives Qp = 3 for the same reason). Qxi <= 1024, Nx >= 1
  *    (periodic: Nx >= 3), dx > 0, dt > 0.
- *  - Speed limit: the Legendre coefficients of the equilibrium, Eq. (feqtrunc), are summed as a positive
- *    power series in v of at most 16384 terms, which converges for |v| <= 0.9955. A cell faster than that is
+ *  - Speed limit: |v| <= 0.9955 (0.9950 for Np = 3 or Nv != 5; for the reverse sweep 0.9949 and 0.9944), the
+ *    speeds up to which a power series in v of 16384 terms gives the Legendre coefficients of the equilibrium,
+ *    Eq. (feqtrunc). The library takes them from recurrences and keeps this range. A cell faster than that is
  *    treated as non-physical: rlb_init returns RLB_EINVAL, a step sets the sticky non-physical flag.
  */
 #ifndef RLB_H
@@ -282,11 +283,12 @@ rlb_status rlb_autotune(rlb_handle h, int32_t trial_steps, rlb_launch *best, dou
  *   stream: cudaStream_t to launch on. The call returns once its small host-side tables have been copied
  *          out (CUDA may first wait for earlier work on that stream, as for any copy from pageable memory);
  *          the steps themselves run asynchronously.
- *   Size limit: 2 Q Nx doubles of stage scratch plus the tables (about 8 (Qxi + 16) (NV_MAX + 2) bytes) and
- *   8 bytes per 61 cells must fit in RLB_STATIC_SCRATCH_BYTES (the array is 2 KB longer), e.g. Q = 24 up to Nx of about 170000, Q = 600
- *   up to about 6800; larger tubes return RLB_EINVAL before anything is launched.
+ *   Size limit: 2 Q Nx doubles of stage scratch plus 28 + 13 Qxi + 4 Q doubles for the tables and 8 bytes per 61
+ *   cells must fit in RLB_STATIC_SCRATCH_BYTES, e.g. Q = 24 up to Nx of about 170000, Q = 600 up to about 6800;
+ *   larger tubes return RLB_EINVAL before anything is launched. (A tube is counted so whatever its tables and
+ *   tile list take; the array is 2 KB longer.)
  *   Set-up: the first call on a device (with that device current) looks up the array's device address and
- *   uploads the series tables that the kernels share with rlb_init; these steps synchronise, so make the first
+ *   uploads the factors that the kernels share with rlb_init; these steps synchronise, so make the first
  *   call on each device before any stream capture. Later calls only enqueue copies into the array and the
  *   kernel launches.
  *   Every call uses the same array and leaves its contents behind: calls that overlap on the GPU (on two

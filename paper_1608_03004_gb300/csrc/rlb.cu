@@ -319,7 +319,7 @@ bool g_tables_ready[64] = {};
 
 // Once per device: fill the recurrence factors of the Legendre coefficients and let the kernels use more than
 // 48 KB of dynamic shared memory.
-rlb_status ensure_series_tables(int dev) {
+rlb_status ensure_tables(int dev) {
   std::lock_guard<std::mutex> lk(g_tables_mu);
   if (dev < 0 || dev >= 64) return RLB_EINVAL;
   if (g_tables_ready[dev]) return RLB_OK;
@@ -700,7 +700,7 @@ rlb_status create(rlb_handle* out, const rlb_tube* tubes, int32_t ntubes, const 
     RLB_CUDA(cudaMemcpyAsync(h->d_halo, h->halo.data(), sizeof(HaloDesc) * h->halo.size(), cudaMemcpyHostToDevice,
                              h->stream));
   }
-  rlb_status st = ensure_series_tables(h->dev);
+  rlb_status st = ensure_tables(h->dev);
   if (st != RLB_OK) return st;
   // resident CTAs per SM of this handle's stage kernel (the persistent grids' default size)
   if (h->storage == RLB_STORAGE_F64) {
@@ -1341,8 +1341,11 @@ rlb_status rlb_quadrature(int32_t Qp, int32_t Qxi, double* pbar, double* wp, dou
 // file-scope array instead; the existing stage kernel runs on it unchanged.
 namespace {
 
-// STATIC_SLACK: the size limit is counted with the tile list and tables that tiles of 61 cells need (static_need), so
-// that the tubes it admits do not depend on the tile width; the list of the present tiles is at most 1 KB longer.
+// The tubes that the size limit admits depend neither on the kernel's tile width nor on the layout of its tables: a tube
+// is counted (static_need) with 8 bytes per STATIC_TILE cells and with STATIC_TAB + STATIC_TAB_XI Qxi + STATIC_TAB_Q Q
+// doubles of tables. The present tiles and tables need at most STATIC_SLACK more: 8 (Nx/60 - Nx/61) bytes, 1020 at the
+// longest tube, and 40 + Qxi - 2 Q doubles, 200 bytes at the smallest Q = 9, each rounded up to 256.
+constexpr size_t STATIC_TILE = 61, STATIC_TAB = 28, STATIC_TAB_XI = 13, STATIC_TAB_Q = 4;
 constexpr size_t STATIC_SLACK = 2048;
 static __device__ __align__(256) double g_static_scratch[(RLB_STATIC_SCRATCH_BYTES + STATIC_SLACK) / sizeof(double)];
 
@@ -1350,7 +1353,7 @@ std::mutex g_static_mu;
 double* g_static_addr[64] = {};
 
 // Once per device, with that device current: the device address of the array (in host code the symbol is
-// only a host-side stand-in and must not be passed to a kernel) and the shared series tables.
+// only a host-side stand-in and must not be passed to a kernel) and the kernels' shared factors.
 rlb_status static_setup(int dev, double** base) {
   if (dev < 0 || dev >= 64) return RLB_EINVAL;
   {
@@ -1363,15 +1366,16 @@ rlb_status static_setup(int dev, double** base) {
     }
     *base = g_static_addr[dev];
   }
-  return ensure_series_tables(dev);
+  return ensure_tables(dev);
 }
 
 size_t align256(size_t bytes) { return (bytes + 255) / 256 * 256; }
 
 // Bytes of the array that a tube is counted with.
 size_t static_need(size_t Qxi, size_t Q, size_t Nx) {
-  return align256(sizeof(TubeDev)) + align256(sizeof(int2) * ((Nx + 60) / 61)) + 256 +
-         align256(sizeof(double) * (28 + 13 * Qxi + 4 * Q)) + 2 * align256(sizeof(double) * Q * Nx);
+  return align256(sizeof(TubeDev)) + align256(sizeof(int2) * ((Nx + STATIC_TILE - 1) / STATIC_TILE)) + 256 +
+         align256(sizeof(double) * (STATIC_TAB + STATIC_TAB_XI * Qxi + STATIC_TAB_Q * Q)) +
+         2 * align256(sizeof(double) * Q * Nx);
 }
 
 }  // namespace

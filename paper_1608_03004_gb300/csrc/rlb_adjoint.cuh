@@ -1,5 +1,5 @@
 // Adjoint (reverse mode) of the FP64 stage kernel, and of the initial equilibrium. Included by rlb.cu inside
-// its anonymous namespace, after the forward kernels (it uses their helpers and series tables).
+// its anonymous namespace, after the forward kernels (it uses their helpers).
 //
 // One forward stage maps F_in to F_out = a F^n + b (F_in + dt L(F_in)) with
 //   L_s(x) = -(xi_j/dx) (Phi_s(x+1/2) - Phi_s(x-1/2)) + r_s(x) (F^eq_s(x) - F_s(x)),  r_s = gamma (1 - beta xi_j)/tau

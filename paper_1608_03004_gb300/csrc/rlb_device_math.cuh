@@ -57,10 +57,11 @@ constexpr double WENO_EPS = 1e-6;
 
 // Products and sums that are rounded exactly as written. The compiler may contract a product into a following
 // addition (an FMA), and may do so differently in different inlined copies of the same expression. The
-// reduced-precision kernel evaluates each interface value and each indicator pair at a lane's edges twice (once
-// in each lane that uses it), and its compensated sums are error-free only if every addition is rounded as
-// written, so its FP32 arithmetic goes through these (mul.rn / add.rn / sub.rn are never contracted). The FP64
-// path evaluates every interface once and keeps the compiler's choices.
+// reduced-precision kernel forms the indicator squares at a lane's edges twice (once in each lane that uses them), and
+// its compensated sums are error-free only if every addition is rounded as written, so its FP32 arithmetic goes through
+// these (mul.rn / add.rn / sub.rn are never contracted). The double forms of these and of the functions up to
+// weno5_interface serve the unit test of the formulas only: the FP64 kernels take the packed limiter (weno5_pair_df2,
+// weno5_combine6_df2) and its gradient (weno5_grad) below.
 __device__ __forceinline__ float mul_x(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_x(double a, double b) { return a * b; }
 __device__ __forceinline__ float add_x(float a, float b) { return __fadd_rn(a, b); }
@@ -77,8 +78,8 @@ __device__ __forceinline__ double sub_x(double a, double b) { return a - b; }
 //   alpha_k = d_k / (eps + beta_k)^2 with d = (1, 6, 3)/10 equals 9 / s_k, s_k = u_k^2,
 //   u_k = (3 eps + 3 beta_k) / sqrt(d_k); the normalised weights are w_k = prod_{l!=k} s_l / sum_m prod_{l!=m} s_l.
 // Each indicator depends on one pair of adjacent differences, and each pair serves three interfaces, so
-// the kernel evaluates the three scaled squares once per pair (weno5_pair) and combines three pairs per
-// interface (weno5_combine). For a wind toward decreasing index the stencil is mirrored: the differences
+// a kernel evaluates the three scaled squares once per pair (weno5_pair) and combines three pairs per
+// interface (weno5_combine6). For a wind toward decreasing index the stencil is mirrored: the differences
 // change sign and order, which swaps the roles of SL and SR.
 constexpr double C0 = 3.1622776601683795;  // sqrt(10)
 constexpr double C1 = 1.2909944487358056;  // sqrt(10/6)
@@ -88,8 +89,8 @@ constexpr float EPS_A = (float)(3.0 * WENO_EPS * C0);
 constexpr float EPS_B = (float)(3.0 * WENO_EPS * C1);
 constexpr float EPS_C = (float)(3.0 * WENO_EPS * C2);
 
-// Reciprocal used by the WENO combination: FP64 as above; FP32 the hardware approximation alone (about 1 ulp
-// of FP32, below the rounding of the FP32 state it serves).
+// Reciprocal of weno5_combine6: in FP32 the hardware approximation alone (about 1 ulp of FP32, below the rounding of
+// the FP32 state it serves).
 __device__ __forceinline__ double rcp_fast(double d) { return rcp_nr(d); }
 __device__ __forceinline__ float rcp_fast(float d) {
   float r;
@@ -100,7 +101,7 @@ __device__ __forceinline__ float rcp_fast(float d) {
 // Scaled indicator squares of the pair (x, y) = (d_j, d_{j+1}) in memory order. fwd: wind toward increasing
 // index; then sA = (C0 (SL + 3eps))^2, sB = (C1 (SC + 3eps))^2, sC = (C2 (SR + 3eps))^2; otherwise SL and SR
 // trade places. (eA, eB, eC) = 3 eps (C0, C1, C2): the velocity's epsilon term, which scales with the square
-// of its quadrature weight. T is double (FP64 path) or float (reduced-precision path).
+// of its quadrature weight.
 template <typename T>
 __device__ __forceinline__ void weno5_pair(T x, T y, bool fwd, T eA, T eB, T eC, T& sA, T& sB, T& sC) {
   const T qx = mul_x(x, x), pxy = mul_x(x, y), qy = mul_x(y, y);
@@ -115,7 +116,7 @@ __device__ __forceinline__ void weno5_pair(T x, T y, bool fwd, T eA, T eB, T eC,
 }
 
 // 6 G of the interface from the three scaled squares (s0, s1, s2) of its stencils and the differences
-// d1..d4 in wind order (the FP64 stage kernel applies the 1/6 in the flux difference, where it costs nothing).
+// d1..d4 in wind order (the kernels apply the 1/6 in the flux difference, where it costs nothing).
 template <typename T>
 __device__ __forceinline__ T weno5_combine6(T s0, T s1, T s2, T d1, T d2, T d3, T d4) {
   const T r0 = fma(T(5.0), d2, mul_x(T(-2.0), d1)), r1 = fma(T(2.0), d3, d2), r2 = fma(T(4.0), d3, -d4);
@@ -132,8 +133,8 @@ __device__ __forceinline__ T weno5_combine(T s0, T s1, T s2, T d1, T d2, T d3, T
 }
 
 // Interface value v2 + G of five samples in memory order m0..m4 around the interface between m2 and m3
-// (wind toward increasing index, fwd) or between m1 and m2 (wind toward decreasing index), computed
-// exactly as the stage kernels do: pairs first, then the combination. eps: the limiter's epsilon.
+// (wind toward increasing index, fwd) or between m1 and m2 (wind toward decreasing index): pairs first, then the
+// combination, as the reduced-precision kernel forms it. eps: the limiter's epsilon.
 template <typename T>
 __device__ __forceinline__ T weno5_interface(T m0, T m1, T m2, T m3, T m4, bool fwd, double eps = WENO_EPS) {
   const T D1 = m1 - m0, D2 = m2 - m1, D3 = m3 - m2, D4 = m4 - m3;
@@ -175,17 +176,6 @@ __device__ __forceinline__ float round_f32(double d) {
   const unsigned m = (((hi & 0x7FFFFFFFu) - (896u << 20)) << 3) | (lo >> 29), rest = lo << 3;
   const unsigned up = rest > 0x80000000u || (rest == 0x80000000u && (m & 1u)) ? 1u : 0u;
   return __uint_as_float((hi & 0x80000000u) | (m + up));  // a carry into the exponent is the right value, up to infinity
-}
-
-// acc += f (whi + wlo)
-__device__ __forceinline__ void df_add_prod(DF& acc, float f, float whi, float wlo) {
-  const float p = __fmul_rn(f, whi);
-  float e = fmaf(f, whi, -p);
-  e = fmaf(f, wlo, e);
-  float s, t;
-  two_sum(acc.hi, p, s, t);
-  acc.hi = s;
-  acc.lo = __fadd_rn(acc.lo, __fadd_rn(t, e));
 }
 
 // acc += a (xhi + xlo)
@@ -353,7 +343,7 @@ __device__ __forceinline__ DF df_split(double d) {
   return {h, l};
 }
 
-// The double equal to the float f (0 for zero and subnormal f), by integer operations on f's bits.
+// The double equal to the float f (0 for zero and subnormal f), by integer operations on f's bits (unit test of df_split).
 __device__ __forceinline__ double df_widen(float f) {
   const unsigned b = __float_as_uint(f), ef = (b >> 23) & 0xFFu;
   const unsigned hi = (b & 0x80000000u) | ((ef + 896u) << 20) | ((b >> 3) & 0xFFFFFu);

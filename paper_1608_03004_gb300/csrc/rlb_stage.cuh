@@ -1,7 +1,6 @@
 // FP64 stage kernel of the time step and the device helpers that the other kernels share (Landau frame,
-// Legendre series of the equilibrium, per-tile coefficients, tile schedules, group barriers). Included by
-// rlb.cu inside its anonymous namespace; the file covers the kernel code that the FP64 profile summary was
-// captured on, host code lives in rlb.cu.
+// Legendre coefficients of the equilibrium, per-tile coefficients, tile schedules, group barriers). Included by
+// rlb.cu inside its anonymous namespace; host code lives in rlb.cu.
 #pragma once
 
 constexpr int NT = 256;                    // threads per CTA
@@ -31,7 +30,8 @@ struct StageArgs {
   int schedule;       // 0: one CTA per tile; 1: persistent, grid stride; 2: persistent, work counter
   int* counter;       // work counter of schedule 2 (zeroed before the launch)
   int split;          // work items per tile (<= 1: one): item k of a tile advances velocity rows
-                      // [k Q / split, (k + 1) Q / split) after reducing the moments over all rows
+                      // [k Q / split, (k + 1) Q / split); under schedules 1 and 2 each item reduces the
+                      // moments over all rows, else the items are a cluster that shares them
 };
 
 // Tile loop of a stage launch. Schedule 0 gives each CTA one tile; the persistent schedules keep a grid of
@@ -86,25 +86,21 @@ __device__ __forceinline__ bool stiff(const TubeDev& T, double beta) {
   return k * k > T.stiff_lim * T.stiff_lim * (1.0 - beta * beta);      // (k gamma)^2 > stiff_lim^2, no square root
 }
 
-// Landau frame from (N0, Nx, T00, T0x, Txx): e, beta, n (Landau), T, and gamma = (1 - beta^2)^-1/2 if gam_out is
-// given. Returns false if non-physical. A cell at rest (T0x = 0, exactly so wherever the state is symmetric in xi)
-// skips the division and square root that give beta = 0, gamma = 1 and n = N0.
-__device__ __forceinline__ bool landau(const double mom[5], double& e, double& beta, double& n, double& T,
-                                       double* gam_out = nullptr) {
+// Landau frame from (N0, Nx, T00, T0x, Txx): e, beta, n (Landau), T. Returns false if non-physical. A cell at rest
+// (T0x = 0, exactly so wherever the state is symmetric in xi) skips the division and square root that give beta = 0 and
+// n = N0.
+__device__ __forceinline__ bool landau(const double mom[5], double& e, double& beta, double& n, double& T) {
   const double A = mom[2] + mom[4];
   const double disc = A * A - 4.0 * mom[3] * mom[3];
   e = 0.5 * ((mom[2] - mom[4]) + sqrt(disc));
-  double gam = 1.0;
   if (mom[3] == 0.0) {
     beta = 0.0;
     n = mom[0];
   } else {
     beta = mom[3] / (mom[4] + e);
-    gam = 1.0 / sqrt(1.0 - beta * beta);
-    n = gam * (mom[0] - beta * mom[1]);
+    n = 1.0 / sqrt(1.0 - beta * beta) * (mom[0] - beta * mom[1]);
   }
   T = e / (3.0 * n);
-  if (gam_out) *gam_out = gam;
   return disc >= 0.0 && e > 0.0 && fabs(beta) < 1.0 && n > 0.0 && T > 0.0;
 }
 
@@ -131,9 +127,10 @@ __host__ __device__ constexpr double beta_limit_d(int NPc) { return NPc <= 2 ? 0
 // gives K. In m:
 //   m (1 - beta^2) a_{m+1,k} = (k + m - 1) beta a_{m,k-1} - (k - m + 1) a_{m,k},
 // and for k = 0 the form without a_{m,-1}, m (1 - beta^2) a_{m+1,0} = m a_{m,0} + (m - 2) beta a_{m,1}.
-// Against extended precision every coefficient is within a few units of FP64 rounding up to |beta| = 0.97 (as the
-// positive power series in beta is, which takes 12 operations for each of its 40 terms at beta = 0.4 and 574 at 0.9;
-// here about 2 operations for each of 18 and 46 steps). FP64 operations bound every kernel that calls this. With the
+// Largest error of a coefficient against extended precision, in units of 2^-52: Np = 2, Nv = 5: 4 up to |beta| = 0.7, 9 at
+// 0.97, 12 at 0.9949; Np = 3, Nv = 8: 7 up to 0.45, 12 at 0.7, 24 at 0.97, 34 at 0.9949. The positive power series in beta
+// has 8 at 0.7, 30 at 0.97 and 145 at 0.9949 for either, and takes 12 operations for each of its 40 terms at beta = 0.4
+// and 574 at 0.9; here about 2 operations for each of 18 and 46 steps. FP64 operations bound every kernel that calls this. With the
 // series, the FP32 steps of 128 uneven moving tubes kept the FP64 pipe 85 % busy; on GB300 they went from 4.42 to 2.43
 // ms, the FP32 stress tube's (half its gas in motion) from 6.5 to 5.2 ms, the 400-cell FP64 tube's from 89 to 54 us.
 template <int KV>

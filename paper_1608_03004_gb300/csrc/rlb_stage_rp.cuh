@@ -15,7 +15,7 @@
 //    storing it and left 5 FP64 moments per cell (M_in); this stage does the same for F_out (M_out);
 //  - the next row's loads are in flight while a row is evaluated, and F^n is loaded at the start of a row's
 //    evaluation (it is needed only at its end);
-//  - FP64 work is per cell only (Landau frame, Legendre series, equilibrium coefficients), kept by each lane
+//  - FP64 work is per cell only (Landau frame, Legendre and equilibrium coefficients), kept by each lane
 //    for its own cells in shared memory, where the lane also keeps its cells' five moment sums between
 //    radial nodes (lane-private columns: no barrier).
 // Rows are walked radial node by radial node, each node's directions in mirror pairs (xi, -xi), so that a pair
