@@ -56,11 +56,14 @@ METRIC = "G velocity-node updates/s"
 UNIT = "G updates/s"
 # Algorithmic flops per velocity-node per RK stage (FMA = 2): WENO5 interface value 54 (the first difference 1,
 # the limiter 53), flux difference and xi/dx 2, equilibrium (Nv+1 = 6 FMAs) 12, collision 5, Runge-Kutta
-# combination 5, moment reduction 6. Per-cell work (Landau solve, Legendre series) is not counted, so these are
-# lower bounds. The FP64 stage kernel runs the limiter's 53 in double-float on the FP32 pipe; the other 31 run
-# on the FP64 pipe, which bounds the kernel.
+# combination 5, moment reduction 6. Per-cell work (Landau solve, Legendre coefficients) is not counted, so these are
+# lower bounds. The FP64 stage kernel runs the limiter's 53 in double-float on the FP32 pipe.
 FLOPS_PER_NODE_STAGE = 84
-FP64_FLOPS_PER_NODE_STAGE = 31
+# What the FP64 stage kernel puts on the FP64 pipe per velocity node and stage, per-cell work again not counted: 12.9
+# operations, all FMAs (default orders, average of the three stages; both rows of a mirror pair share the equilibrium's
+# two Horner chains and the moments' sums): first differences 64/60, moments 2.5, equilibrium 4, collision 2, flux
+# difference and xi/dx 2, Runge-Kutta combination 2 in two of three stages.
+FP64_FLOPS_PER_NODE_STAGE = 2 * (64 / 60 + 2.5 + 4 + 2 + 2 + 2 * 2 / 3)
 # Algorithmic HBM bytes per velocity node per step with one launch per stage: stage inputs read once
 # (1 + 2 + 2 doubles), outputs written once (3 doubles).
 BYTES_PER_NODE_STEP = 64
@@ -574,11 +577,11 @@ def measure(args, specs, desc, precision, autotune, steps, warmup, rank, world, 
                     "method_flops_tflops": method_rate,
                     "method_flops_vs_fp64_peak": method_rate / fp64_peak,
                     "note": "FP64 pipe; peak = SMs x 2 DFMA/clk x 2 flops x max SM clock (derived); achieved = the "
-                            f"{FP64_FLOPS_PER_NODE_STAGE} algorithmic flops per velocity node and stage that run "
-                            f"in FP64. The WENO5 limiter's other {FLOPS_PER_NODE_STAGE - FP64_FLOPS_PER_NODE_STAGE} "
-                            "run in double-float on the FP32 pipe; method_flops_* count all "
-                            f"{FLOPS_PER_NODE_STAGE} against the FP64 peak (above 1: faster than an all-FP64 "
-                            "kernel can be)"}
+                            f"{FP64_FLOPS_PER_NODE_STAGE / 2:.1f} FMAs per velocity node and stage that the kernel "
+                            "runs in FP64 (per-cell work not counted). The WENO5 limiter runs in double-float on the "
+                            "FP32 pipe, and mirror pairs of directions share the moments' sums and the equilibrium; "
+                            f"method_flops_* count the method's {FLOPS_PER_NODE_STAGE} flops per node against the "
+                            "FP64 peak (above 1: faster than an all-FP64 kernel can be)"}
     else:
         roofline = {"bound": "hbm", "achieved": hbm_achieved, "peak": hbm_peak, "unit": "GB/s",
                     "frac": hbm_achieved / hbm_peak, "traffic": traffic, "kernel": "rlb_stage_rp_kernel",
