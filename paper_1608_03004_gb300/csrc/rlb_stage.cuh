@@ -127,7 +127,7 @@ __host__ __device__ constexpr double beta_limit_d(int NPc) { return NPc <= 2 ? 0
 // gives K. In m:
 //   m (1 - beta^2) a_{m+1,k} = (k + m - 1) beta a_{m,k-1} - (k - m + 1) a_{m,k},
 // and for k = 0 the form without a_{m,-1}, m (1 - beta^2) a_{m+1,0} = m a_{m,0} + (m - 2) beta a_{m,1}.
-// Largest error of a coefficient against extended precision, in units of 2^-52: Np = 2, Nv = 5: 4 up to |beta| = 0.7, 9 at
+// Largest error of a coefficient against extended precision, in units of 2^-52: Np = 2, Nv = 5: 5 up to |beta| = 0.7, 9 at
 // 0.97, 12 at 0.9949; Np = 3, Nv = 8: 7 up to 0.45, 12 at 0.7, 24 at 0.97, 34 at 0.9949. The positive power series in beta
 // has 8 at 0.7, 30 at 0.97 and 145 at 0.9949 for either, and takes 12 operations for each of its 40 terms at beta = 0.4
 // and 574 at 0.9; here about 2 operations for each of 18 and 46 steps. FP64 operations bound every kernel that calls this. With the
@@ -679,7 +679,7 @@ __device__ void stage_tile(const StageArgs& A, const TubeDev& T, int x0, int par
   }
 }
 
-// What bounds it: the FP64 pipe (88 % busy on the stress tube, 14.3 FP64 operations per node, 35 % of the issue
+// What bounds it: the FP64 pipe (89 % busy on the stress tube, 14.2 FP64 operations per node, 35 % of the issue
 // slots). Measured on GB300, FP64 stress tube (2^20 cells x 384 velocities, half of it moving), ms per step: 46.0 with
 // one row at a time in scalar double-float and Legendre-basis equilibria, 37.1 with both rows of a mirror pair packed,
 // register operands and Horner equilibria, 34.8 once no conversion instruction was left in the rows (df_split,
